@@ -196,9 +196,9 @@ __global__ void __launch_bounds__(kAosThreads) gpz_aos_range_kernel(const float*
 // kernel's body with the block's records as its tile (one bulk copy of
 // 1024 F contiguous values), so no structure-of-arrays copy is made.
 template <int F, bool PRE>
-__global__ void __launch_bounds__(kThreads, 6) gpz_qse_tile_aos_kernel(QseArgs a) {
+__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_aos_kernel(const __grid_constant__ QseArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
-    __shared__ __align__(8) TileShared S;
+    __shared__ TileShared S;
     if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
         qse_block_tile<F, true, PRE, GridBlock, true>(a, dsm, S, GridBlock{});
     else
@@ -207,12 +207,12 @@ __global__ void __launch_bounds__(kThreads, 6) gpz_qse_tile_aos_kernel(QseArgs a
 
 template <int F, bool PRE>
 cudaError_t launch_qse_tile_aos_fp(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = tile_smem_bytes(F);
+    const size_t smem = tile_smem_bytes(F, a.perm != nullptr);
     auto kern = gpz_qse_tile_aos_kernel<F, PRE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    kern<<<a.nblocks, kThreads, smem, s>>>(a);
+    kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_qse_general(a, s);

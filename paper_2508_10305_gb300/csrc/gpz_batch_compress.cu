@@ -188,9 +188,9 @@ __global__ void __launch_bounds__(kThreads, 5) gpz_batch_compress_kernel(BatchCo
 // The same with the shared-memory tile body (gpz_qse_tile.cuh): groups whose
 // chunks all have 16-byte aligned fields.
 template <int F, bool PRE>
-__global__ void __launch_bounds__(kThreads, 6) gpz_batch_tile_kernel(BatchCompressArgs g) {
+__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_batch_tile_kernel(BatchCompressArgs g) {
     extern __shared__ __align__(128) uint8_t dsm[];
-    __shared__ __align__(8) TileShared S;
+    __shared__ TileShared S;
     __shared__ QseArgs A;
     __shared__ uint32_t slot[2];  // block within its chunk, global block id
     const uint32_t gb = g.block_first + blockIdx.x;
@@ -397,11 +397,11 @@ bool prepare_f() {
            cudaFuncSetAttribute(gpz_batch_compress_kernel<F, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 100) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem_bytes(F)) == cudaSuccess &&
+                                (int)tile_smem_bytes(F, true)) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 100) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem_bytes(F)) == cudaSuccess &&
+                                (int)tile_smem_bytes(F, true)) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 100) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -427,9 +427,9 @@ void launch_f(const BatchCompressArgs& a, int grid, cudaStream_t s, bool general
     if (general)
         gpz_batch_general_kernel<F><<<grid, kThreads, qse_smem_bytes(F), s>>>(a);
     else if (a.tile && a.pre)
-        gpz_batch_tile_kernel<F, true><<<grid, kThreads, tile_smem_bytes(F), s>>>(a);
+        gpz_batch_tile_kernel<F, true><<<grid, kTileThreads, tile_smem_bytes(F, a.any_perm != 0), s>>>(a);
     else if (a.tile)
-        gpz_batch_tile_kernel<F, false><<<grid, kThreads, tile_smem_bytes(F), s>>>(a);
+        gpz_batch_tile_kernel<F, false><<<grid, kTileThreads, tile_smem_bytes(F, a.any_perm != 0), s>>>(a);
     else if (a.pre)
         gpz_batch_compress_kernel<F, true><<<grid, kThreads, qse_fast_smem_bytes(), s>>>(a);
     else

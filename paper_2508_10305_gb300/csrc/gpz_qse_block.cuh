@@ -105,14 +105,14 @@ struct BitAppender {
     }
 };
 
-template <int F>
+template <int F, int TH = kThreads>
 __device__ __forceinline__ void write_raw(const QseArgs& a, uint32_t b, int n_b, int t) {
     const uint64_t first = (uint64_t)b * kBlock;
     uint32_t* out = a.temp + (size_t)b * a.slot_words;
     if (t == 0) out[0] = 1u;
     if (a.interleaved) {  // value k of the block's records is field k % F of particle k / F
         const float* src = a.fields[0] + first * F;
-        for (int k = t; k < F * n_b; k += kThreads) {
+        for (int k = t; k < F * n_b; k += TH) {
             const int i = k / F, f = k - i * F;
             out[1 + f * n_b + i] = __float_as_uint(__ldg(src + k));
         }
@@ -120,11 +120,11 @@ __device__ __forceinline__ void write_raw(const QseArgs& a, uint32_t b, int n_b,
 #pragma unroll
         for (int f = 0; f < F; ++f) {
             const float* src = a.fields[f] + first;
-            for (int i = t; i < n_b; i += kThreads) out[1 + f * n_b + i] = __float_as_uint(__ldg(src + i));
+            for (int i = t; i < n_b; i += TH) out[1 + f * n_b + i] = __float_as_uint(__ldg(src + i));
         }
     }
     if (a.perm)
-        for (int i = t; i < n_b; i += kThreads) a.perm[first + i] = (uint32_t)(first + i);
+        for (int i = t; i < n_b; i += TH) a.perm[first + i] = (uint32_t)(first + i);
     if (t == 0) a.sizes[b] = 1u + (uint32_t)F * (uint32_t)n_b;
 }
 

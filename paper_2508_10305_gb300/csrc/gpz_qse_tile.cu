@@ -2,26 +2,32 @@
 // encoding; Sections 4.1-4.3) of single-array calls whose fields are 16-byte
 // aligned, with the block's input in shared memory instead of registers.
 //
-// One CTA of 256 threads owns one block of 1024 particles, as in
-// gpz_qse_block.cuh's fast path, and produces the same words; what differs
-// is where the data lives:
-//   - thread 0 loads the block's F x 1024 values into a shared tile with one
-//     bulk copy per field, completing on an mbarrier (the few values of a
-//     ragged last block beyond a multiple of four are loaded by plain loads);
-//   - threads 0..F-1 derive their field's constants (minimum, code width,
-//     segment split, record offset) once, into shared memory: with a
+// One CTA of 128 threads owns one block of 1024 particles, eight per thread:
+//   - lane f of warp 0 loads field f's 1024 values into a shared tile with one
+//     bulk copy, completing on an mbarrier (the few values of a ragged last
+//     block beyond a multiple of four are loaded by plain loads);
+//   - lanes 0..F-1 of warp 0 derive their field's constants (minimum, code
+//     width, segment split, place in the key) once, into shared memory: with a
 //     relative bound from the block extremes of the range pass, loaded with
 //     the field's step constants in one round trip while the tile is in
-//     flight; otherwise from the tile;
-//   - each thread quantises its 4 particles of every field from the tile;
+//     flight; otherwise from the tile, a warp per field;
+//   - each thread quantises its 8 particles of every field from the tile;
 //   - once every value is quantised the tile is dead, and the encoded
 //     block's staging words are assembled in the same bytes, then written to
 //     the block's temporary slot by one bulk copy.
-// Holding no input in registers, a thread needs about 40 registers instead
-// of 48, and with the staging words overlaying the tile a CTA needs about 36
-// KB of shared memory for F = 6: six CTAs per SM instead of five.  The
-// kernel is latency-bound (instruction issue waits on shared memory, warp
-// collectives and barriers), so residency is what pays.
+// What bounds it: instruction issue (three fields: 75% of the issue slots
+// busy) and, where a warp's keys are mostly distinct, the unit that executes
+// match (62% busy on the snapshot).  Why 128 threads: whatever a block costs
+// per warp rather than per particle (the constants' loads, the scan over
+// (bin, warp), the barriers) halves against 256 threads of four particles,
+// and eight independent particles per thread hide more latency than the
+// second half of the warps did.  Per block 4,740 warp instructions instead of
+// 7,200 (six fields), 1,330 shared-memory wavefronts instead of 1,980.
+// Measured on a 2^26 x 6 snapshot (relative bound): 0.577 -> 0.472 ms; on
+// 10^8 x 3 scan points (absolute bound): 0.750 -> 0.533 ms.
+// Residency: shared memory allows seven CTAs per SM for six fields (28 KB
+// each); for three fields nine (56 registers) measured best, 7 / 8 / 9 / 10 /
+// 12 CTAs: 0.565 / 0.544 / 0.533 / 0.540 / 0.550 ms on the scan.
 //
 // With a relative bound the block's extremes come from the range pass and
 // must bound the block's values (they are exact there): codes are monotone in
@@ -37,9 +43,9 @@
 namespace gpz {
 
 template <int F, bool PRE>
-__global__ void __launch_bounds__(kThreads, 6) gpz_qse_tile_kernel(QseArgs a) {
+__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
-    __shared__ __align__(8) TileShared S;
+    __shared__ TileShared S;
     if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
         qse_block_tile<F, true, PRE>(a, dsm, S, GridBlock{});
     else
@@ -48,12 +54,12 @@ __global__ void __launch_bounds__(kThreads, 6) gpz_qse_tile_kernel(QseArgs a) {
 
 template <int F, bool PRE>
 cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = tile_smem_bytes(F);
+    const size_t smem = tile_smem_bytes(F, a.perm != nullptr);
     auto kern = gpz_qse_tile_kernel<F, PRE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    kern<<<a.nblocks, kThreads, smem, s>>>(a);
+    kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_qse_general(a, s);

@@ -1,364 +1,313 @@
 // gpz_qse_tile.cuh -- the per-block body of the shared-memory tile
 // compression kernel (Sections 4.1-4.3), used by the single-array kernel
-// (gpz_qse_tile.cu, which describes the design) and by the batched kernel
-// (gpz_batch_compress.cu).  Idx gives the block within its array (b()) and
-// its entry for the general list (id()).
+// (gpz_qse_tile.cu, which describes the design), the interleaved-record
+// kernel (gpz_aos.cu) and the batched kernel (gpz_batch_compress.cu).  Idx
+// gives the block within its array (b()) and its entry for the general list
+// (id()).
 #pragma once
+
+#include <type_traits>
 
 #include "gpz_qse_block.cuh"
 
 namespace gpz {
 
+constexpr int kTileThreads = 128;              // one CTA per particle block
+constexpr int kTileWarps = kTileThreads / 32;
+constexpr int kTileRounds = kBlock / kTileThreads;  // particles per thread
+constexpr int kTileBins = kMaxBins / kTileThreads;  // histogram bins per thread in the scan
+static_assert(kTileBins % 2 == 0 && kTileBins * 11 <= 64, "a thread's counts are appended to one 64-bit word");
+
+// The input tile, which the encoded block's staging words later overlay: an
+// encoding is kept only when it is shorter than the raw block's 1 + F n_b
+// words, so it fits the tile.
+__host__ __device__ constexpr uint32_t tile_region_bytes(int F) { return (uint32_t)F * kBlock * 4u; }
+
+// Dynamic shared memory: the tile, the per-warp histograms and, when the
+// permutation is asked for, the sorted particle indices.
+__host__ __device__ constexpr uint32_t tile_smem_bytes(int F, bool perm) {
+    return tile_region_bytes(F) + (uint32_t)kTileWarps * kMaxBins * 2u + (perm ? kBlock * 2u : 0u);
+}
+
+// Resident CTAs per SM the kernels are compiled for: what shared memory
+// allows (227 KB, 1 KB reserved per CTA, about 0.6 KB of static memory), at
+// most nine (56 registers per thread; more CTAs spill, see gpz_qse_tile.cu).
+constexpr int kTileMaxCtas = 9;
+__host__ __device__ constexpr int tile_ctas(int F) {
+    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, false) + 1024u + 640u));
+    return by_smem < kTileMaxCtas ? by_smem : kTileMaxCtas;
+}
+
 namespace {
 
-__host__ __device__ constexpr uint32_t tile_region_bytes(int F) {
-    const uint32_t tile = (uint32_t)F * kBlock * 4u, stage = kStageWords * 4u;
-    return tile > stage ? tile : stage;
-}
-
-__host__ __device__ constexpr uint32_t tile_smem_bytes(int F) {
-    return tile_region_bytes(F) + kHistBytes + kMaxBins * 2u /*uniq*/ + kMaxBins * 2u /*counts*/ +
-           kBlock * 2u /*perm*/;
-}
-
-// One field's constants for the block, derived once by thread f.
-struct TileField {
-    float mn, inv, s, ebchk;  // block minimum; step constants of the field
-    uint32_t o, ks, wf, bits; // segOffset bits, key shift, record bits, code width
+// One field's constants for the block, derived once by lane f of warp 0.
+struct alignas(16) TileField {
+    float mn, inv;             // block minimum, reciprocal step
+    uint32_t wf, cmask;        // bits in the record and their mask
+    uint32_t rot, kmask;       // segId: the code rotated left by rot, under kmask (its place in the key)
+    float s, ebchk;            // step, verification threshold
+    uint32_t bits, pad[3];     // code width
 };
 
-struct TileShared {
-    uint64_t bar;                       // mbarrier of the tile's bulk copies
-    uint32_t kmin[kMaxFields], kmax[kMaxFields];  // the block's extremes (absolute bound)
+struct alignas(16) TileShared {
+    uint4 blk;                             // flags, record width, key bits
+    uint32_t tn[kTileWarps];               // per warp: particles | non-empty bins << 16
+    uint32_t last[kTileWarps];             // ... its last non-empty bin
+    uint32_t cmax[kTileWarps], dmax[kTileWarps];  // ... largest count and delta
+    uint64_t bar;                          // mbarrier of the tile's bulk copies
+    uint32_t fallback;                     // a value needs a fallback candidate
+    uint2 ext[kMaxFields];                 // the block's extremes (order keys; (0, 0): a non-finite value)
     TileField fc[kMaxFields];
-    // bit 0: a non-finite value; bit 1: a value needs a fallback candidate;
-    // bit 2: a code reaches 2^23 (general path); bit 3: some field's first
-    // candidates need their check
-    uint32_t flags;
-    uint32_t maxcnt, maxdelta;
-    uint32_t warp_tot[kWarps], warp_last[kWarps];
 };
 
-constexpr uint32_t kTfNonFinite = 1u, kTfFallback = 2u, kTfBig = 4u, kTfVerify = 8u;
+constexpr uint32_t kTfNonFinite = 1u;  // a non-finite value: stored raw
+constexpr uint32_t kTfBig = 2u;        // a code reaches 2^23: general path
+constexpr uint32_t kTfVerify = 4u;     // some field's first candidates need their check
 
-// Field f's parameters from the argument block (uniform selection: the
-// by-value parameters are not indexed dynamically).
+// Warp 0, every lane: the fields' constants (lane f) from the block's
+// extremes e and the step constants p: q0 = floor(fma(x - min, 1/s, 1/2)) is
+// monotone in x, so when every value keeps its first candidate the largest
+// code is q0 of the block maximum.
 template <int F>
-__device__ __forceinline__ FieldParams field_params(const QseArgs& a, int f) {
-    if (a.d_params) return a.d_params[f];
-    FieldParams p = a.params[0];
-#pragma unroll
-    for (int k = 1; k < F; ++k)
-        if (k == f) p = a.params[k];
-    return p;
-}
-
-// Field t's constants for the block from its extremes (order keys), by
-// thread t: q0 = floor(fma(x - min, 1/s, 1/2)) is monotone in x, so when
-// every value keeps its first candidate the largest code is q0 of the block
-// maximum.  P is the number of position fields.
-template <int P>
-__device__ __forceinline__ void field_constants(uint32_t kmin, uint32_t kmax, const FieldParams& p, int G, int t,
-                                                TileShared& S) {
-    uint32_t bits;
-    bool big, exact;
-    block_field_width(kmin, kmax, p, bits, big, exact);
-    const float m0 = from_order_key(kmin);
-    TileField c;
-    c.mn = m0 == 0.0f ? 0.0f : m0;  // a zero minimum is stored as +0
-    c.inv = p.inv;
-    c.s = p.s;
-    c.ebchk = p.ebchk;
-    c.bits = bits;
-    const uint32_t g = t < P ? min((uint32_t)G, bits) : 0u;
-    c.o = t < P ? bits - g : 0u;
-    c.wf = t < P ? c.o : bits;
-    c.ks = g;  // this field's segId bits for now; the key shifts follow in every thread
-    S.fc[t] = c;
-    if (big) atomicOr(&S.flags, kTfBig);
-    if (!exact) atomicOr(&S.flags, kTfVerify);
-}
-
-}  // namespace
-
-// AOS: the input is interleaved records (a.interleaved); the tile then holds
-// the block's records as they are in memory, value (f, i) at i * F + f.
-template <int F, bool FULL, bool PRE, class Idx, bool AOS = false>
-__device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, TileShared& S, Idx idx) {
+__device__ __forceinline__ void tile_constants(const uint2 e, const FieldParams& p, int G, TileShared& S) {
     constexpr int P = F < 3 ? F : 3;
+    const int lane = threadIdx.x;
+    const bool fl = lane < F;
+    uint32_t bits = 0u;
+    bool big = false, exact = true;
+    float mn = 0.0f;
+    const bool nonfinite = fl && e.x == 0u;
+    if (fl && e.x != 0u) {
+        block_field_width(e.x, e.y, p, bits, big, exact);
+        const float m0 = from_order_key(e.x);
+        mn = m0 == 0.0f ? 0.0f : m0;  // a zero minimum is stored as +0
+    }
+    const uint32_t g = lane < P ? min((uint32_t)G, bits) : 0u;
+    const uint32_t wf = bits - g;  // a position axis' segOffset bits, an extra field's whole code
+    const uint32_t g1 = __shfl_sync(0xffffffffu, g, 1), g2 = __shfl_sync(0xffffffffu, g, 2);
+    const uint32_t ks = lane == 0 ? g1 + g2 : (lane == 1 ? g2 : 0u);  // the segId bits of the axes after this one
+    const uint32_t W = __reduce_add_sync(0xffffffffu, wf), keybits = __reduce_add_sync(0xffffffffu, g);
+    const uint32_t flags = (__any_sync(0xffffffffu, nonfinite) ? kTfNonFinite : 0u) |
+                           (__any_sync(0xffffffffu, big) ? kTfBig : 0u) |
+                           (__any_sync(0xffffffffu, !exact) ? kTfVerify : 0u);
+    if (fl) {
+        TileField& c = S.fc[lane];
+        c.mn = mn;
+        c.inv = p.inv;
+        c.wf = wf;
+        c.cmask = (1u << (wf & 31u)) - 1u;
+        c.rot = (ks - wf) & 31u;
+        c.kmask = ((1u << g) - 1u) << ks;
+        c.s = p.s;
+        c.ebchk = p.ebchk;
+        c.bits = bits;
+    }
+    if (lane == 0) S.blk = make_uint4(flags, W, keybits, 0u);
+}
+
+// ORs the low n (<= 44) bits of v into the shared words at a bit position.
+__device__ __forceinline__ void or_bits(uint32_t* words, uint32_t pos, unsigned long long v, uint32_t n) {
+    const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32), wi = pos >> 5, end = (pos & 31u) + n;
+    if (n) atomicOr(words + wi, __funnelshift_l(0u, lo, pos));
+    if (end > 32u) atomicOr(words + wi + 1, __funnelshift_l(lo, hi, pos));
+    if (end > 64u) atomicOr(words + wi + 2, __funnelshift_l(hi, 0u, pos));
+}
+
+// Steps 3 to 5 for a block whose records are at most 32 NR bits wide (NR = 2
+// or 4): the common case keeps two registers per record instead of four.
+// AOS: the tile holds records, value (f, i) at i * F + f.
+template <int F, bool FULL, bool AOS, int NR, class Idx>
+__device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, TileShared& S, Idx idx, int n_b,
+                                            uint32_t flags, uint32_t W) {
+    constexpr int P = F < 3 ? F : 3;
+    constexpr int R = kTileRounds, NW = kTileWarps;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const uint32_t b = idx.b();  // the block within its array
-    const uint64_t first = (uint64_t)b * kBlock;
-    const int n_b = FULL ? kBlock : (int)(a.n - first);
-    float* tile = reinterpret_cast<float*>(dsm);                             // [F][1024] input ([1024][F] if AOS)
-    // position of value (f, i) of the block in the tile
-    auto at = [](int f, int i) { return AOS ? i * F + f : f * kBlock + i; };
-    uint32_t* stage = reinterpret_cast<uint32_t*>(dsm);                      // the encoded block, later
-    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F)); // [8][512] per-warp histograms
-    uint16_t* uniq = hist + kWarps * kMaxBins;                               // [512]
-    uint16_t* cnt = uniq + kMaxBins;                                         // [512]
-    uint16_t* sperm = cnt + kMaxBins;                                        // [1024]
+    uint32_t* stage = reinterpret_cast<uint32_t*>(dsm);
+    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F));  // [NW][512] per-warp histograms
+    uint16_t* sperm = hist + NW * kMaxBins;                                    // [1024] (with a.perm)
+    const int i0 = 32 * R * w + lane;  // this thread's particles: i0 + 32 r
+    auto valid = [&](int r) { return FULL || i0 + 32 * r < n_b; };
 
-    // ---- 1. the tile: one bulk copy per field (thread 0); the ragged tail
-    // of a last block by plain loads; the block's extremes
-    // values moved in 16-byte units: per field, or of the whole run of records
-    const uint32_t nvec = AOS ? ((uint32_t)(F * n_b) & ~3u) : ((uint32_t)n_b & ~3u);
-    if (t == 0) {
-        mbar_init(&S.bar, 1);
-        mbar_arrive_expect_tx(&S.bar, (AOS ? 1u : (uint32_t)F) * nvec * 4u);
-        if (nvec) {
-            if (AOS) {
-                bulk_g2s(tile, a.fields[0] + first * F, nvec * 4u, &S.bar);
-            } else {
+    // ---- 3. quantise from the tile, key and record in one pass.  A code is
+    // the low bits of u = 2^23 + q: the rotation puts its segId at the key
+    // place (the exponent bits of u fall outside kmask), the mask takes its
+    // segOffset.
+    uint32_t key[R], rw[R][NR];
 #pragma unroll
-                for (int f = 0; f < F; ++f) bulk_g2s(tile + f * kBlock, a.fields[f] + first, nvec * 4u, &S.bar);
-            }
-        }
-        S.flags = 0u;
-        S.maxcnt = 0u;
-        S.maxdelta = 0u;
-    }
-    if (AOS) {
-        if (!FULL && t < 4) {
-            const int k = (int)nvec + t;
-            if (k < F * n_b) tile[k] = __ldcs(a.fields[0] + first * F + k);
-        }
-    } else if (!FULL && t < 4 * F) {
-        const int f = t >> 2, i = (int)nvec + (t & 3);
-        if (i < n_b) tile[f * kBlock + i] = __ldcs(a.fields[f] + first + i);
-    }
-    {
-        uint32_t* h32 = reinterpret_cast<uint32_t*>(hist + w * kMaxBins);
+    for (int r = 0; r < R; ++r) {
+        key[r] = 0u;
 #pragma unroll
-        for (int k = 0; k < kMaxBins / 64; ++k) h32[lane + 32 * k] = 0u;
+        for (int k = 0; k < NR; ++k) rw[r][k] = 0u;
     }
-    __syncwarp();  // S.flags cleared (thread 0) before threads 0..F-1 of warp 0 set bits in it
-    if (t < F) {
-        if (PRE) {  // from the range pass; (0, 0) marks a non-finite value
-            const uint2 e = __ldg(a.bext + (size_t)b * F + t);
-            const FieldParams p = field_params<F>(a, t);  // loaded with the extremes: one round trip
-            if (e.x == 0u)
-                atomicOr(&S.flags, kTfNonFinite);
-            else
-                field_constants<P>(e.x, e.y, p, a.G, t, S);
-        } else {
-            S.kmin[t] = 0xffffffffu;
-            S.kmax[t] = 0u;
-        }
-    }
-    bool valid[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) valid[r] = FULL || (128 * w + 32 * r + lane < n_b);
-    __syncthreads();  // 1: the mbarrier, the counters and the extremes
-
-    if constexpr (!PRE) {  // the block's extremes from the tile
-        if (!mbar_wait_bounded(&S.bar, 0, a.status)) return;
-        float probe = 0.0f;  // becomes NaN if any value is NaN or infinite (x * 0)
+    auto quantise = [&](auto verify) {
+        constexpr bool VERIFY = decltype(verify)::value;
+        const float* tile = reinterpret_cast<const float*>(dsm);
+        bool pend = false;
 #pragma unroll
         for (int f = 0; f < F; ++f) {
-            float lo = INFINITY, hi = -INFINITY;
+            const uint4 c0 = reinterpret_cast<const uint4*>(&S.fc[f])[0];
+            const uint4 c1 = reinterpret_cast<const uint4*>(&S.fc[f])[1];
+            const float mn = __uint_as_float(c0.x), inv = __uint_as_float(c0.y);
+            const uint32_t wf = c0.z, cmask = c0.w, rot = c1.x, kmask = c1.y;
+            const float s = __uint_as_float(c1.z), ebchk = __uint_as_float(c1.w);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                if (valid[r]) {
-                    const float x = tile[at(f, 128 * w + 32 * r + lane)];
-                    probe = __fmaf_rn(x, 0.0f, probe);
-                    lo = fminf(lo, x);
-                    hi = fmaxf(hi, x);
+            for (int r = 0; r < R; ++r) {
+                const float x = AOS ? tile[(i0 + 32 * r) * F + f] : tile[f * kBlock + i0 + 32 * r];
+                const float tt = __fmaf_rn(__fsub_rn(x, mn), inv, 0.5f);
+                const float u = __fadd_rd(tt, 8388608.0f);  // 2^23 + floor(t), t < 2^23 here
+                if (VERIFY) {
+                    const float xh = __fmaf_rn(__fsub_rn(u, 8388608.0f), s, mn);
+                    pend |= valid(r) && !(fabsf(__fsub_rn(x, xh)) <= ebchk);
                 }
-            }
-            const uint32_t lk = __reduce_min_sync(0xffffffffu, lo == INFINITY ? 0xffffffffu : order_key(lo));
-            const uint32_t hk = __reduce_max_sync(0xffffffffu, hi == -INFINITY ? 0u : order_key(hi));
-            if (lane == 0) {
-                atomicMin(&S.kmin[f], lk);
-                atomicMax(&S.kmax[f], hk);
-            }
-        }
-        if (__any_sync(0xffffffffu, probe != probe) && lane == 0) atomicOr(&S.flags, kTfNonFinite);
-        __syncthreads();  // 1b: the extremes
-    }
-
-    // ---- 2. field constants (thread f) from the tile's extremes
-    // (with a relative bound this was done before barrier 1)
-    if (t < F && !PRE && !(S.flags & kTfNonFinite))
-        field_constants<P>(S.kmin[t], S.kmax[t], field_params<F>(a, t), a.G, t, S);
-    if constexpr (!PRE) __syncthreads();  // 2: the field constants
-    uint32_t flags = S.flags;
-    if (flags & kTfNonFinite) {
-        if (PRE && !mbar_wait_bounded(&S.bar, 0, a.status)) return;  // no copy may outlive the CTA
-        raw_block<F, kCmTemp>(a, b, n_b, t);
-        return;
-    }
-    // key shifts (fields after f below it) and the record width
-    uint32_t W = 0, keybits = 0;
+                const uint32_t ub = __float_as_uint(u);
+                if (f < P) key[r] |= __funnelshift_l(ub, ub, rot) & kmask;
+                // append below the record so far (field 0 ends most significant)
 #pragma unroll
-    for (int f = F - 1; f >= 0; --f) {
-        keybits += f < P ? S.fc[f].ks : 0u;
-        W += S.fc[f].wf;
-    }
-    if ((flags & kTfBig) || W > kFastRecordBits) {
-        if (PRE) mbar_wait_bounded(&S.bar, 0, a.status);
-        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();
-        return;
-    }
-
-    // ---- 3. quantise from the tile, key and record in one pass
-    if (PRE && !mbar_wait_bounded(&S.bar, 0, a.status)) return;
-    uint32_t key[4] = {0u, 0u, 0u, 0u};
-    uint32_t rw[4][4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) rw[r][0] = rw[r][1] = rw[r][2] = rw[r][3] = 0u;
-    bool pend = false;
-    {
-        // key shift of position field f: the segId bits of the position fields after it
-        uint32_t kshift[P];
-        {
-            uint32_t ks = 0;
-#pragma unroll
-            for (int f = P - 1; f >= 0; --f) {
-                kshift[f] = ks;
-                ks += S.fc[f].ks;
+                for (int k = NR - 1; k > 0; --k) rw[r][k] = __funnelshift_l(rw[r][k - 1], rw[r][k], wf);
+                rw[r][0] = (rw[r][0] << wf) | (ub & cmask);
             }
         }
-        const bool verify = (flags & kTfVerify) != 0u, wide = W > 64u;  // uniform
-#pragma unroll
-        for (int f = 0; f < F; ++f) {
-            const TileField c = S.fc[f];
-            FieldParams p;
-            p.eb = 0.0f;
-            p.s = c.s;
-            p.inv = c.inv;
-            p.ebchk = c.ebchk;
-            float x[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) x[r] = tile[at(f, 128 * w + 32 * r + lane)];
-            const uint32_t ks = f < P ? kshift[f < P ? f : 0] : 0u;
-            if (!verify) {
-                if (!wide)
-                    quantise_append<2, false>(x, valid, c.mn, p, f < P, c.o, ks, c.wf, key, rw, pend);
-                else
-                    quantise_append<4, false>(x, valid, c.mn, p, f < P, c.o, ks, c.wf, key, rw, pend);
-            } else {
-                if (!wide)
-                    quantise_append<2, true>(x, valid, c.mn, p, f < P, c.o, ks, c.wf, key, rw, pend);
-                else
-                    quantise_append<4, true>(x, valid, c.mn, p, f < P, c.o, ks, c.wf, key, rw, pend);
-            }
-        }
-        if (verify && __any_sync(0xffffffffu, pend) && lane == 0) atomicOr(&S.flags, kTfFallback);
+        return pend;
+    };
+    if (flags & kTfVerify) {
+        if (__any_sync(0xffffffffu, quantise(std::true_type{})) && lane == 0) S.fallback = 1u;
+    } else {
+        quantise(std::false_type{});
     }
 
     // ---- 4. stable counting sort: warp-local ranks in storage order
     uint16_t* myhist = hist + w * kMaxBins;
-    uint32_t rank[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid[r] ? key[r] : 0xffffffffu);
+    for (int r = 0; r < R; ++r) {
+        const uint32_t peers = __match_any_sync(0xffffffffu, valid(r) ? key[r] : 0xffffffffu);
         uint32_t before = 0u;
-        if (valid[r]) before = myhist[key[r]];
+        if (valid(r)) before = myhist[key[r]];
         __syncwarp();
-        if (valid[r] && lane == 31 - __clz(peers)) myhist[key[r]] = (uint16_t)(before + __popc(peers));
+        if (valid(r)) myhist[key[r]] = (uint16_t)(before + __popc(peers));  // every peer stores the same count
         __syncwarp();
-        rank[r] = before + __popc(peers & lanemask_lt());
+        key[r] |= (before + __popc(peers & lanemask_lt())) << 16;  // the rank above the 9 key bits
     }
     __syncthreads();  // C: every value quantised (the tile is dead) and ranked
-    if (S.flags & kTfFallback) {
+    if (S.fallback) {
         if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();
         return;
     }
+    const uint32_t hdr = 1u + (uint32_t)F + (uint32_t)((F + 3) >> 2);
+    const uint32_t rwords = ceil_words((uint32_t)n_b * W);
     {
-        // the staging words, assembled by OR, overlay the tile: clear them
+        // the staging words, assembled by OR, overlay the tile: clear what
+        // the block can need (deltas <= 512 x 9 bits, counts <= 512 x 11)
+        const uint32_t need = min((hdr + 144u + 176u + rwords + 3u) >> 2, tile_region_bytes(F) / 16u);
         uint4* s4 = reinterpret_cast<uint4*>(stage);
-        for (uint32_t k = t; k < kStageWords / 4u; k += kThreads) s4[k] = make_uint4(0u, 0u, 0u, 0u);
+        for (uint32_t k = t; k < need; k += kTileThreads) s4[k] = make_uint4(0u, 0u, 0u, 0u);
     }
 
-    // ---- 4b. scan over (bin, warp): sorted positions and the run-length code
-    const int nbins = 1 << keybits;
-    const int b0 = 2 * t;
-    uint32_t c0 = 0, c1 = 0;  // counts of bins b0 and b0 + 1 over the warps
-    if (b0 < nbins) {
+    // ---- 4b. scan over (bin, warp): sorted positions and the run-length
+    // code.  Thread t owns bins b0 .. b0 + kTileBins - 1; two 16-bit counts
+    // per word, none of whose sums exceeds 1024.
+    constexpr int BW = kTileBins / 2;
+    const uint32_t b0 = (uint32_t)kTileBins * t;
+    uint32_t row[NW][BW], sum[BW];
 #pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) {
-            const uint32_t pair = *reinterpret_cast<const uint32_t*>(hist + ww * kMaxBins + b0);
-            c0 += pair & 0xffffu;
-            c1 += pair >> 16;
+    for (int k = 0; k < BW; ++k) sum[k] = 0u;
+#pragma unroll
+    for (int ww = 0; ww < NW; ++ww)
+    {
+        const uint16_t* cell = hist + ww * kMaxBins + b0;
+        if constexpr (BW == 2) {
+            const uint2 v = *reinterpret_cast<const uint2*>(cell);
+            row[ww][0] = v.x;
+            row[ww][BW - 1] = v.y;
+        } else {
+            row[ww][0] = *reinterpret_cast<const uint32_t*>(cell);
         }
+#pragma unroll
+        for (int k = 0; k < BW; ++k) sum[k] += row[ww][k];
     }
-    const uint32_t tot = c0 + c1;
-    const uint32_t nz = (c0 ? 1u : 0u) + (c1 ? 1u : 0u);
+    uint32_t c[kTileBins], tot = 0u, nz = 0u, cm = 0u, mylast = 0u;
+#pragma unroll
+    for (int k = 0; k < kTileBins; ++k) {
+        c[k] = (k & 1) ? sum[k >> 1] >> 16 : sum[k >> 1] & 0xffffu;
+        tot += c[k];
+        nz += c[k] ? 1u : 0u;
+        cm = max(cm, c[k]);
+        if (c[k]) mylast = b0 + k;
+    }
     // one scan of both: the counts sum to at most 1024 and the non-empty bins
     // to at most 512, so they share a word
-    const uint32_t incl_tn = warp_incl_sum(tot | (nz << 16));
-    const uint32_t incl_tot = incl_tn & 0xffffu, incl_nz = incl_tn >> 16;
-    const uint32_t cmax = __reduce_max_sync(0xffffffffu, max(c0, c1));
-    // the last non-empty bin up to this thread's (0 when none: a first id's
-    // delta is the id itself), for the deltas of the unique ids
-    uint32_t last = c1 ? (uint32_t)b0 + 1u : (c0 ? (uint32_t)b0 : 0u);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) last = max(last, __shfl_up_sync(0xffffffffu, last, o));
+    const uint32_t incl = warp_incl_sum(tot | (nz << 16));
+    cm = __reduce_max_sync(0xffffffffu, cm);
+    // the last non-empty bin before this thread's, in its warp
+    const uint32_t filled = __ballot_sync(0xffffffffu, tot != 0u), below = filled & lanemask_lt();
+    uint32_t prev = __shfl_sync(0xffffffffu, mylast, below ? 31 - __clz(below) : 0);
+    if (!below) prev = 0u;
+    const uint32_t wlast = __shfl_sync(0xffffffffu, mylast, filled ? 31 - __clz(filled) : 0);
     if (lane == 31) {
-        S.warp_tot[w] = incl_tn;
-        S.warp_last[w] = last;
+        S.tn[w] = incl;
+        S.last[w] = wlast;
+        S.cmax[w] = cm;
     }
-    if (lane == 0) atomicMax(&S.maxcnt, cmax);
     __syncthreads();  // D
-    uint32_t base_tot = 0, base_nz = 0, U = 0, prev = 0;
+    uint32_t excl = incl - (tot | (nz << 16)), all = 0u, maxcnt = 0u;
 #pragma unroll
-    for (int ww = 0; ww < kWarps; ++ww) {
-        const uint32_t vtn = S.warp_tot[ww], vl = S.warp_last[ww];
+    for (int ww = 0; ww < NW; ++ww) {
+        const uint32_t v = S.tn[ww];
         if (ww < w) {
-            base_tot += vtn & 0xffffu;
-            base_nz += vtn >> 16;
-            prev = max(prev, vl);
+            excl += v;
+            prev = max(prev, S.last[ww]);  // 0 when none: a first id's delta is the id itself
         }
-        U += vtn >> 16;
+        all += v;
+        maxcnt = max(maxcnt, S.cmax[ww]);
     }
+    const uint32_t U = all >> 16;
+    uint32_t dm = 0u;
     {
-        const uint32_t up = __shfl_up_sync(0xffffffffu, last, 1);
-        if (lane > 0) prev = max(prev, up);  // the last non-empty bin before b0
-    }
-    uint32_t dmax = 0;
-    if (b0 < nbins) {
-        const uint32_t start0 = base_tot + incl_tot - tot, start1 = start0 + c0;
-        const uint32_t idx0 = base_nz + incl_nz - nz, idx1 = idx0 + (c0 ? 1u : 0u);
-        // each warp's sorted start of the two bins: the start plus the counts
-        // of the warps before it (re-read rather than held across the barrier)
-        uint32_t run = start0 | (start1 << 16);  // neither half overflows: both < 1024
+        uint32_t start = excl & 0xffffu, pv = prev;
+        uint32_t run[BW];
 #pragma unroll
-        for (int ww = 0; ww < kWarps; ++ww) {
-            uint32_t* cell = reinterpret_cast<uint32_t*>(hist + ww * kMaxBins + b0);
-            const uint32_t pair = *cell;
-            *cell = run;
-            run += pair;
+        for (int k = 0; k < kTileBins; ++k) {
+            run[k >> 1] = (k & 1) ? run[k >> 1] | (start << 16) : start;
+            start += c[k];
+            if (c[k]) {
+                dm = max(dm, b0 + k - pv);
+                pv = b0 + k;
+            }
         }
-        if (c0) {
-            uniq[idx0] = (uint16_t)b0;
-            cnt[idx0] = (uint16_t)c0;
+        // each warp's sorted start of the bins: the start plus the counts of the warps before it
+        if (tot) {
+#pragma unroll
+            for (int ww = 0; ww < NW; ++ww)
+            {
+                uint16_t* cell = hist + ww * kMaxBins + b0;
+                if constexpr (BW == 2)
+                    *reinterpret_cast<uint2*>(cell) = make_uint2(run[0], run[BW - 1]);
+                else
+                    *reinterpret_cast<uint32_t*>(cell) = run[0];
+#pragma unroll
+                for (int k = 0; k < BW; ++k) run[k] += row[ww][k];
+            }
         }
-        if (c1) {
-            uniq[idx1] = (uint16_t)(b0 + 1);
-            cnt[idx1] = (uint16_t)c1;
-        }
-        if (c0) dmax = (uint32_t)b0 - prev;
-        if (c1) dmax = max(dmax, (uint32_t)b0 + 1u - (c0 ? (uint32_t)b0 : prev));
     }
-    dmax = __reduce_max_sync(0xffffffffu, dmax);
-    if (lane == 0 && dmax) atomicMax(&S.maxdelta, dmax);
+    dm = __reduce_max_sync(0xffffffffu, dm);
+    if (lane == 0) S.dmax[w] = dm;
     __syncthreads();  // E
+    uint32_t maxdelta = 0u;
+#pragma unroll
+    for (int ww = 0; ww < NW; ++ww) maxdelta = max(maxdelta, S.dmax[ww]);
 
     // ---- encoded size; raw when not smaller (keeps the bound size a bound)
-    const uint32_t wd = bit_width(S.maxdelta), wc = bit_width(S.maxcnt);
-    const uint32_t hdr = 1u + (uint32_t)F + (uint32_t)((F + 3) >> 2);
+    const uint32_t wd = bit_width(maxdelta), wc = bit_width(maxcnt);
     const uint32_t dwords = ceil_words(U * wd), cwords = ceil_words(U * wc);
-    const uint32_t rwords = ceil_words((uint32_t)n_b * W);
     const uint32_t enc = hdr + dwords + cwords + rwords;
+    const uint32_t b = idx.b();
     if (enc >= 1u + (uint32_t)F * (uint32_t)n_b) {
-        raw_block<F, kCmTemp>(a, b, n_b, t);
+        write_raw<F, kTileThreads>(a, b, n_b, t);
         return;
     }
 
     // ---- 5. block header and the three arrays (Section 4.3), assembled in the
-    // cleared staging words -- each thread ORs in two deltas, two counts and
-    // its four records at their positions -- then one bulk copy to the
+    // cleared staging words -- each thread ORs in the deltas and counts of its
+    // bins and its records at their positions -- then one bulk copy to the
     // temporary slot
     if (t == 0) stage[0] = (U << 1) | (wd << 12) | (wc << 17);
     if (t >= 1 && t <= F) stage[t] = __float_as_uint(S.fc[t - 1].mn);
@@ -369,51 +318,160 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
             if ((f >> 2) == t) word |= S.fc[f].bits << (8 * (f & 3));
         stage[1 + F + t] = word;
     }
-    {
-        // deltas and counts of unique ids 2t and 2t+1: at most 2 x 9 and
-        // 2 x 11 bits, so each pair is ORed into at most two words
-        const uint32_t k0 = 2u * (uint32_t)t;
-        if (k0 < U) {
-            const bool two = k0 + 1 < U;
-            const uint32_t u0 = uniq[k0], u1 = two ? (uint32_t)uniq[k0 + 1] : u0;
-            const uint32_t dv = (u0 - (k0 ? (uint32_t)uniq[k0 - 1] : 0u)) | ((u1 - u0) << wd);
-            const uint32_t cv = (uint32_t)cnt[k0] | ((two ? (uint32_t)cnt[k0 + 1] : 0u) << wc);
-            const uint32_t nd = (two ? 2u : 1u) * wd, nc = (two ? 2u : 1u) * wc;
-            const uint32_t dp = 32u * hdr + k0 * wd, cp = 32u * (hdr + dwords) + k0 * wc;
-            if (nd) {
-                atomicOr(stage + (dp >> 5), dv << (dp & 31u));
-                if ((dp & 31u) + nd > 32u) atomicOr(stage + (dp >> 5) + 1, dv >> (32u - (dp & 31u)));
-            }
-            if (nc) {
-                atomicOr(stage + (cp >> 5), cv << (cp & 31u));
-                if ((cp & 31u) + nc > 32u) atomicOr(stage + (cp >> 5) + 1, cv >> (32u - (cp & 31u)));
+    if (tot) {
+        unsigned long long dv = 0ull, cv = 0ull;
+        uint32_t nd = 0u, nc = 0u, pv = prev;
+#pragma unroll
+        for (int k = 0; k < kTileBins; ++k) {
+            if (c[k]) {
+                dv |= (unsigned long long)(b0 + k - pv) << nd;
+                cv |= (unsigned long long)c[k] << nc;
+                nd += wd;
+                nc += wc;
+                pv = b0 + k;
             }
         }
+        const uint32_t k0 = excl >> 16;  // index of the thread's first run
+        or_bits(stage, 32u * hdr + k0 * wd, dv, nd);
+        or_bits(stage, 32u * (hdr + dwords) + k0 * wc, cv, nc);
     }
-    // the records: each thread ORs its own four at their sorted positions
     {
         const uint32_t rbase = 32u * (hdr + dwords + cwords);
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            if (!valid[r]) continue;
-            const uint32_t dest = myhist[key[r]] + rank[r];  // sorted position
-            if (a.perm) sperm[dest] = (uint16_t)(128 * w + 32 * r + lane);
+        for (int r = 0; r < R; ++r) {
+            if (!valid(r)) continue;
+            const uint32_t dest = myhist[key[r] & 0xffffu] + (key[r] >> 16);  // sorted position
+            if (a.perm) sperm[dest] = (uint16_t)(i0 + 32 * r);
             if (W == 0u) continue;
-            const uint32_t bp = rbase + dest * W, wi = bp >> 5, sh = bp & 31u, end = sh + W;
+            const uint32_t bp = rbase + dest * W, end = (bp & 31u) + W;
+            uint32_t* at = stage + (bp >> 5);
             // the record is W bits, least significant word first, zero above W
-            atomicOr(stage + wi, rw[r][0] << sh);
-            if (end > 32u) atomicOr(stage + wi + 1, __funnelshift_l(rw[r][0], rw[r][1], sh));
-            if (end > 64u) atomicOr(stage + wi + 2, __funnelshift_l(rw[r][1], rw[r][2], sh));
-            if (end > 96u) atomicOr(stage + wi + 3, __funnelshift_l(rw[r][2], rw[r][3], sh));
-            if (end > 128u) atomicOr(stage + wi + 4, __funnelshift_l(rw[r][3], 0u, sh));
+            atomicOr(at, __funnelshift_l(0u, rw[r][0], bp));
+#pragma unroll
+            for (int k = 1; k <= NR; ++k)
+                if (end > 32u * k)
+                    atomicOr(at + k, __funnelshift_l(rw[r][k - 1], k < NR ? rw[r][k < NR ? k : 0] : 0u, bp));
         }
     }
     fence_proxy_async_shared();  // the staging words are read by a bulk copy (async proxy)
     __syncthreads();
-    if (t == 0) bulk_s2g(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
-    if (a.perm)
-        for (int j = t; j < n_b; j += kThreads) a.perm[first + j] = (uint32_t)first + sperm[j];
-    if (t == 0) a.sizes[b] = enc;
+    if (t == 0) {
+        a.sizes[b] = enc;
+        bulk_s2g(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
+    }
+    if (a.perm) {
+        const uint64_t first = (uint64_t)b * kBlock;
+        for (int j = t; j < n_b; j += kTileThreads) a.perm[first + j] = (uint32_t)first + sperm[j];
+    }
+}
+
+}  // namespace
+
+// AOS: the input is interleaved records (a.interleaved); the tile then holds
+// the block's records as they are in memory, value (f, i) at i * F + f.
+template <int F, bool FULL, bool PRE, class Idx, bool AOS = false>
+__device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, TileShared& S, Idx idx) {
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    const uint32_t b = idx.b();  // the block within its array
+    const uint64_t first = (uint64_t)b * kBlock;
+    const int n_b = FULL ? kBlock : (int)(a.n - first);
+    float* tile = reinterpret_cast<float*>(dsm);  // [F][1024] input ([1024][F] if AOS)
+
+    // ---- 1. the tile: one bulk copy per field (lane f of warp 0; one copy of
+    // the whole run of records if AOS); the ragged tail of a last block by
+    // plain loads
+    const uint32_t nvec = (AOS ? (uint32_t)(F * n_b) : (uint32_t)n_b) & ~3u;  // values moved in 16-byte units
+    if (w == 0) {
+        if (lane == 0) {
+            mbar_init(&S.bar, AOS ? 1 : F);
+            S.fallback = 0u;
+        }
+        __syncwarp();
+        if (lane < (AOS ? 1 : F)) {
+            mbar_arrive_expect_tx(&S.bar, nvec * 4u);
+            if (nvec) {
+                const float* src = AOS ? a.fields[0] + first * F : a.fields[lane] + first;
+                bulk_g2s(tile + lane * kBlock, src, nvec * 4u, &S.bar);
+            }
+        }
+    }
+    if (!FULL) {
+        if (AOS) {
+            const int k = (int)nvec + t;
+            if (t < 4 && k < F * n_b) tile[k] = __ldcs(a.fields[0] + first * F + k);
+        } else if (t < 4 * F) {
+            const int f = t >> 2, i = (int)nvec + (t & 3);
+            if (i < n_b) tile[f * kBlock + i] = __ldcs(a.fields[f] + first + i);
+        }
+    }
+    {
+        uint4* h4 = reinterpret_cast<uint4*>(dsm + tile_region_bytes(F)) + w * (kMaxBins / 8);
+#pragma unroll
+        for (int k = 0; k < kMaxBins / 256; ++k) h4[lane + 32 * k] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    // ---- 2. the field constants from the block's extremes: those of the
+    // range pass (loaded with the step constants while the tile is in
+    // flight), or found in the tile, a warp per field
+    if constexpr (!PRE) {
+        __syncthreads();  // the mbarrier and the plainly loaded values
+        if (!mbar_wait_bounded(&S.bar, 0, a.status)) return;
+        for (int f = w; f < F; f += kTileWarps) {
+            float lo = INFINITY, hi = -INFINITY;
+            float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;  // become NaN if a value is NaN or infinite (x * 0)
+            if (FULL && !AOS) {
+                const float4* v4 = reinterpret_cast<const float4*>(tile + f * kBlock) + lane;
+#pragma unroll
+                for (int k = 0; k < kBlock / 128; ++k) {
+                    const float4 v = v4[32 * k];
+                    lo = fminf(lo, fminf(fminf(v.x, v.y), fminf(v.z, v.w)));
+                    hi = fmaxf(hi, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+                    p0 = __fmaf_rn(v.x, 0.0f, p0);
+                    p1 = __fmaf_rn(v.y, 0.0f, p1);
+                    p2 = __fmaf_rn(v.z, 0.0f, p2);
+                    p3 = __fmaf_rn(v.w, 0.0f, p3);
+                }
+            } else {
+#pragma unroll 4
+                for (int i = lane; i < n_b; i += 32) {
+                    const float v = AOS ? tile[i * F + f] : tile[f * kBlock + i];
+                    lo = fminf(lo, v);
+                    hi = fmaxf(hi, v);
+                    p0 = __fmaf_rn(v, 0.0f, p0);
+                }
+            }
+            const float probe = __fadd_rn(__fadd_rn(p0, p1), __fadd_rn(p2, p3));
+            const uint32_t lk = __reduce_min_sync(0xffffffffu, lo == INFINITY ? 0xffffffffu : order_key(lo));
+            const uint32_t hk = __reduce_max_sync(0xffffffffu, hi == -INFINITY ? 0u : order_key(hi));
+            const bool nonfinite = __any_sync(0xffffffffu, probe != probe);
+            if (lane == 0) S.ext[f] = nonfinite ? make_uint2(0u, 0u) : make_uint2(lk, hk);
+        }
+        __syncthreads();  // the extremes
+    }
+    if (w == 0) {
+        uint2 e = make_uint2(0u, 0u);
+        FieldParams p = {};
+        if (lane < F) {
+            e = PRE ? __ldg(a.bext + (size_t)b * F + lane) : S.ext[lane];
+            p = a.d_params ? a.d_params[lane] : a.params[lane];
+        }
+        tile_constants<F>(e, p, a.G, S);
+    }
+    __syncthreads();  // the constants (with a range pass also the mbarrier and the plainly loaded values)
+    if (PRE && !mbar_wait_bounded(&S.bar, 0, a.status)) return;  // no copy may outlive the CTA
+    const uint4 blk = S.blk;
+    const uint32_t flags = blk.x, W = blk.y;
+    if (flags & kTfNonFinite) {
+        write_raw<F, kTileThreads>(a, b, n_b, t);
+        return;
+    }
+    if ((flags & kTfBig) || W > kFastRecordBits) {
+        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();
+        return;
+    }
+    if (F <= 2 || W <= 64u)  // two fields of codes below 2^23 never need more
+        tile_encode<F, FULL, AOS, 2>(a, dsm, S, idx, n_b, flags, W);
+    else
+        tile_encode<F, FULL, AOS, 4>(a, dsm, S, idx, n_b, flags, W);
 }
 
 }  // namespace gpz

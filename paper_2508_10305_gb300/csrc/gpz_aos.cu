@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_aos_k
 
 template <int F, bool PRE>
 cudaError_t launch_qse_tile_aos_fp(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = tile_smem_bytes(F, a.perm != nullptr);
+    const size_t smem = tile_smem_bytes(F);
     auto kern = gpz_qse_tile_aos_kernel<F, PRE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);

@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_batch_general_kernel(BatchCom
     const uint32_t count = *(volatile const uint32_t*)g.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
         const uint32_t gb = __ldcg(g.general_list + i);
+        if (gb & kCodedBlock) continue;
         load_chunk_args(g, __ldg(g.block_map + gb), gb, A, slot);
         __syncthreads();
         const uint32_t b = slot[0];
@@ -397,11 +398,11 @@ bool prepare_f() {
            cudaFuncSetAttribute(gpz_batch_compress_kernel<F, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 100) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem_bytes(F, true)) == cudaSuccess &&
+                                (int)tile_smem_bytes(F)) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 100) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem_bytes(F, true)) == cudaSuccess &&
+                                (int)tile_smem_bytes(F)) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_tile_kernel<F, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 100) == cudaSuccess &&
            cudaFuncSetAttribute(gpz_batch_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -427,9 +428,9 @@ void launch_f(const BatchCompressArgs& a, int grid, cudaStream_t s, bool general
     if (general)
         gpz_batch_general_kernel<F><<<grid, kThreads, qse_smem_bytes(F), s>>>(a);
     else if (a.tile && a.pre)
-        gpz_batch_tile_kernel<F, true><<<grid, kTileThreads, tile_smem_bytes(F, a.any_perm != 0), s>>>(a);
+        gpz_batch_tile_kernel<F, true><<<grid, kTileThreads, tile_smem_bytes(F), s>>>(a);
     else if (a.tile)
-        gpz_batch_tile_kernel<F, false><<<grid, kTileThreads, tile_smem_bytes(F, a.any_perm != 0), s>>>(a);
+        gpz_batch_tile_kernel<F, false><<<grid, kTileThreads, tile_smem_bytes(F), s>>>(a);
     else if (a.pre)
         gpz_batch_compress_kernel<F, true><<<grid, kThreads, qse_fast_smem_bytes(), s>>>(a);
     else

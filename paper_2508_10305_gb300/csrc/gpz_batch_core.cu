@@ -122,7 +122,6 @@ gpz_status core_add_compress(BatchCore& c, const gpz_compress_chunk& d) {
     ch.bulk_ok = vec ? 1 : 0;
     c.kind = 0;
     c.any_rel = c.any_rel || q.mode == GPZ_EB_REL;
-    c.any_perm = c.any_perm || d.perm != nullptr;
     c.chunks.push_back(ch);
     return GPZ_OK;
 }
@@ -295,7 +294,6 @@ gpz_status core_enqueue(const BatchCore& c, const BatchDevice& dev, uint8_t* ws,
     a.rdone = reinterpret_cast<uint32_t*>(ws + L.rdone);
     a.rparams = reinterpret_cast<FieldParams*>(ws + L.rparams);
     a.bext = c.any_rel ? reinterpret_cast<uint2*>(ws + L.bext) : nullptr;
-    a.any_perm = c.any_perm ? 1 : 0;
     a.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
     a.sizes = reinterpret_cast<uint32_t*>(ws + L.sizes);
     a.chunk_status = status;

@@ -45,7 +45,6 @@ struct BatchCore {
     uint32_t total_blocks = 0;
     uint64_t temp_words = 0;
     bool any_rel = false;
-    bool any_perm = false;
     int sms = 0;
     gpz_batch_config cfg{};
     BatchLayout L{};

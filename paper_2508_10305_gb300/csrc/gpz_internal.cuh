@@ -73,7 +73,7 @@ struct QseArgs {
     uint32_t* sizes;            // [nblocks] words per block
     uint32_t* perm;             // [n] or nullptr
     uint32_t* status;
-    uint32_t* general_list;     // [nblocks] blocks left to the general kernel
+    uint32_t* general_list;     // [nblocks] blocks left to the general kernel (kCodedBlock: only recorded)
     uint32_t* general_count;    // zeroed
     // Fused compaction only (gpz_qse_direct_kernel): the stream's payload,
     // the words it can hold, the per-block look-back states (zeroed) and a
@@ -83,6 +83,10 @@ struct QseArgs {
     unsigned long long* bstate;
     uint32_t* deferred_count;
 };
+
+// In a general-list entry: a block with a value that takes a fallback
+// candidate, which the tile kernel has coded itself.
+constexpr uint32_t kCodedBlock = 0x80000000u;
 
 constexpr uint32_t kPlaced = 0x80000000u;  // in a block's word count: already in the stream
 
@@ -318,12 +322,16 @@ __device__ __forceinline__ void fence_proxy_async_shared() {
 // One thread: copy `bytes` (a multiple of 16) from shared memory to global
 // memory, both 16-byte aligned, with one bulk copy, and wait until the copy
 // has read its source (so that the CTA may exit or reuse the words).
-__device__ __forceinline__ void bulk_s2g(void* gdst, const void* ssrc, uint32_t bytes) {
+__device__ __forceinline__ void bulk_s2g_start(void* gdst, const void* ssrc, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst), "r"(smem_u32(ssrc)),
                  "r"(bytes)
                  : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_s2g_wait() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_s2g(void* gdst, const void* ssrc, uint32_t bytes) {
+    bulk_s2g_start(gdst, ssrc, bytes);
+    bulk_s2g_wait();
 }
 
 // ---------------------------------------------------------------- acquire / release (look-back scan)

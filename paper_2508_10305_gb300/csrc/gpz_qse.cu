@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_qse_general_kernel(QseArgs a)
     const uint32_t count = *(volatile const uint32_t*)a.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
         const uint32_t b = a.general_list[i];
+        if (b & kCodedBlock) continue;
         if ((uint64_t)(b + 1) * kBlock <= a.n)
             qse_block_general<F, true>(a, dsm, S, b);
         else

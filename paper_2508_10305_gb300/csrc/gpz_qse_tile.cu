@@ -15,9 +15,9 @@
 //   - once every value is quantised the tile is dead, and the encoded
 //     block's staging words are assembled in the same bytes, then written to
 //     the block's temporary slot by one bulk copy.
-// What bounds it: instruction issue (three fields: 75% of the issue slots
-// busy) and, where a warp's keys are mostly distinct, the unit that executes
-// match (62% busy on the snapshot).  Why 128 threads: whatever a block costs
+// What bounds it: instruction issue (71% of the issue slots busy with three
+// fields, 60% with six) and shared-memory wavefronts (66-70% of their peak).
+// Why 128 threads: whatever a block costs
 // per warp rather than per particle (the constants' loads, the scan over
 // (bin, warp), the barriers) halves against 256 threads of four particles,
 // and eight independent particles per thread hide more latency than the
@@ -25,17 +25,27 @@
 // 7,200 (six fields), 1,330 shared-memory wavefronts instead of 1,980.
 // Measured on a 2^26 x 6 snapshot (relative bound): 0.577 -> 0.472 ms; on
 // 10^8 x 3 scan points (absolute bound): 0.750 -> 0.533 ms.
+// Ranks: match runs once per distinct key of a warp's 32 and its unit was 62%
+// busy on the snapshot.  Where the keys are mostly distinct the ranks are
+// the old counts that shared atomics return; the order in which the hardware
+// serves the lanes of one instruction is not defined, so the sorted order is
+// checked and a block it fails goes to the general kernel (none has).  The
+// snapshot 0.472 -> 0.391 ms, 2^25 x 3 uniform positions 0.340 -> 0.170 ms.
+// Fallback candidates (values whose rounding is near the bound) are coded in
+// place, in a second pass of the warps that have one, instead of redoing the
+// block in the general kernel: the scan (2% of its blocks) 0.533 -> 0.502 ms.
 // Residency: shared memory allows seven CTAs per SM for six fields (28 KB
 // each); for three fields nine (56 registers) measured best, 7 / 8 / 9 / 10 /
-// 12 CTAs: 0.565 / 0.544 / 0.533 / 0.540 / 0.550 ms on the scan.
+// 12 CTAs: 0.565 / 0.544 / 0.533 / 0.540 / 0.550 ms on the scan (and with the
+// later steps 7 / 8 / 9: 0.539 / 0.518 / 0.502 ms).
 //
 // With a relative bound the block's extremes come from the range pass and
 // must bound the block's values (they are exact there): codes are monotone in
 // the value, so every code then fits the width derived from the maximum, and
 // every key stays below 2^keybits, which the histogram's indexing relies on.
 //
-// Blocks the fast path cannot take (a value needing a fallback candidate, a
-// code >= 2^23, a record > 128 bits) go to the general kernel's list; blocks
+// Blocks the fast path cannot take (a fallback candidate that could change
+// its field's width, or none that passes, a code >= 2^23, a record > 128 bits) go to the general kernel's list; blocks
 // with a non-finite value or no gain are stored raw -- both exactly as in
 // gpz_qse_block.cuh.
 #include "gpz_qse_tile.cuh"
@@ -54,7 +64,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_kerne
 
 template <int F, bool PRE>
 cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = tile_smem_bytes(F, a.perm != nullptr);
+    const size_t smem = tile_smem_bytes(F);
     auto kern = gpz_qse_tile_kernel<F, PRE>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);

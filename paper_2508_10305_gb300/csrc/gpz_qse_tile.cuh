@@ -23,20 +23,26 @@ static_assert(kTileBins % 2 == 0 && kTileBins * 11 <= 64, "a thread's counts are
 // words, so it fits the tile.
 __host__ __device__ constexpr uint32_t tile_region_bytes(int F) { return (uint32_t)F * kBlock * 4u; }
 
-// Dynamic shared memory: the tile, the per-warp histograms and, when the
-// permutation is asked for, the sorted particle indices.
-__host__ __device__ constexpr uint32_t tile_smem_bytes(int F, bool perm) {
-    return tile_region_bytes(F) + (uint32_t)kTileWarps * kMaxBins * 2u + (perm ? kBlock * 2u : 0u);
-}
+// Dynamic shared memory: the tile and the per-warp histograms, whose space
+// later takes the sorted order (one word per particle).
+constexpr uint32_t kTileHistBytes = (uint32_t)kTileWarps * kMaxBins * 2u;
+static_assert(kTileHistBytes >= kBlock * 4u, "the sorted order overlays the histograms");
+__host__ __device__ constexpr uint32_t tile_smem_bytes(int F) { return tile_region_bytes(F) + kTileHistBytes; }
 
 // Resident CTAs per SM the kernels are compiled for: what shared memory
 // allows (227 KB, 1 KB reserved per CTA, about 0.6 KB of static memory), at
 // most nine (56 registers per thread; more CTAs spill, see gpz_qse_tile.cu).
 constexpr int kTileMaxCtas = 9;
 __host__ __device__ constexpr int tile_ctas(int F) {
-    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, false) + 1024u + 640u));
+    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F) + 1024u + 640u));
     return by_smem < kTileMaxCtas ? by_smem : kTileMaxCtas;
 }
+
+// Ranking a warp's round of 32 keys: match takes time in proportion to the
+// distinct keys (23 cycles of its SM-wide unit per round on scan data, 45 on
+// uniform positions), a shared atomic in proportion to the most lanes on one
+// bank; the first round's distinct keys decide for the others.
+constexpr int kMatchMaxDistinct = 16;
 
 namespace {
 
@@ -55,11 +61,14 @@ struct alignas(16) TileShared {
     uint32_t last[kTileWarps];             // ... its last non-empty bin
     uint32_t cmax[kTileWarps], dmax[kTileWarps];  // ... largest count and delta
     uint64_t bar;                          // mbarrier of the tile's bulk copies
-    uint32_t fallback;                     // a value needs a fallback candidate
+    uint32_t fallback;                     // kFbCoded, kFbGeneral
+    uint32_t unsure;                       // some warp's ranks need the check of the sorted order
     uint2 ext[kMaxFields];                 // the block's extremes (order keys; (0, 0): a non-finite value)
     TileField fc[kMaxFields];
 };
 
+constexpr uint32_t kFbCoded = 1u;      // a value took a fallback candidate
+constexpr uint32_t kFbGeneral = 2u;    // a value the tile kernel cannot code
 constexpr uint32_t kTfNonFinite = 1u;  // a non-finite value: stored raw
 constexpr uint32_t kTfBig = 2u;        // a code reaches 2^23: general path
 constexpr uint32_t kTfVerify = 4u;     // some field's first candidates need their check
@@ -124,7 +133,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     uint32_t* stage = reinterpret_cast<uint32_t*>(dsm);
     uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F));  // [NW][512] per-warp histograms
-    uint16_t* sperm = hist + NW * kMaxBins;                                    // [1024] (with a.perm)
+    uint32_t* order = reinterpret_cast<uint32_t*>(hist);                       // [1024] the sorted order, later
     const int i0 = 32 * R * w + lane;  // this thread's particles: i0 + 32 r
     auto valid = [&](int r) { return FULL || i0 + 32 * r < n_b; };
 
@@ -133,34 +142,58 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     // place (the exponent bits of u fall outside kmask), the mask takes its
     // segOffset.
     uint32_t key[R], rw[R][NR];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        key[r] = 0u;
-#pragma unroll
-        for (int k = 0; k < NR; ++k) rw[r][k] = 0u;
-    }
-    auto quantise = [&](auto verify) {
-        constexpr bool VERIFY = decltype(verify)::value;
+    // MODE 0: first candidates, known to pass.  1: first candidates, checked;
+    // true when one fails.  2: every candidate; true when the block needs the
+    // general path (no candidate passes, or one that could change the
+    // field's width).
+    auto quantise = [&](auto mode) {
+        constexpr int MODE = decltype(mode)::value;
         const float* tile = reinterpret_cast<const float*>(dsm);
         bool pend = false;
 #pragma unroll
+        for (int r = 0; r < R; ++r) {
+            key[r] = 0u;
+#pragma unroll
+            for (int k = 0; k < NR; ++k) rw[r][k] = 0u;
+        }
+        constexpr int UNROLL = MODE == 2 ? 1 : F;  // the rare pass stays a loop
+#pragma unroll UNROLL
         for (int f = 0; f < F; ++f) {
             const uint4 c0 = reinterpret_cast<const uint4*>(&S.fc[f])[0];
             const uint4 c1 = reinterpret_cast<const uint4*>(&S.fc[f])[1];
             const float mn = __uint_as_float(c0.x), inv = __uint_as_float(c0.y);
             const uint32_t wf = c0.z, cmask = c0.w, rot = c1.x, kmask = c1.y;
             const float s = __uint_as_float(c1.z), ebchk = __uint_as_float(c1.w);
+            // the smallest and the largest code of the field's width: a fallback
+            // candidate below the one or above the other could change the width
+            float half = 0.0f, top = 0.0f;
+            if (MODE == 2) {
+                const uint32_t bits = S.fc[f].bits;
+                half = __uint2float_rn((1u << bits) >> 1);
+                top = __uint2float_rn((1u << bits) - 1u);
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 const float x = AOS ? tile[(i0 + 32 * r) * F + f] : tile[f * kBlock + i0 + 32 * r];
                 const float tt = __fmaf_rn(__fsub_rn(x, mn), inv, 0.5f);
                 const float u = __fadd_rd(tt, 8388608.0f);  // 2^23 + floor(t), t < 2^23 here
-                if (VERIFY) {
-                    const float xh = __fmaf_rn(__fsub_rn(u, 8388608.0f), s, mn);
-                    pend |= valid(r) && !(fabsf(__fsub_rn(x, xh)) <= ebchk);
+                uint32_t ub = __float_as_uint(u);
+                if (MODE) {
+                    const float q = __fsub_rn(u, 8388608.0f);
+                    auto ok = [&](float c) { return fabsf(__fsub_rn(x, __fmaf_rn(c, s, mn))) <= ebchk; };
+                    if (MODE == 1) {
+                        pend |= valid(r) && !ok(q);
+                    } else if (valid(r) && !ok(q)) {  // the next candidates, in the format's order
+                        if (q > 0.0f && ok(__fsub_rn(q, 1.0f))) {
+                            pend |= q == half;
+                            ub -= 1u;
+                        } else {
+                            pend |= !(ok(__fadd_rn(q, 1.0f)) && q != top);
+                            ub += 1u;
+                        }
+                    }
                 }
-                const uint32_t ub = __float_as_uint(u);
-                if (f < P) key[r] |= __funnelshift_l(ub, ub, rot) & kmask;
+                if (MODE == 2 || f < P) key[r] |= __funnelshift_l(ub, ub, rot) & kmask;
                 // append below the record so far (field 0 ends most significant)
 #pragma unroll
                 for (int k = NR - 1; k > 0; --k) rw[r][k] = __funnelshift_l(rw[r][k - 1], rw[r][k], wf);
@@ -169,28 +202,54 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
         }
         return pend;
     };
-    if (flags & kTfVerify) {
-        if (__any_sync(0xffffffffu, quantise(std::true_type{})) && lane == 0) S.fallback = 1u;
-    } else {
-        quantise(std::false_type{});
+    if (!(flags & kTfVerify)) {
+        quantise(std::integral_constant<int, 0>{});
+    } else if (__any_sync(0xffffffffu, quantise(std::integral_constant<int, 1>{}))) {
+        const bool fail = __any_sync(0xffffffffu, quantise(std::integral_constant<int, 2>{}));  // rare: once more
+        if (lane == 0) atomicOr(&S.fallback, fail ? kFbGeneral : kFbCoded);
     }
 
-    // ---- 4. stable counting sort: warp-local ranks in storage order
+    // ---- 4. counting sort: warp-local ranks, round after round.  The old
+    // count that the shared atomic returns is the particle's rank; within one
+    // round the lanes of equal keys get distinct ranks in the order in which
+    // the hardware serves them, which is checked below (stability).
     uint16_t* myhist = hist + w * kMaxBins;
+    {
+        uint32_t peers = __match_any_sync(0xffffffffu, valid(0) ? key[0] : 0xffffffffu);
+        if (valid(0)) myhist[key[0]] = (uint16_t)__popc(peers);  // every peer stores the same count
+        const uint32_t rank0 = __popc(peers & lanemask_lt());
+        const int distinct = __popc(__ballot_sync(0xffffffffu, valid(0) && rank0 == 0u));
+        key[0] |= rank0 << 16;  // the rank above the 9 key bits
+        __syncwarp();
+        if (distinct > kMatchMaxDistinct) {
+            if (lane == 0) S.unsure = 1u;
+            uint32_t* h32 = reinterpret_cast<uint32_t*>(myhist);  // two bins per word
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid(r) ? key[r] : 0xffffffffu);
-        uint32_t before = 0u;
-        if (valid(r)) before = myhist[key[r]];
-        __syncwarp();
-        if (valid(r)) myhist[key[r]] = (uint16_t)(before + __popc(peers));  // every peer stores the same count
-        __syncwarp();
-        key[r] |= (before + __popc(peers & lanemask_lt())) << 16;  // the rank above the 9 key bits
+            for (int r = 1; r < R; ++r) {
+                if (valid(r)) {
+                    const uint32_t sh = (key[r] & 1u) << 4;
+                    const uint32_t old = atomicAdd(h32 + (key[r] >> 1), 1u << sh);
+                    key[r] |= ((old >> sh) & 0xffffu) << 16;
+                }
+                __syncwarp();  // the next round's counts come after this one's
+            }
+        } else {
+#pragma unroll
+            for (int r = 1; r < R; ++r) {
+                peers = __match_any_sync(0xffffffffu, valid(r) ? key[r] : 0xffffffffu);
+                uint32_t before = 0u;
+                if (valid(r)) before = myhist[key[r]];
+                __syncwarp();
+                if (valid(r)) myhist[key[r]] = (uint16_t)(before + __popc(peers));
+                __syncwarp();
+                key[r] |= (before + __popc(peers & lanemask_lt())) << 16;
+            }
+        }
     }
     __syncthreads();  // C: every value quantised (the tile is dead) and ranked
-    if (S.fallback) {
-        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();
-        return;
+    if (const uint32_t fb = S.fallback) {
+        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id() | (fb & kFbGeneral ? 0u : kCodedBlock);
+        if (fb & kFbGeneral) return;
     }
     const uint32_t hdr = 1u + (uint32_t)F + (uint32_t)((F + 3) >> 2);
     const uint32_t rwords = ceil_words((uint32_t)n_b * W);
@@ -340,8 +399,8 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (!valid(r)) continue;
-            const uint32_t dest = myhist[key[r] & 0xffffu] + (key[r] >> 16);  // sorted position
-            if (a.perm) sperm[dest] = (uint16_t)(i0 + 32 * r);
+            const uint32_t k9 = key[r] & 0xffffu, dest = myhist[k9] + (key[r] >> 16);  // sorted position
+            key[r] = k9 | (dest << 16);
             if (W == 0u) continue;
             const uint32_t bp = rbase + dest * W, end = (bp & 31u) + W;
             uint32_t* at = stage + (bp >> 5);
@@ -357,12 +416,39 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     __syncthreads();
     if (t == 0) {
         a.sizes[b] = enc;
-        bulk_s2g(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
+        bulk_s2g_start(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
     }
-    if (a.perm) {
+    const bool unsure = S.unsure != 0u;
+    if (unsure || a.perm) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (valid(r)) order[key[r] >> 16] = ((key[r] & 0xffffu) << 10) | (uint32_t)(i0 + 32 * r);
+        __syncthreads();
+    }
+    // ---- the sort was stable if (key, index) increases strictly along the
+    // sorted positions; else the general kernel redoes the block
+    bool bad = false;
+    if (unsure) {
+#pragma unroll
+    for (int k = 0; k < kBlock / (4 * kTileThreads); ++k) {
+        const int j = 4 * (t + kTileThreads * k);
+        const uint4 v = reinterpret_cast<const uint4*>(order)[t + kTileThreads * k];
+        uint32_t next = __shfl_down_sync(0xffffffffu, v.x, 1);
+        if (lane == 31) next = j + 4 < kBlock ? order[j + 4] : 0xffffffffu;
+        bad |= (FULL || j + 1 < n_b) && v.x >= v.y;
+        bad |= (FULL || j + 2 < n_b) && v.y >= v.z;
+        bad |= (FULL || j + 3 < n_b) && v.z >= v.w;
+        bad |= (FULL || j + 4 < n_b) && v.w >= next;
+    }
+        bad = __syncthreads_or(bad);
+    }
+    if (bad) {
+        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();
+    } else if (a.perm) {
         const uint64_t first = (uint64_t)b * kBlock;
-        for (int j = t; j < n_b; j += kTileThreads) a.perm[first + j] = (uint32_t)first + sperm[j];
+        for (int j = t; j < n_b; j += kTileThreads) a.perm[first + j] = (uint32_t)first + (order[j] & 1023u);
     }
+    if (t == 0) bulk_s2g_wait();
 }
 
 }  // namespace
@@ -385,6 +471,7 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         if (lane == 0) {
             mbar_init(&S.bar, AOS ? 1 : F);
             S.fallback = 0u;
+            S.unsure = 0u;
         }
         __syncwarp();
         if (lane < (AOS ? 1 : F)) {

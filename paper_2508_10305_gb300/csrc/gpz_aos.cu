@@ -242,7 +242,7 @@ cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s) {
 // records with contiguous stores (4-byte aligned records; 16-byte stores
 // when they are 16-byte aligned).
 template <int F>
-__global__ void __launch_bounds__(kDecThreads, 8) gpz_decompress_aos_kernel(DecArgs a) {
+__global__ void __launch_bounds__(kDecThreads, F <= 3 ? 10 : 8) gpz_decompress_aos_kernel(DecArgs a) {
     __shared__ DecSharedRec<F> S;
     decode_block<F, DecGridBlock, false, true, DecSharedRec<F>>(a, S, DecGridBlock{});
 }

@@ -13,8 +13,8 @@ namespace gpz {
 // block's table entries (block_loc), so a CTA needs one round trip for its
 // chunk and its place, and one for its words.
 template <int F>
-__global__ void __launch_bounds__(kDecThreads, 8) gpz_batch_decompress_kernel(BatchDecompressArgs g) {
-    __shared__ DecShared S;
+__global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_batch_decompress_kernel(BatchDecompressArgs g) {
+    __shared__ DecShared<F> S;
     __shared__ DecArgs A;
     __shared__ uint32_t s_b;  // block within its chunk
     const int t = threadIdx.x, lane = t & 31;
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(kDecThreads, 8) gpz_batch_decompress_kernel(Ba
         s_b = gb - ch->block_base;
     }
     __syncthreads();
-    decode_block<F, DecSlotBlock, false, false, DecShared, true>(A, S, DecSlotBlock{&s_b}, hw_pre);
+    decode_block<F, DecSlotBlock, false, false, DecShared<F>, true>(A, S, DecSlotBlock{&s_b}, hw_pre);
 }
 
 cudaError_t launch_batch_decompress(const BatchDecompressArgs& a, int F, cudaStream_t s) {

@@ -10,8 +10,19 @@ namespace gpz {
 
 
 constexpr int kDecWarps = kDecThreads / 32;
-// deltas (<= 512 x 9 bits) + counts (<= 512 x 11 bits) + records (<= 1024 x 128 bits)
-constexpr uint32_t kDecStageWords = 144u + 176u + 4096u;
+constexpr int kDecGroups = kBlock / (4 * kDecThreads);  // groups of four positions per thread: 4t.. of each 4 kDecThreads
+constexpr int kDecRuns = kMaxBins / kDecThreads;        // runs per thread
+static_assert(kDecRuns == 4, "a thread's four counts fit a 64-bit window");
+// deltas (<= 512 x 9 bits) + counts (<= 512 x 11 bits) + records (<= 1024 x
+// 128 bits, wider ones are read from the stream)
+__host__ __device__ constexpr uint32_t dec_stage_words(int F) {
+    return 144u + 176u + 32u * (31u * (uint32_t)F < 128u ? 31u * (uint32_t)F : 128u);
+}
+// Resident CTAs per SM: 40 registers per thread for up to three fields (whose
+// staged words leave room for twelve CTAs), 48 for more.  8 / 10 / 12 CTAs:
+// 10^8 x 3 scan points 0.383 / 0.368 / 0.357 ms, a 2^26 x 6 snapshot 0.340 /
+// 0.317 / 0.352 ms.
+__host__ __device__ constexpr int dec_ctas(int F) { return F <= 3 ? 12 : 10; }
 // words read past the staged ones: a value or record is extracted from a
 // window of words that may reach past its array; those bits are never used
 constexpr uint32_t kDecStagePad = 8u;
@@ -19,23 +30,20 @@ constexpr uint32_t kDecStagePad = 8u;
 
 __device__ __forceinline__ uint32_t mask_bits(uint32_t w) { return w >= 32u ? 0xffffffffu : ((1u << w) - 1u); }
 
-// Value k of a fixed-length array of width w (<= 31) starting at A.
-__device__ __forceinline__ uint32_t extract(const uint32_t* A, uint32_t k, uint32_t w) {
-    if (w == 0u) return 0u;
+// Values k .. k + 3 of a fixed-length array of width w (<= 11) held in shared
+// memory (the words after the last value's may lie past the array: their
+// bits are masked off).
+__device__ __forceinline__ void extract4_s(const uint32_t* A, uint32_t k, uint32_t w, uint32_t (&v)[4]) {
     const uint32_t p = k * w;
-    const uint32_t wi = p >> 5, sh = p & 31u;
-    const uint32_t lo = __ldg(A + wi);
-    const uint32_t hi = (sh + w > 32u) ? __ldg(A + wi + 1) : 0u;
-    return __funnelshift_r(lo, hi, sh) & mask_bits(w);
-}
-
-// Value k of a fixed-length array of width w (<= 31) held in shared memory
-// (the word after the value's first may lie past the array: its bits are
-// masked off).
-__device__ __forceinline__ uint32_t extract_s(const uint32_t* A, uint32_t k, uint32_t w) {
-    const uint32_t p = k * w;
-    const uint32_t wi = p >> 5, sh = p & 31u;
-    return __funnelshift_r(A[wi], A[wi + 1], sh) & mask_bits(w);
+    const uint32_t* a = A + (p >> 5);
+    const uint32_t x0 = a[0], x1 = a[1], x2 = a[2], m = (1u << w) - 1u;
+    uint32_t lo = __funnelshift_r(x0, x1, p), hi = __funnelshift_r(x1, x2, p);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        v[i] = lo & m;
+        lo = __funnelshift_r(lo, hi, w);
+        hi >>= w;
+    }
 }
 
 // (float)q for q < 2^23 with two full-rate operations.
@@ -43,21 +51,11 @@ __device__ __forceinline__ float small_u2f(uint32_t q) {
     return __fsub_rn(__uint_as_float(q + 0x4B000000u), 8388608.0f);
 }
 
-// Rebuild four consecutive values x = fma((float)q, step, min) and store them
-// at out[first .. first + 3]: fp32, or widened to fp64 (exact) when OUT64 --
-// then `out` holds a double array's address.
+// Store four consecutive values at out[first .. first + 3]: fp32, or widened
+// to fp64 (exact) when OUT64 -- then `out` holds a double array's address.
 template <bool OUT64>
-__device__ __forceinline__ void store4(float* out, uint64_t first, const uint32_t* qv, uint32_t bits, float s, float mn,
-                                       int left) {
+__device__ __forceinline__ void store4(float* out, uint64_t first, const float* v, int left) {
     if (OUT64) {
-        float v[4];
-        if (bits <= 23u) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(small_u2f(qv[e]), s, mn);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(__uint2float_rn(qv[e]), s, mn);
-        }
         double* dst = reinterpret_cast<double*>(out) + first;
         if (left >= 4 && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
             reinterpret_cast<double2*>(dst)[0] = make_double2((double)v[0], (double)v[1]);
@@ -70,14 +68,6 @@ __device__ __forceinline__ void store4(float* out, uint64_t first, const uint32_
         return;
     }
     float* dst = out + first;
-    float v[4];
-    if (bits <= 23u) {  // uniform: codes below 2^23 convert with one add
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(small_u2f(qv[e]), s, mn);
-    } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(__uint2float_rn(qv[e]), s, mn);
-    }
     if (left >= 4 && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
         __stcs(reinterpret_cast<float4*>(dst), make_float4(v[0], v[1], v[2], v[3]));
     } else {
@@ -97,13 +87,16 @@ constexpr uint32_t rec_words() { return (uint32_t)(kBlock * F + kBlock / 8); }
 
 // store4's values, for records j .. j + 3 of field f, into that staging.
 template <int F>
-__device__ __forceinline__ void store4_rec(float* recs, int j, int f, const uint32_t* qv, uint32_t bits, float s,
-                                           float mn, int left) {
+__device__ __forceinline__ void store4_rec(float* recs, int j, int f, const float* v, int left) {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const float q = bits <= 23u ? small_u2f(qv[e]) : __uint2float_rn(qv[e]);
-        if (e < left) recs[rec_slot<F>(j + e, f)] = __fmaf_rn(q, s, mn);
-    }
+    for (int e = 0; e < 4; ++e)
+        if (e < left) recs[rec_slot<F>(j + e, f)] = v[e];
+}
+
+// x = fma((float)q, step, min) of four codes.
+__device__ __forceinline__ void rebuild4(const uint32_t* q, uint32_t bits, float s, float mn, float* v) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(bits <= 23u ? small_u2f(q[e]) : __uint2float_rn(q[e]), s, mn);
 }
 
 // Records wider than 128 bits (rare): every code is read field by field from
@@ -153,10 +146,12 @@ __device__ __forceinline__ void decode_wide(const DecArgs& a, const uint32_t* bl
             }
             qv[e] = f < P ? (code | (((key[e] >> kacc[f]) & gm) << wfv[f])) : code;
         }
+        float v[4];
+        rebuild4(qv, bf, sf, mnf, v);
         if (AOS)
-            store4_rec<F>(recs, j0, f, qv, bf, sf, mnf, n_b - j0);
+            store4_rec<F>(recs, j0, f, v, n_b - j0);
         else
-            store4<OUT64>(a.out[f], first + j0, qv, bf, sf, mnf, n_b - j0);
+            store4<OUT64>(a.out[f], first + j0, v, n_b - j0);
     }
 }
 
@@ -167,16 +162,18 @@ struct DecCore {  // everything a block's decoding keeps in shared memory but it
     uint32_t bad;
     // the block's constants, checked by warp 0 and read by every warp
     uint32_t ok, raw, U, wd, wc, W, keybits, G;
-    uint4 lay[kMaxFields];      // per field: bits in the record, segId bits of a position axis,
-                                // segId mask shifted above the segOffset bits, code width
-    float2 ms[kMaxFields];      // per field: block minimum, step
+    uint4 lay[kMaxFields];      // per field: bits in the record and their mask, segId bits of a position
+                                // axis, segId mask shifted above the segOffset bits
+    float4 ms[kMaxFields];      // per field: block minimum, step, the code width's bits (as an integer), 0
 };
 
+template <int F>
 struct DecShared : DecCore {
+    static constexpr uint32_t kWords = dec_stage_words(F);
     uint64_t bar;  // the staging bulk copy
     // the block's words after its header, from word `shift` (the source's
     // offset from a 16-byte boundary, 0..3)
-    alignas(16) uint32_t stage[kDecStageWords + kDecStagePad + 4];
+    alignas(16) uint32_t stage[kWords + kDecStagePad + 4];
 };
 
 // The same for interleaved output: the stage also takes the block's values
@@ -184,50 +181,84 @@ struct DecShared : DecCore {
 constexpr uint32_t cmax(uint32_t x, uint32_t y) { return x > y ? x : y; }
 template <int F>
 struct DecSharedRec : DecCore {
+    static constexpr uint32_t kWords = dec_stage_words(F);
     uint64_t bar;
-    alignas(16) uint32_t stage[cmax(kDecStageWords + kDecStagePad + 4, 4 + rec_words<F>())];
+    alignas(16) uint32_t stage[cmax(kWords + kDecStagePad + 4, 4 + rec_words<F>())];
 };
 
-// Codes of fields F-1 .. 0 of four records, consumed from the least
-// significant end: field F-1 sits at bit 0 of the record and field 0 at the
-// top.  rr[e] holds record e in its low bits (two words when W <= 64, else
+// NG groups of four positions (j[g] .. j[g] + 3, keys key[g]): their records
+// from the staged words, then the codes of fields F-1 .. 0, consumed from the
+// least significant end: field F-1 sits at bit 0 of the record and field 0 at
+// the top.  rr holds a record in its low bits (two words when W <= 64, else
 // four); after each field the record is shifted right by the field's width
 // and the key right by the axis' segId bits.  q = segId * 2^o + segOffset for
-// a position axis, the whole code otherwise.
-template <int F, bool WIDE, bool OUT64 = false, bool AOS = false>
-__device__ __forceinline__ void decode_fields(const DecArgs& a, uint32_t (&rr)[4][4], uint32_t (&key)[4],
-                                              const DecCore& L, uint64_t first, int left, float* recs = nullptr,
-                                              int jl = 0) {
+// a position axis, the whole code otherwise.  Words past the record array
+// (inside the staging pad) hold bits above W, which are never consumed.
+// AOS: sync() once every record is in registers, then the values go to recs.
+template <int F, int NG, bool WIDE, bool OUT64, bool AOS, class Sync>
+__device__ __forceinline__ void decode_groups(const DecArgs& a, const DecCore& L, const uint32_t* sR, uint32_t W,
+                                              const int (&j)[NG], uint32_t (&key)[NG][4], uint64_t base, int n_b,
+                                              float* recs, Sync sync) {
     constexpr int P = F < 3 ? F : 3;
+    constexpr int NR = WIDE ? 4 : 2;
+    uint32_t rr[NG][4][NR];
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t p = (uint32_t)(j[g] + e) * W;
+            const uint32_t* at = sR + (p >> 5);
+            uint32_t x = at[0];
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                const uint32_t y = at[k + 1];
+                rr[g][e][k] = __funnelshift_r(x, y, p);
+                x = y;
+            }
+        }
+    sync();
 #pragma unroll
     for (int f = F - 1; f >= 0; --f) {
         const uint4 lay = L.lay[f];
-        const uint32_t wf = lay.x, cm = mask_bits(wf);
-        uint32_t qv[4];
+        const float4 ms = L.ms[f];
+        const uint32_t wf = lay.x, cm = lay.y;
+        const bool small = __float_as_uint(ms.z) <= 23u;  // uniform: codes below 2^23 convert with one add
+        float v[NG][4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            uint32_t q = rr[e][0] & cm;
-            if (f < P) {
-                q |= (key[e] << wf) & lay.z;
-                key[e] >>= lay.y;
-            }
-            qv[e] = q;
-            if (f > 0) {
-                rr[e][0] = __funnelshift_r(rr[e][0], rr[e][1], wf);
-                if (WIDE) {
-                    rr[e][1] = __funnelshift_r(rr[e][1], rr[e][2], wf);
-                    rr[e][2] = __funnelshift_r(rr[e][2], rr[e][3], wf);
-                    rr[e][3] >>= wf;
-                } else {
-                    rr[e][1] >>= wf;
+        for (int g = 0; g < NG; ++g)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t q = rr[g][e][0] & cm;
+                if (f < P) {
+                    q |= (key[g][e] << wf) & lay.w;
+                    key[g][e] >>= lay.z;
+                }
+                v[g][e] = __uint_as_float(q);
+                if (f > 0) {
+#pragma unroll
+                    for (int k = 0; k < NR; ++k)
+                        rr[g][e][k] = k + 1 < NR ? __funnelshift_r(rr[g][e][k], rr[g][e][k + 1 < NR ? k + 1 : k], wf)
+                                                 : rr[g][e][k] >> wf;
                 }
             }
+        if (small) {
+#pragma unroll
+            for (int g = 0; g < NG; ++g)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[g][e] = __fmaf_rn(small_u2f(__float_as_uint(v[g][e])), ms.y, ms.x);
+        } else {
+#pragma unroll
+            for (int g = 0; g < NG; ++g)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[g][e] = __fmaf_rn(__uint2float_rn(__float_as_uint(v[g][e])), ms.y, ms.x);
         }
-        const float2 ms = L.ms[f];
-        if (AOS)
-            store4_rec<F>(recs, jl, f, qv, lay.w, ms.y, ms.x, left);
-        else
-            store4<OUT64>(a.out[f], first, qv, lay.w, ms.y, ms.x, left);
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            if (AOS)
+                store4_rec<F>(recs, j[g], f, v[g], n_b - j[g]);
+            else
+                store4<OUT64>(a.out[f], base + j[g], v[g], n_b - j[g]);
+        }
     }
 }
 
@@ -243,7 +274,6 @@ struct DecSlotBlock {
     __device__ __forceinline__ uint32_t b() const { return *slot; }
 };
 
-// Decode block idx.b() of the stream described by a (every thread of the CTA).
 // The format checks and the block's constants (warp 0 alone; every lane
 // calls): from the stream header words hv (lane k holds word k), the block's
 // first words bw (lane k holds word k, up to the block header's end) and the
@@ -314,8 +344,8 @@ __device__ __forceinline__ void decode_checks(const DecArgs& a, DecCore& S, uint
         S.G = G;
     }
     if (fl) {
-        S.lay[lane] = make_uint4(wf, g, mask_bits(g) << wf, bf);  // g + wf = bits <= 31
-        S.ms[lane] = make_float2(mn, step);
+        S.lay[lane] = make_uint4(wf, mask_bits(wf), g, mask_bits(g) << wf);  // g + wf = bits <= 31
+        S.ms[lane] = make_float4(mn, step, __uint_as_float(bf), 0.0f);
     }
 }
 
@@ -395,53 +425,55 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
     // the deltas, counts and (when at most 128 bits wide) the records are in
     // the staging area, contiguous as in the stream
     const bool fast = W <= 128u;  // then dwords + cwords + rwords <= the staged words
-    const uint32_t ndc = dwords + cwords;
-    const uint32_t* sD = stage;
-    const uint32_t* sC = stage + dwords;
-    const uint32_t* sR = stage + ndc;
-    const uint32_t k0 = 2u * t, k1 = k0 + 1u;
-    const bool v0 = k0 < U, v1 = k1 < U;
-    uint32_t d0 = v0 ? extract_s(sD, k0, wd) : 0u, d1 = v1 ? extract_s(sD, k1, wd) : 0u;
-    uint32_t c0 = v0 ? extract_s(sC, k0, wc) : 0u, c1 = v1 ? extract_s(sC, k1, wc) : 0u;
+    const uint32_t* sR = stage + dwords + cwords;
+    const uint32_t k0 = (uint32_t)kDecRuns * t;
+    const int nrun = (int)min((uint32_t)kDecRuns, U > k0 ? U - k0 : 0u);  // this thread's runs
 
     // ---- 3. unique ids and run starts
     {
-        bool bad = (v0 && (d0 >= idlimit || c0 == 0u || c0 > (uint32_t)n_b || (k0 > 0 && d0 == 0u))) ||
-                   (v1 && (d1 >= idlimit || c1 == 0u || c1 > (uint32_t)n_b || d1 == 0u));
-        if (bad) d0 = d1 = c0 = c1 = 0u;  // keep the sums small; the block is rejected below
-        // one scan of both sums: a warp's id sum is below 2^15 (32 x 2 x 511)
-        // and its count sum at most 2^16 (32 x 2 x 1024), so they share a word
-        const uint32_t su = d0 + d1, sc = c0 + c1;
-        const uint32_t iuc = warp_incl_sum(su | (sc << 15));
-        const uint32_t iu = iuc & 0x7fffu, ic = iuc >> 15;
+        uint32_t d[kDecRuns], c[kDecRuns], su = 0u, sc = 0u;
+        extract4_s(stage, min(k0, U), wd, d);
+        extract4_s(stage + dwords, min(k0, U), wc, c);
+        bool bad = false;
+#pragma unroll
+        for (int k = 0; k < kDecRuns; ++k) {
+            if (k < nrun) {
+                bad |= c[k] == 0u || (d[k] == 0u && k0 + k > 0u);
+                su += d[k];
+                sc += c[k];
+            }
+        }
+        // one scan of both sums; a thread's ids beyond 511 or counts beyond
+        // 1024 already make the block corrupt, and without them a warp's id sum
+        // is below 2^14 and its count sum at most 2^15
+        if (su > 511u || sc > 1024u) {
+            bad = true;
+            su = sc = 0u;
+        }
+        const uint32_t iuc = warp_incl_sum(su | (sc << 14));
         if (lane == 31) S.warp_uc[w] = iuc;
         __syncthreads();
-        uint32_t bu = 0, bc = 0, total = 0;
+        uint32_t u = (iuc & 0x3fffu) - su, st = (iuc >> 14) - sc, total = 0;
 #pragma unroll
         for (int ww = 0; ww < kDecWarps; ++ww) {
-            const uint32_t uc = S.warp_uc[ww], cu = uc & 0x7fffu, cc = uc >> 15;
+            const uint32_t uc = S.warp_uc[ww];
             if (ww < w) {
-                bu += cu;
-                bc += cc;
+                u += uc & 0x3fffu;
+                st += uc >> 14;
             }
-            total += cc;
+            total += uc >> 14;
         }
-        const uint32_t u0 = bu + iu - su + d0, u1 = u0 + d1;
-        const uint32_t s0 = bc + ic - sc, s1 = s0 + c0;
-        if (v0) {
-            if (u0 >= idlimit || s0 >= (uint32_t)n_b) {
-                bad = true;
-            } else {
-                uniq[k0] = (uint16_t)u0;
-                atomicOr(&mask[s0 >> 5], 1u << (s0 & 31u));
-            }
-        }
-        if (v1) {
-            if (u1 >= idlimit || s1 >= (uint32_t)n_b) {
-                bad = true;
-            } else {
-                uniq[k1] = (uint16_t)u1;
-                atomicOr(&mask[s1 >> 5], 1u << (s1 & 31u));
+#pragma unroll
+        for (int k = 0; k < kDecRuns; ++k) {
+            if (k < nrun && !bad) {
+                u += d[k];
+                if (u >= idlimit || st >= (uint32_t)n_b) {
+                    bad = true;
+                } else {
+                    uniq[k0 + k] = (uint16_t)u;
+                    atomicOr(&mask[st >> 5], 1u << (st & 31u));
+                }
+                st += c[k];
             }
         }
         if (t == 0 && total != (uint32_t)n_b) bad = true;
@@ -452,69 +484,55 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
         if (t == 0) set_status(a.status, kStCorrupt);
         return;
     }
-    // every warp scans the 32 mask words itself (no further barrier): lane i
-    // holds word i and the run starts before it; thread t's positions lie in
-    // word t/8
-    uint32_t mrow, prow;
+
+    // ---- 4. the run of position j is the number of run starts up to j, less
+    // one: every warp scans the 32 mask words itself (no further barrier; lane
+    // i holds word i and the starts before it); a group's four positions lie in
+    // one word, and position 0 starts a run, so every index is in 0..U-1
+    int j[kDecGroups];
+    uint32_t key[kDecGroups][4];
     {
         const uint32_t mw = mask[lane];
         const uint32_t pc = __popc(mw);
         const uint32_t pre = warp_incl_sum(pc) - pc;
-        const int src = (t >> 3) & 31;
-        mrow = __shfl_sync(0xffffffffu, mw, src);
-        prow = __shfl_sync(0xffffffffu, pre, src);
+#pragma unroll
+        for (int g = 0; g < kDecGroups; ++g) {
+            j[g] = 4 * (t + g * kDecThreads);
+            const uint32_t m = __shfl_sync(0xffffffffu, mw, j[g] >> 5) >> (j[g] & 31);
+            const uint32_t before = __shfl_sync(0xffffffffu, mw, j[g] >> 5) & ((1u << (j[g] & 31)) - 1u);
+            uint32_t run = __shfl_sync(0xffffffffu, pre, j[g] >> 5) + __popc(before) - 1u;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                run += (m >> e) & 1u;
+                key[g][e] = uniq[run];
+            }
+        }
     }
-
-    // ---- 4. positions 4t..4t+3 (with interleaved output every thread stays
-    // for the barriers of the staging in record order)
-    const int j0 = 4 * t;
-    if (!AOS && j0 >= n_b) return;
-    const bool act = j0 < n_b;
+    const uint64_t base = (uint64_t)b * kBlock;
     float* recs = reinterpret_cast<float*>(stage);  // AOS, once the stage's words are consumed
-    uint32_t key[4] = {0u, 0u, 0u, 0u};
-    if (act) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const uint32_t bit = (uint32_t)(j0 + e) & 31u;
-            int run = (int)(prow + __popc(mrow & ((2u << bit) - 1u))) - 1;
-            run = run < 0 ? 0 : (run >= (int)U ? (int)U - 1 : run);
-            key[e] = uniq[run];
-        }
-    }
+    auto sync = [] {
+        if (AOS) __syncthreads();
+    };
     if (!fast) {
-        if (AOS) __syncthreads();  // the staged deltas and counts are consumed
-        if (act)
-            decode_wide<F, OUT64, AOS>(a, blk, hdr + dwords + cwords, rwords, W, S.G, j0, n_b, (uint64_t)b * kBlock,
-                                       key[0], key[1], key[2], key[3], recs);
-        if (AOS) store_records<F>(a, recs, b, n_b);
-        return;
-    }
-    // records j0..j0+3 from the staged words; words past the record array
-    // (inside the staging pad) hold bits above W, which are never consumed
-    const bool wide = W > 64u;
-    uint32_t rr[4][4];
+        sync();  // the staged deltas and counts are consumed
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const uint32_t p = (uint32_t)((act ? j0 : 0) + e) * W;
-        const uint32_t wi = p >> 5, sh = p & 31u;
-        const uint32_t x0 = sR[wi], x1 = sR[wi + 1], x2 = sR[wi + 2];
-        rr[e][0] = __funnelshift_r(x0, x1, sh);
-        rr[e][1] = __funnelshift_r(x1, x2, sh);
-        if (wide) {
-            const uint32_t x3 = sR[wi + 3], x4 = sR[wi + 4];
-            rr[e][2] = __funnelshift_r(x2, x3, sh);
-            rr[e][3] = __funnelshift_r(x3, x4, sh);
-        } else {
-            rr[e][2] = rr[e][3] = 0u;
+        for (int g = 0; g < kDecGroups; ++g)
+            if (j[g] < n_b)
+                decode_wide<F, OUT64, AOS>(a, blk, hdr + dwords + cwords, rwords, W, S.G, j[g], n_b, base, key[g][0],
+                                           key[g][1], key[g][2], key[g][3], recs);
+    } else if (W <= 64u) {
+        decode_groups<F, kDecGroups, false, OUT64, AOS>(a, S, sR, W, j, key, base, n_b, recs, sync);
+    } else if (AOS) {  // every record in registers before the first value is staged
+        decode_groups<F, kDecGroups, true, OUT64, AOS>(a, S, sR, W, j, key, base, n_b, recs, sync);
+    } else {
+#pragma unroll 1
+        for (int g = 0; g < kDecGroups; ++g) {
+            const int jg[1] = {g == 0 ? j[0] : j[kDecGroups - 1]};
+            uint32_t kg[1][4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) kg[0][e] = g == 0 ? key[0][e] : key[kDecGroups - 1][e];
+            decode_groups<F, 1, true, OUT64, AOS>(a, S, sR, W, jg, kg, base, n_b, recs, sync);
         }
-    }
-    const uint64_t first = (uint64_t)b * kBlock + j0;
-    if (AOS) __syncthreads();  // every record is in registers: the stage takes the values
-    if (act) {
-        if (wide)
-            decode_fields<F, true, OUT64, AOS>(a, rr, key, S, first, n_b - j0, recs, j0);
-        else
-            decode_fields<F, false, OUT64, AOS>(a, rr, key, S, first, n_b - j0, recs, j0);
     }
     if (AOS) store_records<F>(a, recs, b, n_b);
 }
@@ -524,7 +542,7 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
 // DecSharedRec<F>).  PREHW: lanes 0, 1, 2 of every warp pass in hw_pre the
 // words round trip 1 would load (the payload size and the block's two table
 // entries), loaded earlier by the caller.
-template <int F, class Idx, bool OUT64 = false, bool AOS = false, class Sh = DecShared, bool PREHW = false>
+template <int F, class Idx, bool OUT64 = false, bool AOS = false, class Sh = DecShared<F>, bool PREHW = false>
 __device__ __forceinline__ void decode_block(const DecArgs& a, Sh& S, Idx idx, uint32_t hw_pre = 0u) {
     uint32_t* stage = S.stage;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -572,7 +590,7 @@ __device__ __forceinline__ void decode_block(const DecArgs& a, Sh& S, Idx idx, u
     const uint32_t shift = (uint32_t)((reinterpret_cast<uintptr_t>(src) >> 2) & 3u);
     uint32_t nst = 0, units = 0;
     if (inside && nw > hdr) {
-        nst = min(nw - hdr, kDecStageWords);
+        nst = min(nw - hdr, Sh::kWords);
         const uint64_t avail = a.total_words - (uint64_t)(src - Sw) + shift;  // words from the boundary to the stream's end
         units = (uint32_t)(min((uint64_t)(nst + shift + 3u), avail) >> 2);
         if (units * 4u < shift) units = 0;

@@ -19,7 +19,7 @@ constexpr int kMaxBins = 512;            // 2^(3 * kMaxSegBits) linearised segme
 constexpr int kRow = 33;                 // padded shared-memory row of 32 values
 constexpr int kPadWords = 32 * kRow;     // 1056: 1024 values in padded rows
 constexpr int kQseThreads = 256;         // one CTA per particle block, 4 particles per thread
-constexpr int kDecThreads = 256;         // one CTA per particle block, 4 positions per thread
+constexpr int kDecThreads = 128;         // one CTA per particle block, 8 positions per thread
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;

@@ -108,8 +108,7 @@ uint64_t gpz_decompress_workspace_size(void);
 
 /* Compress (Sections 4.1-4.4).
  *   d_fields:     host array of n_fields device pointers, field f's n fp32
- *                 values at d_fields[f]; each 4-byte aligned (16-byte
- *                 alignment enables bulk-copy staging).
+ *                 values at d_fields[f]; each 4-byte aligned.
  *   n:            particles (0 allowed: the stream is then a bare header).
  *   p:            parameters (host).
  *   d_out:        device buffer for the stream, 16-byte aligned, of

@@ -59,7 +59,7 @@ def build(force=False, verbose=False, ptxas_info=False):
             raise RuntimeError("nvcc failed for %s:\n%s%s" % (src, r.stdout, r.stderr))
         return obj, r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(max(8, os.cpu_count() or 8), len(srcs))) as ex:
         results = list(ex.map(compile_one, srcs))
     if verbose or ptxas_info:
         for _, err in results:

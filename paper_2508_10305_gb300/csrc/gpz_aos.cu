@@ -13,7 +13,7 @@
 #include "gpz.h"
 #include "gpz_host.hpp"
 #include "gpz_internal.cuh"
-#include "gpz_qse_tile.cuh"
+#include "gpz_qse_tile_launch.cuh"
 #include "gpz_decode_block.cuh"
 
 using namespace gpz;
@@ -195,47 +195,7 @@ __global__ void __launch_bounds__(kAosThreads) gpz_aos_range_kernel(const float*
 // Compression straight from 16-byte aligned interleaved records: the tile
 // kernel's body with the block's records as its tile (one bulk copy of
 // 1024 F contiguous values), so no structure-of-arrays copy is made.
-template <int F, bool PRE>
-__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_aos_kernel(const __grid_constant__ QseArgs a) {
-    extern __shared__ __align__(128) uint8_t dsm[];
-    __shared__ TileShared S;
-    if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
-        qse_block_tile<F, true, PRE, GridBlock, true>(a, dsm, S, GridBlock{});
-    else
-        qse_block_tile<F, false, PRE, GridBlock, true>(a, dsm, S, GridBlock{});
-}
-
-template <int F, bool PRE>
-cudaError_t launch_qse_tile_aos_fp(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = tile_smem_bytes(F);
-    auto kern = gpz_qse_tile_aos_kernel<F, PRE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_qse_general(a, s);
-}
-
-cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s) {
-    if (a.nblocks == 0) return cudaSuccess;
-    const bool pre = a.bext != nullptr;
-    switch (a.F) {
-#define GPZ_CASE(FF) \
-    case FF: return pre ? launch_qse_tile_aos_fp<FF, true>(a, s) : launch_qse_tile_aos_fp<FF, false>(a, s);
-        GPZ_CASE(1)
-        GPZ_CASE(2)
-        GPZ_CASE(3)
-        GPZ_CASE(4)
-        GPZ_CASE(5)
-        GPZ_CASE(6)
-        GPZ_CASE(7)
-        GPZ_CASE(8)
-#undef GPZ_CASE
-    }
-    return cudaErrorInvalidValue;
-}
+cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s) { return launch_qse_tile_layout<kTileRecords>(a, s); }
 
 // Decompression into interleaved records: the block decoder stages the
 // block's values in record order in shared memory and writes the block's
@@ -244,7 +204,7 @@ cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s) {
 template <int F>
 __global__ void __launch_bounds__(kDecThreads, F <= 3 ? 10 : 8) gpz_decompress_aos_kernel(DecArgs a) {
     __shared__ DecSharedRec<F> S;
-    decode_block<F, DecGridBlock, false, true, DecSharedRec<F>>(a, S, DecGridBlock{});
+    decode_block<F, kOutRecords, false>(a, S, DecGridBlock{});
 }
 
 cudaError_t launch_decompress_aos(const DecArgs& a, cudaStream_t s) {

@@ -2,8 +2,8 @@
 // Validates arguments, lays out the workspace, finalises the per-field
 // constants and enqueues the kernels on the caller's stream:
 //   compress:   [range (relative bound)] -> Q.S.E. (shared-memory tile kernel,
-//               or, for fields not 16-byte aligned, block widths + register
-//               kernel) -> look-back scan -> copy
+//               or, with fused compaction, the register kernel) -> look-back
+//               scan -> copy
 //   decompress: decode
 #include <atomic>
 #include <cmath>
@@ -284,15 +284,12 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         const bool rel = p->mode == GPZ_EB_REL;
         if (!rel)
             for (int f = 0; f < F; ++f) hp[f] = finalise(p->eb[f]);
-        bool vec_ok = true;
-        for (int f = 0; f < F && n > 0; ++f) vec_ok = vec_ok && aligned(d_fields[f], 16);
-        if (interleaved) vec_ok = aligned(interleaved, 16);
         const bool fused = (p->flags & GPZ_FLAG_FUSED_COMPACTION) != 0u;
-        // the shared-memory tile kernel takes 16-byte aligned fields and derives
-        // each block's widths itself; the register kernel reads them from the
+        // the shared-memory tile kernel derives each block's widths itself; the
+        // register kernel of the fused compaction reads them from the
         // block-info pass (relative bound)
-        const bool tile = vec_ok && !fused;
-        if (interleaved && (!tile || (rel && !range_done))) {  // the caller's side of the contract
+        // the caller's side of the contract
+        if (interleaved && (fused || !aligned(interleaved, 16) || (rel && !range_done))) {
             rc = GPZ_ERR_INVALID_ARG;
             break;
         }
@@ -305,7 +302,6 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
             }
             ra.n = n;
             ra.F = F;
-            ra.vec_ok = vec_ok ? 1 : 0;
             ra.partials = reinterpret_cast<float2*>(ws + L.partials);
             ra.done_counter = range_counter;
             ra.d_params = d_params;
@@ -316,7 +312,7 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
                 if ((rc = cuda_status(launch_range(ra, grid, s))) != GPZ_OK) break;
                 rec.mark("range");
             }
-            if (nb > 0 && !tile) {
+            if (nb > 0 && fused) {
                 if ((rc = cuda_status(launch_block_info(ra.bext, d_params, (uint32_t)nb, F,
                                                         reinterpret_cast<unsigned long long*>(ws + L.binfo), s))) !=
                     GPZ_OK)
@@ -334,11 +330,10 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         qa.nblocks = (uint32_t)nb;
         qa.F = F;
         qa.G = p->seg_bits;
-        qa.bulk_ok = vec_ok ? 1 : 0;
         qa.interleaved = interleaved ? 1 : 0;
         qa.d_params = rel ? d_params : nullptr;
         qa.bext = rel ? reinterpret_cast<const uint2*>(ws + L.bext) : nullptr;
-        qa.binfo = rel && !tile ? reinterpret_cast<const unsigned long long*>(ws + L.binfo) : nullptr;
+        qa.binfo = rel && fused ? reinterpret_cast<const unsigned long long*>(ws + L.binfo) : nullptr;
         qa.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
         qa.slot_words = slot_words_of(F);
         qa.sizes = reinterpret_cast<uint32_t*>(ws + L.sizes);
@@ -355,10 +350,10 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
             qa.deferred_count = status + 8;
         }
         if (nb > 0) {
-            const cudaError_t e = fused ? launch_qse_direct(qa, s) : tile ? launch_qse_tile(qa, s) : launch_qse(qa, s);
+            const cudaError_t e = fused ? launch_qse_direct(qa, s) : launch_qse_tile(qa, s);
             if ((rc = cuda_status(e)) != GPZ_OK) break;
             rec.mark("qse");
-            ++g_launches;  // launch_qse enqueues two kernels: the fast path and the general list
+            ++g_launches;  // two kernels: the fast path and the general list
         }
 
         uint32_t* stream_words = static_cast<uint32_t*>(d_out);

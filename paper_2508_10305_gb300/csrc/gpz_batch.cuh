@@ -37,7 +37,7 @@ struct BatchChunk {
     uint32_t range_slices;           // range items per field (relative bound), else 0
     uint32_t index;                  // position in the caller's descriptor array
     int F, G, mode;
-    int bulk_ok;                     // every field pointer 16-byte aligned
+    int aligned;                     // every field pointer 16-byte aligned
 };
 
 // chunks[] holds the groups one after another; a group is chunks
@@ -58,7 +58,8 @@ struct BatchCompressArgs {
     uint2* bext;                 // [all blocks][kMaxFields]: each block's extremes from the range items
                                  // (a chunk's blocks from block_base * kMaxFields, b * F + f), or nullptr
     int pre;                     // the group's blocks read their extremes from bext (relative bounds)
-    int tile;                    // every chunk's fields 16-byte aligned: the shared-memory tile kernel
+    int tile;                    // the shared-memory tile kernel, else the register kernel
+    int aligned;                 // every chunk's fields 16-byte aligned
     uint32_t* temp;
     uint32_t* sizes;             // [all blocks] words per block
     uint32_t* general_list;      // [the group's blocks] global block ids left to the general kernel
@@ -102,6 +103,7 @@ struct BatchDecompressArgs {
     const uint4* block_loc;      // [all blocks] as BatchMapArgs
     uint32_t block_first;        // the group's first block
     uint32_t total_blocks;       // the group's blocks
+    int aligned;                 // every chunk's fields 16-byte aligned
     uint32_t* chunk_status;      // [chunks] zeroed
 };
 
@@ -124,7 +126,10 @@ __device__ __forceinline__ uint32_t search_chunk(const uint32_t* end, uint32_t n
     return lo;
 }
 
-// Launch wrappers (gpz_batch_compress.cu, gpz_batch_decode.cu).
+// Launch wrappers (gpz_batch_compress.cu, gpz_batch_tile.cu,
+// gpz_batch_tile_unaligned.cu, gpz_batch_decode.cu).
+cudaError_t batch_tile_aligned(const BatchCompressArgs* a, int F, int grid, cudaStream_t s);
+cudaError_t batch_tile_unaligned(const BatchCompressArgs* a, int F, int grid, cudaStream_t s);
 cudaError_t launch_batch_map(const BatchMapArgs& a, cudaStream_t s);
 cudaError_t launch_batch_range(const BatchCompressArgs& a, cudaStream_t s);
 cudaError_t launch_batch_compress(const BatchCompressArgs& a, int F, cudaStream_t s);

@@ -220,9 +220,7 @@ gpz_status gpz_batch_tune(gpz_batch* p, void* d_ws, uint64_t ws_size, uint64_t* 
     // body (when a group can take the tile body), the range slice (relative
     // bounds only), then the compaction grid
     std::vector<std::vector<gpz_batch_config>> stages;
-    bool any_bulk = false;
-    for (const auto& g : c.groups) any_bulk = any_bulk || g.bulk;
-    if (c.kind == 0 && any_bulk) stages.push_back({{0, 0, 0, 1}, {0, 0, 0, 2}});
+    if (c.kind == 0) stages.push_back({{0, 0, 0, 1}, {0, 0, 0, 2}});
     if (c.kind == 0 && c.any_rel) {
         std::vector<gpz_batch_config> v;
         for (uint32_t sl : {16384u, 65536u, 262144u, 1048576u}) v.push_back({sl, 0, 0, 0});

@@ -5,56 +5,13 @@
 // look-back scan over all blocks and one compaction pass that also writes
 // every chunk's header and block table (Section 4.4, steps 2 and 3).  Each
 // chunk's stream is the one a call of its own produces.
-#include "gpz_batch.cuh"
+#include "gpz_batch_args.cuh"
 #include "gpz_qse_block.cuh"
-#include "gpz_qse_tile.cuh"
 #include "gpz_copy_block.cuh"
 
 namespace gpz {
 
 namespace {
-
-// Per-chunk argument block of the per-block code, built in shared memory by
-// the CTA's threads in parallel (d_params stays null: the constants are
-// copied in, read from L2).  Thread 64 also stores the block's index within
-// its chunk in *slot.
-__device__ __forceinline__ void load_chunk_args(const BatchCompressArgs& g, uint32_t c, uint32_t gb, QseArgs& A,
-                                                uint32_t* slot) {
-    const int t = threadIdx.x;
-    const BatchChunk* ch = g.chunks + c;
-    if (t < kMaxFields) A.fields[t] = ch->in[t];
-    if (t >= 32 && t < 32 + 4 * kMaxFields) {
-        const int f = (t - 32) >> 2, k = (t - 32) & 3;
-        const uint32_t* src = ch->mode ? reinterpret_cast<const uint32_t*>(g.rparams + (size_t)c * kMaxFields + f)
-                                       : reinterpret_cast<const uint32_t*>(ch->params + f);
-        reinterpret_cast<uint32_t*>(A.params + f)[k] = __ldcg(src + k);
-    }
-    if (t == 64) {
-        const uint32_t base = ch->block_base;
-        slot[0] = gb - base;
-        slot[1] = gb;
-        A.n = ch->n;
-        A.nblocks = ch->nblocks;
-        A.F = ch->F;
-        A.G = ch->G;
-        A.bulk_ok = ch->bulk_ok;
-        A.interleaved = 0;
-        A.d_params = nullptr;
-        A.bext = g.pre ? g.bext + (size_t)ch->block_base * kMaxFields : nullptr;
-        A.binfo = nullptr;  // the fused kernel derives the widths from the extremes
-        A.temp = g.temp + ch->temp_base;
-        A.slot_words = batch_slot_words(ch->F);
-        A.sizes = g.sizes + base;
-        A.perm = ch->perm;
-        A.status = g.chunk_status + c;
-        A.general_list = g.general_list;
-        A.general_count = g.general_count;
-        A.direct = nullptr;  // the batched form keeps the three-step compaction
-        A.direct_capacity = 0;
-        A.bstate = nullptr;
-        A.deferred_count = nullptr;
-    }
-}
 
 // One range item: minimum and maximum of one slice of one field of a
 // relative-bound chunk, merged into the chunk's order keys; the CTA that
@@ -78,35 +35,8 @@ __device__ __forceinline__ void range_item(const BatchCompressArgs& g, uint32_t 
     for (uint64_t b = b_first + warp; b < b_end; b += kWarps) {
         const float* xb = x + b * kBlock;
         const int n_b = (int)min((uint64_t)kBlock, n - b * kBlock);
-        float blo = INFINITY, bhi = -INFINITY, probe = 0.0f;
-        if (ch->bulk_ok && n_b == kBlock) {  // two rounds of four 16-byte loads per lane
-            const float4* x4 = reinterpret_cast<const float4*>(xb);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float4 v[4];
-#pragma unroll
-                for (int k = 0; k < 4; ++k) v[k] = __ldcs(x4 + lane + 32 * (4 * h + k));
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    blo = fminf(blo, fminf(fminf(v[k].x, v[k].y), fminf(v[k].z, v[k].w)));
-                    bhi = fmaxf(bhi, fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w)));
-                    probe = __fmaf_rn(v[k].x, 0.0f, probe);
-                    probe = __fmaf_rn(v[k].y, 0.0f, probe);
-                    probe = __fmaf_rn(v[k].z, 0.0f, probe);
-                    probe = __fmaf_rn(v[k].w, 0.0f, probe);
-                }
-            }
-        } else {
-            for (int i = lane; i < n_b; i += 32) {
-                const float v = __ldcs(xb + i);
-                blo = fminf(blo, v);
-                bhi = fmaxf(bhi, v);
-                probe = __fmaf_rn(v, 0.0f, probe);
-            }
-        }
-        blo = warp_min_f32(blo);
-        bhi = warp_max_f32(bhi);
-        const bool nonfinite = __any_sync(0xffffffffu, probe != probe);
+        float blo, bhi;
+        const bool nonfinite = block_extremes(xb, n_b, blo, bhi);
         if (lane == 0 && bext)
             bext[b * (uint64_t)F + f] = nonfinite ? make_uint2(0u, 0u) : make_uint2(order_key(blo), order_key(bhi));
         lo = fminf(lo, blo);
@@ -183,24 +113,6 @@ __global__ void __launch_bounds__(kThreads, 5) gpz_batch_compress_kernel(BatchCo
         qse_block_fast<F, true, SlotBlock, kCmTemp, PRE>(A, dsm, S, idx);
     else
         qse_block_fast<F, false, SlotBlock, kCmTemp, PRE>(A, dsm, S, idx);
-}
-
-// The same with the shared-memory tile body (gpz_qse_tile.cuh): groups whose
-// chunks all have 16-byte aligned fields.
-template <int F, bool PRE>
-__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_batch_tile_kernel(BatchCompressArgs g) {
-    extern __shared__ __align__(128) uint8_t dsm[];
-    __shared__ TileShared S;
-    __shared__ QseArgs A;
-    __shared__ uint32_t slot[2];  // block within its chunk, global block id
-    const uint32_t gb = g.block_first + blockIdx.x;
-    load_chunk_args(g, __ldg(g.block_map + gb), gb, A, slot);
-    __syncthreads();
-    const SlotBlock idx{slot};
-    if ((uint64_t)(idx.b() + 1) * kBlock <= A.n)
-        qse_block_tile<F, true, PRE>(A, dsm, S, idx);
-    else
-        qse_block_tile<F, false, PRE>(A, dsm, S, idx);
 }
 
 // Blocks the fast path left to the general one (rare); the grid walks the
@@ -387,26 +299,19 @@ __global__ void __launch_bounds__(32 * kCompactWarps) gpz_batch_compact_kernel(B
 
 // ------------------------------------------------------------------ launches
 
+template <class K>
+bool prepare_kernel(K kern, uint32_t smem, bool carveout) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+           (!carveout || cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100) == cudaSuccess);
+}
+
 template <int F>
 bool prepare_f() {
-    return cudaFuncSetAttribute(gpz_batch_compress_kernel<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)qse_fast_smem_bytes()) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_compress_kernel<F, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                100) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_compress_kernel<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)qse_fast_smem_bytes()) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_compress_kernel<F, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                100) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_tile_kernel<F, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem_bytes(F)) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_tile_kernel<F, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                100) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_tile_kernel<F, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)tile_smem_bytes(F)) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_tile_kernel<F, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                100) == cudaSuccess &&
-           cudaFuncSetAttribute(gpz_batch_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)qse_smem_bytes(F)) == cudaSuccess;
+    return batch_tile_aligned(nullptr, F, 0, nullptr) == cudaSuccess &&
+           batch_tile_unaligned(nullptr, F, 0, nullptr) == cudaSuccess &&
+           prepare_kernel(gpz_batch_compress_kernel<F, false>, qse_fast_smem_bytes(), true) &&
+           prepare_kernel(gpz_batch_compress_kernel<F, true>, qse_fast_smem_bytes(), true) &&
+           prepare_kernel(gpz_batch_general_kernel<F>, qse_smem_bytes(F), false);
 }
 
 bool batch_prepare_kernels(int F) {
@@ -427,10 +332,6 @@ template <int F>
 void launch_f(const BatchCompressArgs& a, int grid, cudaStream_t s, bool general) {
     if (general)
         gpz_batch_general_kernel<F><<<grid, kThreads, qse_smem_bytes(F), s>>>(a);
-    else if (a.tile && a.pre)
-        gpz_batch_tile_kernel<F, true><<<grid, kTileThreads, tile_smem_bytes(F), s>>>(a);
-    else if (a.tile)
-        gpz_batch_tile_kernel<F, false><<<grid, kTileThreads, tile_smem_bytes(F), s>>>(a);
     else if (a.pre)
         gpz_batch_compress_kernel<F, true><<<grid, kThreads, qse_fast_smem_bytes(), s>>>(a);
     else
@@ -463,7 +364,9 @@ cudaError_t launch_batch_range(const BatchCompressArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_batch_compress(const BatchCompressArgs& a, int F, cudaStream_t s) {
-    return launch_group(a, F, (int)a.total_blocks, s, false);
+    const int grid = (int)a.total_blocks;
+    if (!a.tile) return launch_group(a, F, grid, s, false);
+    return a.aligned ? batch_tile_aligned(&a, F, grid, s) : batch_tile_unaligned(&a, F, grid, s);
 }
 
 cudaError_t launch_batch_general(const BatchCompressArgs& a, int F, int grid, cudaStream_t s) {

@@ -101,10 +101,10 @@ gpz_status core_add_compress(BatchCore& c, const gpz_compress_chunk& d) {
     if (c.count() >= kMaxItems) return GPZ_ERR_UNSUPPORTED;
     BatchChunk ch;
     std::memset(&ch, 0, sizeof(ch));
-    bool vec = true;
+    ch.aligned = 1;
     for (int f = 0; f < F; ++f) {
         ch.in[f] = d.n ? d.fields[f] : nullptr;
-        vec = vec && (d.n == 0 || aligned(d.fields[f], 16));
+        if (!aligned(ch.in[f], 16)) ch.aligned = 0;
         if (q.mode == GPZ_EB_REL)
             ch.rel[f] = q.eb[f];
         else
@@ -119,7 +119,6 @@ gpz_status core_add_compress(BatchCore& c, const gpz_compress_chunk& d) {
     ch.F = F;
     ch.G = q.seg_bits;
     ch.mode = q.mode;
-    ch.bulk_ok = vec ? 1 : 0;
     c.kind = 0;
     c.any_rel = c.any_rel || q.mode == GPZ_EB_REL;
     c.chunks.push_back(ch);
@@ -136,7 +135,11 @@ gpz_status core_add_decompress(BatchCore& c, const gpz_decompress_chunk& d) {
     if (c.count() >= kMaxItems) return GPZ_ERR_UNSUPPORTED;
     BatchChunk ch;
     std::memset(&ch, 0, sizeof(ch));
-    for (int f = 0; f < F; ++f) ch.out[f] = d.n ? d.fields[f] : nullptr;
+    ch.aligned = 1;
+    for (int f = 0; f < F; ++f) {
+        ch.out[f] = d.n ? d.fields[f] : nullptr;
+        if (!aligned(ch.out[f], 16)) ch.aligned = 0;
+    }
     ch.src = static_cast<const uint32_t*>(d.in);
     ch.words = d.in_size / 4;
     ch.n = d.n;
@@ -166,14 +169,14 @@ gpz_status core_finish(BatchCore& c, const gpz_batch_config* cfg) {
             BatchGroup g{};
             g.F = ch.F;
             g.pre = pre;
-            g.bulk = 1;
+            g.aligned = 1;
             g.first = k;
             g.block_first = (uint32_t)blocks;
             c.groups.push_back(g);
         }
         BatchGroup& g = c.groups.back();
         ++g.count;
-        g.bulk = g.bulk && ch.bulk_ok;
+        g.aligned = g.aligned && ch.aligned;
         ch.block_base = (uint32_t)blocks;
         ch.temp_base = temp;
         blocks += ch.nblocks;
@@ -279,6 +282,7 @@ gpz_status core_enqueue(const BatchCore& c, const BatchDevice& dev, uint8_t* ws,
             a.block_loc = reinterpret_cast<const uint4*>(ws + L.loc);
             a.block_first = g.block_first;
             a.total_blocks = g.blocks;
+            a.aligned = g.aligned;
             a.chunk_status = status;
             if (launch_batch_decompress(a, g.F, s) != cudaSuccess) return GPZ_ERR_CUDA;
             rec.mark("batch_decompress");
@@ -308,7 +312,8 @@ gpz_status core_enqueue(const BatchCore& c, const BatchDevice& dev, uint8_t* ws,
         a.general_list = reinterpret_cast<uint32_t*>(ws + L.list) + g.block_first;
         a.general_count = ctrl + k;
         a.pre = g.pre && a.bext != nullptr;
-        a.tile = g.bulk && cfg.qse_form == 1;
+        a.tile = cfg.qse_form == 1;
+        a.aligned = g.aligned;
         if (g.range_items > 0) {
             if (launch_batch_range(a, s) != cudaSuccess) return GPZ_ERR_CUDA;
             rec.mark("batch_range");

@@ -12,7 +12,7 @@ namespace gpz {
 // One CTA per block of the group.  The map kernel has gathered every
 // block's table entries (block_loc), so a CTA needs one round trip for its
 // chunk and its place, and one for its words.
-template <int F>
+template <int F, int OUT>
 __global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_batch_decompress_kernel(BatchDecompressArgs g) {
     __shared__ DecShared<F> S;
     __shared__ DecArgs A;
@@ -37,23 +37,28 @@ __global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_batch_decompress
         s_b = gb - ch->block_base;
     }
     __syncthreads();
-    decode_block<F, DecSlotBlock, false, false, DecShared<F>, true>(A, S, DecSlotBlock{&s_b}, hw_pre);
+    decode_block<F, OUT, true>(A, S, DecSlotBlock{&s_b}, hw_pre);
 }
 
-cudaError_t launch_batch_decompress(const BatchDecompressArgs& a, int F, cudaStream_t s) {
+template <int OUT>
+cudaError_t launch_batch_decompress_out(const BatchDecompressArgs& a, int F, cudaStream_t s) {
     const unsigned grid = a.total_blocks;
     switch (F) {
-        case 1: gpz_batch_decompress_kernel<1><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 2: gpz_batch_decompress_kernel<2><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 3: gpz_batch_decompress_kernel<3><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 4: gpz_batch_decompress_kernel<4><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 5: gpz_batch_decompress_kernel<5><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 6: gpz_batch_decompress_kernel<6><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 7: gpz_batch_decompress_kernel<7><<<grid, kDecThreads, 0, s>>>(a); break;
-        case 8: gpz_batch_decompress_kernel<8><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 1: gpz_batch_decompress_kernel<1, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 2: gpz_batch_decompress_kernel<2, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 3: gpz_batch_decompress_kernel<3, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 4: gpz_batch_decompress_kernel<4, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 5: gpz_batch_decompress_kernel<5, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 6: gpz_batch_decompress_kernel<6, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 7: gpz_batch_decompress_kernel<7, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
+        case 8: gpz_batch_decompress_kernel<8, OUT><<<grid, kDecThreads, 0, s>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+
+cudaError_t launch_batch_decompress(const BatchDecompressArgs& a, int F, cudaStream_t s) {
+    return a.aligned ? launch_batch_decompress_out<kOut32>(a, F, s) : launch_batch_decompress_out<kOutAny>(a, F, s);
 }
 
 }  // namespace gpz

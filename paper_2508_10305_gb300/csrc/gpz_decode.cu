@@ -29,57 +29,46 @@
 
 namespace gpz {
 
-template <int F>
+template <int F, int OUT>
 __global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_decompress_kernel(DecArgs a) {
     __shared__ DecShared<F> S;
-    decode_block<F>(a, S, DecGridBlock{});
+    decode_block<F, OUT, false>(a, S, DecGridBlock{});
 }
 
-template <int F>
-cudaError_t launch_dec_f(const DecArgs& a, cudaStream_t s) {
-    gpz_decompress_kernel<F><<<a.nblocks, kDecThreads, 0, s>>>(a);
+template <int OUT>
+cudaError_t launch_decompress_out(const DecArgs& a, cudaStream_t s) {
+    if (a.nblocks == 0) return cudaSuccess;
+    switch (a.F) {
+        case 1: gpz_decompress_kernel<1, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 2: gpz_decompress_kernel<2, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 3: gpz_decompress_kernel<3, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 4: gpz_decompress_kernel<4, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 5: gpz_decompress_kernel<5, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 6: gpz_decompress_kernel<6, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 7: gpz_decompress_kernel<7, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 8: gpz_decompress_kernel<8, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
+}
+
+static bool all_aligned(const DecArgs& a) {
+    for (int f = 0; f < a.F; ++f)
+        if (reinterpret_cast<uintptr_t>(a.out[f]) & 15u) return false;
+    return true;
 }
 
 cudaError_t launch_decompress(const DecArgs& a, cudaStream_t s) {
     if (a.nblocks == 0) return cudaSuccess;
     if (a.interleaved) return launch_decompress_aos(a, s);  // gpz_aos.cu
-    switch (a.F) {
-        case 1: return launch_dec_f<1>(a, s);
-        case 2: return launch_dec_f<2>(a, s);
-        case 3: return launch_dec_f<3>(a, s);
-        case 4: return launch_dec_f<4>(a, s);
-        case 5: return launch_dec_f<5>(a, s);
-        case 6: return launch_dec_f<6>(a, s);
-        case 7: return launch_dec_f<7>(a, s);
-        case 8: return launch_dec_f<8>(a, s);
-    }
-    return cudaErrorInvalidValue;
+    return all_aligned(a) ? launch_decompress_out<kOut32>(a, s) : launch_decompress_out<kOutAny>(a, s);
 }
 
 // The same decoder storing fp64 (gpz_decompress_f64 on a version-1 stream):
 // a.out[f] holds the address of field f's double array, and every value is
 // the fp32 reconstruction widened exactly.
-template <int F>
-__global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_decompress64_kernel(DecArgs a) {
-    __shared__ DecShared<F> S;
-    decode_block<F, DecGridBlock, true>(a, S, DecGridBlock{});
-}
-
 cudaError_t launch_decompress64(const DecArgs& a, cudaStream_t s) {
-    if (a.nblocks == 0) return cudaSuccess;
-    switch (a.F) {
-        case 1: gpz_decompress64_kernel<1><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 2: gpz_decompress64_kernel<2><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 3: gpz_decompress64_kernel<3><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 4: gpz_decompress64_kernel<4><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 5: gpz_decompress64_kernel<5><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 6: gpz_decompress64_kernel<6><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 7: gpz_decompress64_kernel<7><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 8: gpz_decompress64_kernel<8><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    return all_aligned(a) ? launch_decompress_out<kOut64>(a, s) : launch_decompress_out<kOutAny64>(a, s);
 }
 
 }  // namespace gpz

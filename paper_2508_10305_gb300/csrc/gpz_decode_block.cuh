@@ -79,19 +79,11 @@ __device__ __forceinline__ void store4(float* out, uint64_t first, const float* 
 
 // Interleaved output: a block's values in record order in shared memory,
 // value (j, f) at word j * F + f + j / 8 (the padding word every eight
-// records spreads a warp's four-apart records over the banks).
+// records spreads the records of a warp over the banks when F is even).
 template <int F>
 __device__ __forceinline__ int rec_slot(int j, int f) { return j * F + f + (j >> 3); }
 template <int F>
 constexpr uint32_t rec_words() { return (uint32_t)(kBlock * F + kBlock / 8); }
-
-// store4's values, for records j .. j + 3 of field f, into that staging.
-template <int F>
-__device__ __forceinline__ void store4_rec(float* recs, int j, int f, const float* v, int left) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        if (e < left) recs[rec_slot<F>(j + e, f)] = v[e];
-}
 
 // x = fma((float)q, step, min) of four codes.
 __device__ __forceinline__ void rebuild4(const uint32_t* q, uint32_t bits, float s, float mn, float* v) {
@@ -99,19 +91,56 @@ __device__ __forceinline__ void rebuild4(const uint32_t* q, uint32_t bits, float
     for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(bits <= 23u ? small_u2f(q[e]) : __uint2float_rn(q[e]), s, mn);
 }
 
+// Where a block's values go: fp32 fields or fp64 fields, 16-byte aligned or of
+// any alignment, or interleaved fp32 records.
+enum : int { kOut32, kOutAny, kOut64, kOutAny64, kOutRecords };
+
+// The positions a thread rebuilds, in groups of four: four consecutive ones,
+// stored with 16-byte stores, into aligned fields; otherwise one of each run
+// of kDecThreads, so that a warp's 4-byte (8-byte) stores, or its words in the
+// record stage, are consecutive.  (Into odd rows of a
+// 10^7 x 6 snapshot: 53 us; with 4-byte stores of four consecutive positions
+// per lane 55, with 16-byte units completed by shuffles from the next lane
+// 68; aligned rows 50.)
+__host__ __device__ constexpr bool out_strided(int out) { return out != kOut32 && out != kOut64; }
+template <int OUT>
+__device__ __forceinline__ int out_pos(int g, int e) {
+    const int t = threadIdx.x;
+    return out_strided(OUT) ? t + kDecThreads * (4 * g + e) : 4 * (t + kDecThreads * g) + e;
+}
+
+// The values of group g's positions of field f, in the block starting at
+// particle `base`, those below n_b.
+template <int F, int OUT>
+__device__ __forceinline__ void store_group(const DecArgs& a, int f, int g, const float* v, uint64_t base, int n_b,
+                                            float* recs) {
+    if (!out_strided(OUT)) {
+        const int j = out_pos<OUT>(g, 0);
+        store4<OUT == kOut64>(a.out[f], base + j, v, n_b - j);
+        return;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int j = out_pos<OUT>(g, e);
+        if (j >= n_b) continue;
+        if (OUT == kOutRecords)
+            recs[rec_slot<F>(j, f)] = v[e];
+        else if (OUT == kOutAny64)
+            __stcs(reinterpret_cast<double*>(a.out[f]) + base + j, (double)v[e]);
+        else
+            __stcs(a.out[f] + base + j, v[e]);
+    }
+}
+
 // Records wider than 128 bits (rare): every code is read field by field from
 // the stream itself; the block header is re-read here so that the common path
 // passes nothing through memory.
-template <int F, bool OUT64 = false, bool AOS = false>
+template <int F, int OUT>
 __device__ __forceinline__ void decode_wide(const DecArgs& a, const uint32_t* blk, uint32_t rwords_off,
-                                         uint32_t rwords, uint32_t W, uint32_t G, int j0, int n_b, uint64_t first,
-                                         uint32_t key0, uint32_t key1, uint32_t key2, uint32_t key3,
-                                         float* recs = nullptr) {
+                                            uint32_t rwords, uint32_t W, uint32_t G, int grp, int n_b, uint64_t base,
+                                            const uint32_t (&key)[4], float* recs) {
     constexpr int P = F < 3 ? F : 3;
     const uint32_t* R = blk + rwords_off;
-    const uint32_t key[4] = {key0, key1, key2, key3};
-    uint32_t rs = W;
-    uint32_t ks = 0;
     // walk the fields from the top of the record down: field 0 is most significant
     uint32_t kacc[F], racc[F], wfv[F], gv[F];
     {
@@ -127,8 +156,6 @@ __device__ __forceinline__ void decode_wide(const DecArgs& a, const uint32_t* bl
             k += g;
         }
     }
-    (void)rs;
-    (void)ks;
     for (int f = 0; f < F; ++f) {
         const uint32_t bf = (__ldg(blk + 1 + F + (f >> 2)) >> (8 * (f & 3))) & 0xffu;
         const float mnf = __uint_as_float(__ldg(blk + 1 + f));
@@ -137,8 +164,9 @@ __device__ __forceinline__ void decode_wide(const DecArgs& a, const uint32_t* bl
         uint32_t qv[4];
         for (int e = 0; e < 4; ++e) {
             uint32_t code = 0u;
-            if (cm && j0 + e < n_b) {
-                const uint32_t p = (uint32_t)(j0 + e) * W + racc[f];
+            const int j = out_pos<OUT>(grp, e);
+            if (cm && j < n_b) {
+                const uint32_t p = (uint32_t)j * W + racc[f];
                 const uint32_t wi = p >> 5, sh = p & 31u;
                 const uint32_t lo = __ldg(R + wi);
                 const uint32_t hi = (sh + wfv[f] > 32u) && (wi + 1 < rwords) ? __ldg(R + wi + 1) : 0u;
@@ -148,10 +176,7 @@ __device__ __forceinline__ void decode_wide(const DecArgs& a, const uint32_t* bl
         }
         float v[4];
         rebuild4(qv, bf, sf, mnf, v);
-        if (AOS)
-            store4_rec<F>(recs, j0, f, v, n_b - j0);
-        else
-            store4<OUT64>(a.out[f], first + j0, v, n_b - j0);
+        store_group<F, OUT>(a, f, grp, v, base, n_b, recs);
     }
 }
 
@@ -186,7 +211,7 @@ struct DecSharedRec : DecCore {
     alignas(16) uint32_t stage[cmax(kWords + kDecStagePad + 4, 4 + rec_words<F>())];
 };
 
-// NG groups of four positions (j[g] .. j[g] + 3, keys key[g]): their records
+// Groups g0 .. g0 + NG - 1 of four positions (keys key[g - g0]): their records
 // from the staged words, then the codes of fields F-1 .. 0, consumed from the
 // least significant end: field F-1 sits at bit 0 of the record and field 0 at
 // the top.  rr holds a record in its low bits (two words when W <= 64, else
@@ -194,10 +219,11 @@ struct DecSharedRec : DecCore {
 // and the key right by the axis' segId bits.  q = segId * 2^o + segOffset for
 // a position axis, the whole code otherwise.  Words past the record array
 // (inside the staging pad) hold bits above W, which are never consumed.
-// AOS: sync() once every record is in registers, then the values go to recs.
-template <int F, int NG, bool WIDE, bool OUT64, bool AOS, class Sync>
+// kOutRecords: sync() once every record is in registers, then the values go to
+// recs.
+template <int F, int NG, bool WIDE, int OUT, class Sync>
 __device__ __forceinline__ void decode_groups(const DecArgs& a, const DecCore& L, const uint32_t* sR, uint32_t W,
-                                              const int (&j)[NG], uint32_t (&key)[NG][4], uint64_t base, int n_b,
+                                              int g0, uint32_t (&key)[NG][4], uint64_t base, int n_b,
                                               float* recs, Sync sync) {
     constexpr int P = F < 3 ? F : 3;
     constexpr int NR = WIDE ? 4 : 2;
@@ -206,7 +232,7 @@ __device__ __forceinline__ void decode_groups(const DecArgs& a, const DecCore& L
     for (int g = 0; g < NG; ++g)
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const uint32_t p = (uint32_t)(j[g] + e) * W;
+            const uint32_t p = (uint32_t)out_pos<OUT>(g0 + g, e) * W;
             const uint32_t* at = sR + (p >> 5);
             uint32_t x = at[0];
 #pragma unroll
@@ -253,12 +279,7 @@ __device__ __forceinline__ void decode_groups(const DecArgs& a, const DecCore& L
                 for (int e = 0; e < 4; ++e) v[g][e] = __fmaf_rn(__uint2float_rn(__float_as_uint(v[g][e])), ms.y, ms.x);
         }
 #pragma unroll
-        for (int g = 0; g < NG; ++g) {
-            if (AOS)
-                store4_rec<F>(recs, j[g], f, v[g], n_b - j[g]);
-            else
-                store4<OUT64>(a.out[f], base + j[g], v[g], n_b - j[g]);
-        }
+        for (int g = 0; g < NG; ++g) store_group<F, OUT>(a, f, g0 + g, v[g], base, n_b, recs);
     }
 }
 
@@ -378,11 +399,12 @@ __device__ __forceinline__ void store_records(const DecArgs& a, const float* rec
     }
 }
 
-// AOS: the values go to interleaved records at out[0]; `stage` must then
+// kOutRecords: the values go to interleaved records at out[0]; `stage` must then
 // hold rec_words<F>() words.
-template <int F, bool OUT64 = false, bool AOS = false>
+template <int F, int OUT>
 __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32_t* stage,
                                             const uint32_t* blk, uint32_t b, int n_b) {
+    constexpr bool OUT64 = OUT == kOut64 || OUT == kOutAny64, AOS = OUT == kOutRecords;
     uint16_t* uniq = S.uniq;
     uint32_t* mask = S.mask;
     uint32_t& s_bad = S.bad;
@@ -487,9 +509,9 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
 
     // ---- 4. the run of position j is the number of run starts up to j, less
     // one: every warp scans the 32 mask words itself (no further barrier; lane
-    // i holds word i and the starts before it); a group's four positions lie in
-    // one word, and position 0 starts a run, so every index is in 0..U-1
-    int j[kDecGroups];
+    // i holds word i and the starts before it).  Consecutive positions of a
+    // group lie in one word; strided ones in one word per warp.  Position 0
+    // starts a run, so every index is in 0..U-1.
     uint32_t key[kDecGroups][4];
     {
         const uint32_t mw = mask[lane];
@@ -497,14 +519,22 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
         const uint32_t pre = warp_incl_sum(pc) - pc;
 #pragma unroll
         for (int g = 0; g < kDecGroups; ++g) {
-            j[g] = 4 * (t + g * kDecThreads);
-            const uint32_t m = __shfl_sync(0xffffffffu, mw, j[g] >> 5) >> (j[g] & 31);
-            const uint32_t before = __shfl_sync(0xffffffffu, mw, j[g] >> 5) & ((1u << (j[g] & 31)) - 1u);
-            uint32_t run = __shfl_sync(0xffffffffu, pre, j[g] >> 5) + __popc(before) - 1u;
+            if (out_strided(OUT)) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                run += (m >> e) & 1u;
-                key[g][e] = uniq[run];
+                for (int e = 0; e < 4; ++e) {
+                    const int word = out_pos<OUT>(g, e) >> 5;  // the same for the whole warp
+                    const uint32_t m = __shfl_sync(0xffffffffu, mw, word) & lanemask_le();
+                    key[g][e] = uniq[__shfl_sync(0xffffffffu, pre, word) + __popc(m) - 1u];
+                }
+            } else {
+                const int j = out_pos<OUT>(g, 0);
+                const uint32_t word = __shfl_sync(0xffffffffu, mw, j >> 5);
+                uint32_t run = __shfl_sync(0xffffffffu, pre, j >> 5) + __popc(word & ((1u << (j & 31)) - 1u)) - 1u;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    run += (word >> ((j & 31) + e)) & 1u;
+                    key[g][e] = uniq[run];
+                }
             }
         }
     }
@@ -517,32 +547,29 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
         sync();  // the staged deltas and counts are consumed
 #pragma unroll
         for (int g = 0; g < kDecGroups; ++g)
-            if (j[g] < n_b)
-                decode_wide<F, OUT64, AOS>(a, blk, hdr + dwords + cwords, rwords, W, S.G, j[g], n_b, base, key[g][0],
-                                           key[g][1], key[g][2], key[g][3], recs);
+            decode_wide<F, OUT>(a, blk, hdr + dwords + cwords, rwords, W, S.G, g, n_b, base, key[g], recs);
     } else if (W <= 64u) {
-        decode_groups<F, kDecGroups, false, OUT64, AOS>(a, S, sR, W, j, key, base, n_b, recs, sync);
+        decode_groups<F, kDecGroups, false, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
     } else if (AOS) {  // every record in registers before the first value is staged
-        decode_groups<F, kDecGroups, true, OUT64, AOS>(a, S, sR, W, j, key, base, n_b, recs, sync);
+        decode_groups<F, kDecGroups, true, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
     } else {
 #pragma unroll 1
         for (int g = 0; g < kDecGroups; ++g) {
-            const int jg[1] = {g == 0 ? j[0] : j[kDecGroups - 1]};
             uint32_t kg[1][4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) kg[0][e] = g == 0 ? key[0][e] : key[kDecGroups - 1][e];
-            decode_groups<F, 1, true, OUT64, AOS>(a, S, sR, W, jg, kg, base, n_b, recs, sync);
+            decode_groups<F, 1, true, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
         }
     }
     if (AOS) store_records<F>(a, recs, b, n_b);
 }
 
 
-// AOS: out[0] receives interleaved records of F fields (Sh then a
+// kOutRecords: out[0] receives interleaved records of F fields (Sh then a
 // DecSharedRec<F>).  PREHW: lanes 0, 1, 2 of every warp pass in hw_pre the
 // words round trip 1 would load (the payload size and the block's two table
 // entries), loaded earlier by the caller.
-template <int F, class Idx, bool OUT64 = false, bool AOS = false, class Sh = DecShared<F>, bool PREHW = false>
+template <int F, int OUT, bool PREHW, class Sh, class Idx>
 __device__ __forceinline__ void decode_block(const DecArgs& a, Sh& S, Idx idx, uint32_t hw_pre = 0u) {
     uint32_t* stage = S.stage;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -606,7 +633,7 @@ __device__ __forceinline__ void decode_block(const DecArgs& a, Sh& S, Idx idx, u
     if (w == 0) decode_checks<F>(a, S, hv, bw, step, inside, b, off, end, payload_words, n_b);
     __syncthreads();
     if (units && !__syncthreads_and(mbar_wait_bounded(&S.bar, 0, a.status))) return;  // uniform
-    decode_tail<F, OUT64, AOS>(a, S, stage + shift, blk, b, n_b);
+    decode_tail<F, OUT>(a, S, stage + shift, blk, b, n_b);
 }
 
 }  // namespace gpz

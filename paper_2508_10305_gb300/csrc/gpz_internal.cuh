@@ -48,7 +48,6 @@ struct RangeArgs {
     const float* fields[kMaxFields];
     uint64_t n;
     int F;
-    int vec_ok;                 // every field pointer 16-byte aligned
     double rel[kMaxFields];
     float2* partials;           // [gridDim.x][F] (min, max)
     uint32_t* done_counter;
@@ -62,7 +61,6 @@ struct QseArgs {
     uint32_t nblocks;
     int F;
     int G;
-    int bulk_ok;                // every field pointer 16-byte aligned: stage tiles with bulk copies
     int interleaved;            // fields[0] holds F-field records: field f of particle i at fields[0][i * F + f]
     FieldParams params[kMaxFields];
     const FieldParams* d_params; // device constants (relative bound) or nullptr
@@ -359,11 +357,10 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
 // ---------------------------------------------------------------- launch wrappers (defined in the .cu files)
 
 cudaError_t launch_range(const RangeArgs& a, int grid, cudaStream_t s);
-cudaError_t launch_qse(const QseArgs& a, cudaStream_t s);         // fast kernel, then the general list
-cudaError_t launch_qse_direct(const QseArgs& a, cudaStream_t s);  // the same with blocks placed directly
+cudaError_t launch_qse_direct(const QseArgs& a, cudaStream_t s);  // register kernel placing blocks directly, then the general list
 cudaError_t launch_qse_general(const QseArgs& a, cudaStream_t s);
-cudaError_t launch_qse_pre(const QseArgs& a, cudaStream_t s);     // fast kernel reading a.bext
-cudaError_t launch_qse_tile(const QseArgs& a, cudaStream_t s);    // shared-memory tile kernel (16-byte aligned fields)
+cudaError_t launch_qse_tile(const QseArgs& a, cudaStream_t s);    // shared-memory tile kernel, then the general list
+cudaError_t launch_qse_tile_unaligned(const QseArgs& a, cudaStream_t s);  // the same on 4-byte aligned fields
 cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s); // the same on interleaved records (16-byte aligned)
 cudaError_t launch_decompress_aos(const DecArgs& a, cudaStream_t s); // decompression into interleaved records
 cudaError_t launch_block_info(const uint2* bext, const FieldParams* d_params, uint32_t nblocks, int F,

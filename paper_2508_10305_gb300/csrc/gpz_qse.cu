@@ -1,40 +1,16 @@
-// gpz_qse.cu -- the fused per-block compression kernel (stages 1-3 of GPZ:
-// quantisation, sorting, encoding; Sections 4.1-4.3, the "Q.S.E." kernel of
-// Table 1) and the global range pass of the relative error bound.
-//
-// One CTA of 256 threads owns one block of 1024 particles; every thread
-// holds 4 particles of every field in registers (no shared-memory tile).
-// Thread (warp w, lane l) owns elements 128w + 32r + l, r = 0..3, so that each
-// warp covers 128 consecutive particles in storage order.  Per CTA:
-//   1. coalesced streaming loads; per-field exact fp32 minimum (Section 4.1:
-//      per-thread, then warp reduction, then a shared atomic per warp), or,
-//      with a relative bound, the block's extremes the range pass already
-//      found (gpz_qse_pre.cu);
-//   2. quantisation q = floor(fma(x - min, 1/s, 1/2)) with the stream
-//      format's fp32 verification (skipped for blocks where it provably
-//      passes); blocks that need a fallback candidate, codes >= 2^23 or
-//      records wider than 128 bits go to the general kernel; for codes below
-//      2^23 the floor and the int<->float conversions are one add in
-//      round-down mode against 2^23 (full-rate pipes);
-//   3. segId / segOffset by shift and mask (Section 5.1), the linearised
-//      segId (key) and the per-particle record of offsets and extra-field
-//      codes;
-//   4. stable counting sort by key (Section 4.2): each warp ranks its 128
-//      elements in storage order with __match_any_sync into a per-warp
-//      histogram; a CTA-wide scan over (bin, warp) gives every element its
-//      sorted position.  The non-empty bins are the run-length code (unique
-//      ids and counts, Section 4.3);
-//   5. fixed-length coding (Section 4.3) into staging words cleared at the
-//      start: the deltas and counts by thread-serial bit appenders, each
-//      record ORed in by its own thread at its sorted position; the encoded
-//      block is copied out with 16-byte stores;
-//   6. the block goes to its temporary slot with its word count (step 1 of
-//      the three-step compaction, Section 4.4).
+// gpz_qse.cu -- the global range pass of the relative error bound, and the
+// general compression kernel for the rare blocks that the fused kernels leave
+// (codes >= 2^23, records wider than 128 bits, a fallback candidate that
+// changes a field's width; Sections 4.1-4.3 in gpz_qse_block.cuh).
 #include "gpz_qse_block.cuh"
 
 namespace gpz {
 
 // ------------------------------------------------------------------ range pass (relative bound)
+//
+// Bound by HBM: 1.61 GB of a 2^26 x 6 snapshot in 0.262 ms (6.2 TB/s).  Fields
+// of any alignment are read with 16-byte loads: a 10^7 x 6 snapshot with odd
+// rows 62 -> 56 us (55 aligned).
 
 // One warp per (block, field) item, field-major, so that consecutive warps
 // stream consecutive blocks of a field.  Each item yields the block's
@@ -58,34 +34,8 @@ __global__ void __launch_bounds__(kRangeThreads, 8) gpz_range_kernel(RangeArgs a
         const uint64_t b = it - (uint64_t)f * nb;
         const float* x = a.fields[f] + b * kBlock;
         const int n_b = (int)min((uint64_t)kBlock, a.n - b * kBlock);
-        float lo = INFINITY, hi = -INFINITY, probe = 0.0f;  // probe: NaN if any value is NaN or infinite
-        if (a.vec_ok && n_b == kBlock) {  // 256 16-byte words: all eight of a lane in flight at once
-            const float4* x4 = reinterpret_cast<const float4*>(x);
-            float4 v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = __ldcs(x4 + lane + 32 * k);
-            {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    lo = fminf(lo, fminf(fminf(v[k].x, v[k].y), fminf(v[k].z, v[k].w)));
-                    hi = fmaxf(hi, fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w)));
-                    probe = __fmaf_rn(v[k].x, 0.0f, probe);
-                    probe = __fmaf_rn(v[k].y, 0.0f, probe);
-                    probe = __fmaf_rn(v[k].z, 0.0f, probe);
-                    probe = __fmaf_rn(v[k].w, 0.0f, probe);
-                }
-            }
-        } else {
-            for (int i = lane; i < n_b; i += 32) {
-                const float v = __ldcs(x + i);
-                lo = fminf(lo, v);
-                hi = fmaxf(hi, v);
-                probe = __fmaf_rn(v, 0.0f, probe);
-            }
-        }
-        lo = warp_min_f32(lo);
-        hi = warp_max_f32(hi);
-        const bool nonfinite = __any_sync(0xffffffffu, probe != probe);
+        float lo, hi;
+        const bool nonfinite = block_extremes(x, n_b, lo, hi);
         if (lane == 0) {
             a.bext[b * (uint64_t)a.F + f] = nonfinite ? make_uint2(0u, 0u) : make_uint2(order_key(lo), order_key(hi));
             if (lo <= hi) {  // some value is not NaN
@@ -159,29 +109,6 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_qse_general_kernel(QseArgs a)
     }
 }
 
-template <int F>
-__global__ void __launch_bounds__(kThreads, 5) gpz_qse_kernel(QseArgs a) {
-    extern __shared__ __align__(16) uint8_t dsm[];
-    __shared__ QseFastShared S;
-    if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
-        qse_block_fast<F, true>(a, dsm, S, GridBlock{});
-    else
-        qse_block_fast<F, false>(a, dsm, S, GridBlock{});
-}
-
-template <int F>
-cudaError_t launch_qse_f(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = qse_fast_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(gpz_qse_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gpz_qse_kernel<F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    gpz_qse_kernel<F><<<a.nblocks, kThreads, smem, s>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_qse_general(a, s);
-}
-
 // the blocks left to the general path (usually none); the grid walks the list
 template <int F>
 cudaError_t launch_qse_general_f(const QseArgs& a, cudaStream_t s) {
@@ -192,22 +119,6 @@ cudaError_t launch_qse_general_f(const QseArgs& a, cudaStream_t s) {
     const unsigned ggrid = a.nblocks < 2u * 152u ? a.nblocks : 2u * 152u;
     gpz_qse_general_kernel<F><<<ggrid, kThreads, gsmem, s>>>(a);
     return cudaGetLastError();
-}
-
-cudaError_t launch_qse(const QseArgs& a, cudaStream_t s) {
-    if (a.nblocks == 0) return cudaSuccess;
-    if (a.bext) return launch_qse_pre(a, s);
-    switch (a.F) {
-        case 1: return launch_qse_f<1>(a, s);
-        case 2: return launch_qse_f<2>(a, s);
-        case 3: return launch_qse_f<3>(a, s);
-        case 4: return launch_qse_f<4>(a, s);
-        case 5: return launch_qse_f<5>(a, s);
-        case 6: return launch_qse_f<6>(a, s);
-        case 7: return launch_qse_f<7>(a, s);
-        case 8: return launch_qse_f<8>(a, s);
-    }
-    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_qse_general(const QseArgs& a, cudaStream_t s) {

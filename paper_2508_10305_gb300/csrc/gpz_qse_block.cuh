@@ -1,7 +1,11 @@
-// gpz_qse_block.cuh -- the per-block body of the fused compression kernel
-// (quantisation, sorting, encoding; Sections 4.1-4.3), shared by the
-// single-array kernels (gpz_qse.cu) and the batched kernels
-// (gpz_batch_compress.cu).  See gpz_qse.cu for the design.
+// gpz_qse_block.cuh -- per-block code of compression (quantisation, sorting,
+// encoding; Sections 4.1-4.3): the general path (gpz_qse.cu,
+// gpz_batch_compress.cu) and the register form of the fast path, which serves
+// the fused compaction (gpz_qse_direct.cu) and is a launch shape of batched
+// plans (gpz_batch_compress.cu).  In the register form one CTA of 256 threads
+// owns a block and every thread holds 4 particles of every field in
+// registers; the tile form (gpz_qse_tile.cuh) is the one that single calls and
+// batched plans run by default.
 #pragma once
 
 #include "gpz_internal.cuh"
@@ -60,6 +64,53 @@ __device__ __forceinline__ uint32_t order_key(float x) {
 }
 __device__ __forceinline__ float from_order_key(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+}
+
+// The extremes of one block's n_b values of a field over its non-NaN values
+// (lo > hi when there are none), and whether a value is NaN or infinite (one
+// warp; every lane returns the same).  A whole block is read as 16-byte words,
+// eight in flight per lane, from the first boundary on -- the words before
+// it and after the last one (four in all, when the field is not aligned) by
+// one 4-byte load.
+__device__ __forceinline__ bool block_extremes(const float* x, int n_b, float& lo, float& hi) {
+    const int lane = threadIdx.x & 31;
+    lo = INFINITY;
+    hi = -INFINITY;
+    float probe = 0.0f;  // becomes NaN if a value is NaN or infinite (x * 0)
+    if (n_b == kBlock) {
+        const int head = (int)((0u - (uint32_t)(reinterpret_cast<uintptr_t>(x) >> 2)) & 3u);  // words before the boundary
+        const float4* x4 = reinterpret_cast<const float4*>(x + head);
+        float4 v[8];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) v[k] = __ldcs(x4 + lane + 32 * k);
+        // an unaligned field has 255 words; the last lane reads its own again
+        v[7] = __ldcs(x4 + lane + 32 * (head && lane == 31 ? 6 : 7));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            lo = fminf(lo, fminf(fminf(v[k].x, v[k].y), fminf(v[k].z, v[k].w)));
+            hi = fmaxf(hi, fmaxf(fmaxf(v[k].x, v[k].y), fmaxf(v[k].z, v[k].w)));
+            probe = __fmaf_rn(v[k].x, 0.0f, probe);
+            probe = __fmaf_rn(v[k].y, 0.0f, probe);
+            probe = __fmaf_rn(v[k].z, 0.0f, probe);
+            probe = __fmaf_rn(v[k].w, 0.0f, probe);
+        }
+        if (head) {
+            const float e = __ldcs(x + ((lane & 3) < head ? lane & 3 : kBlock - 4 + (lane & 3)));
+            lo = fminf(lo, e);
+            hi = fmaxf(hi, e);
+            probe = __fmaf_rn(e, 0.0f, probe);
+        }
+    } else {
+        for (int i = lane; i < n_b; i += 32) {
+            const float v = __ldcs(x + i);
+            lo = fminf(lo, v);
+            hi = fmaxf(hi, v);
+            probe = __fmaf_rn(v, 0.0f, probe);
+        }
+    }
+    lo = warp_min_f32(lo);
+    hi = warp_max_f32(hi);
+    return __any_sync(0xffffffffu, probe != probe);
 }
 
 // Verification of one candidate code: the decompressor's reconstruction.

@@ -1,6 +1,5 @@
 // gpz_qse_tile.cu -- the fused compression kernel (quantisation, sorting,
-// encoding; Sections 4.1-4.3) of single-array calls whose fields are 16-byte
-// aligned, with the block's input in shared memory instead of registers.
+// encoding; Sections 4.1-4.3) of single-array calls, with the block's input in shared memory instead of registers.
 //
 // One CTA of 128 threads owns one block of 1024 particles, eight per thread:
 //   - lane f of warp 0 loads field f's 1024 values into a shared tile with one
@@ -48,52 +47,17 @@
 // its field's width, or none that passes, a code >= 2^23, a record > 128 bits) go to the general kernel's list; blocks
 // with a non-finite value or no gain are stored raw -- both exactly as in
 // gpz_qse_block.cuh.
-#include "gpz_qse_tile.cuh"
+#include "gpz_qse_tile_launch.cuh"
 
 namespace gpz {
 
-template <int F, bool PRE>
-__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
-    extern __shared__ __align__(128) uint8_t dsm[];
-    __shared__ TileShared S;
-    if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
-        qse_block_tile<F, true, PRE>(a, dsm, S, GridBlock{});
-    else
-        qse_block_tile<F, false, PRE>(a, dsm, S, GridBlock{});
-}
-
-template <int F, bool PRE>
-cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
-    const size_t smem = tile_smem_bytes(F);
-    auto kern = gpz_qse_tile_kernel<F, PRE>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_qse_general(a, s);
-}
-
+// Fields that are all 16-byte aligned take the kernel without shifts.
 cudaError_t launch_qse_tile(const QseArgs& a, cudaStream_t s) {
     if (a.nblocks == 0) return cudaSuccess;
-    if (!a.bulk_ok) return cudaErrorInvalidValue;
     if (a.interleaved) return launch_qse_tile_aos(a, s);  // gpz_aos.cu
-    const bool pre = a.bext != nullptr;
-    switch (a.F) {
-#define GPZ_CASE(FF) \
-    case FF: return pre ? launch_qse_tile_fp<FF, true>(a, s) : launch_qse_tile_fp<FF, false>(a, s);
-        GPZ_CASE(1)
-        GPZ_CASE(2)
-        GPZ_CASE(3)
-        GPZ_CASE(4)
-        GPZ_CASE(5)
-        GPZ_CASE(6)
-        GPZ_CASE(7)
-        GPZ_CASE(8)
-#undef GPZ_CASE
-    }
-    return cudaErrorInvalidValue;
+    for (int f = 0; f < a.F; ++f)
+        if (reinterpret_cast<uintptr_t>(a.fields[f]) & 15u) return launch_qse_tile_unaligned(a, s);
+    return launch_qse_tile_layout<kTileAligned>(a, s);
 }
 
 }  // namespace gpz

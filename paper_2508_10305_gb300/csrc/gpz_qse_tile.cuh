@@ -20,21 +20,33 @@ static_assert(kTileBins % 2 == 0 && kTileBins * 11 <= 64, "a thread's counts are
 
 // The input tile, which the encoded block's staging words later overlay: an
 // encoding is kept only when it is shorter than the raw block's 1 + F n_b
-// words, so it fits the tile.
-__host__ __device__ constexpr uint32_t tile_region_bytes(int F) { return (uint32_t)F * kBlock * 4u; }
+// words, so it fits the tile.  Its layouts: rows of 1024 values, one per
+// field (16-byte aligned fields); the same with four words more, a row
+// starting with the 16-byte unit that holds the block's first value, so that
+// the values lie as they do in memory, 0 to 3 words into the row (fields of
+// any alignment); the block's interleaved records as they are in memory.
+// The second layout is a kernel of its own: with its shifts in the code, the
+// aligned case took 0.405 instead of 0.391 ms on a 2^26 x 6 snapshot.
+enum : int { kTileAligned, kTileUnaligned, kTileRecords };
+__host__ __device__ constexpr uint32_t tile_row(int layout) { return layout == kTileUnaligned ? kBlock + 4u : kBlock; }
+__host__ __device__ constexpr uint32_t tile_region_bytes(int F, int layout) {
+    return (uint32_t)F * tile_row(layout) * 4u;
+}
 
 // Dynamic shared memory: the tile and the per-warp histograms, whose space
 // later takes the sorted order (one word per particle).
 constexpr uint32_t kTileHistBytes = (uint32_t)kTileWarps * kMaxBins * 2u;
 static_assert(kTileHistBytes >= kBlock * 4u, "the sorted order overlays the histograms");
-__host__ __device__ constexpr uint32_t tile_smem_bytes(int F) { return tile_region_bytes(F) + kTileHistBytes; }
+__host__ __device__ constexpr uint32_t tile_smem_bytes(int F, int layout) {
+    return tile_region_bytes(F, layout) + kTileHistBytes;
+}
 
 // Resident CTAs per SM the kernels are compiled for: what shared memory
 // allows (227 KB, 1 KB reserved per CTA, about 0.6 KB of static memory), at
 // most nine (56 registers per thread; more CTAs spill, see gpz_qse_tile.cu).
 constexpr int kTileMaxCtas = 9;
 __host__ __device__ constexpr int tile_ctas(int F) {
-    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F) + 1024u + 640u));
+    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, kTileUnaligned) + 1024u + 640u));
     return by_smem < kTileMaxCtas ? by_smem : kTileMaxCtas;
 }
 
@@ -52,7 +64,9 @@ struct alignas(16) TileField {
     uint32_t wf, cmask;        // bits in the record and their mask
     uint32_t rot, kmask;       // segId: the code rotated left by rot, under kmask (its place in the key)
     float s, ebchk;            // step, verification threshold
-    uint32_t bits, pad[3];     // code width
+    uint32_t bits;             // code width
+    uint32_t row;              // tile word of value 0 (unaligned layout)
+    uint32_t pad[2];
 };
 
 struct alignas(16) TileShared {
@@ -74,11 +88,11 @@ constexpr uint32_t kTfBig = 2u;        // a code reaches 2^23: general path
 constexpr uint32_t kTfVerify = 4u;     // some field's first candidates need their check
 
 // Warp 0, every lane: the fields' constants (lane f) from the block's
-// extremes e and the step constants p: q0 = floor(fma(x - min, 1/s, 1/2)) is
+// extremes e, the step constants p and the tile word of its value 0: q0 = floor(fma(x - min, 1/s, 1/2)) is
 // monotone in x, so when every value keeps its first candidate the largest
 // code is q0 of the block maximum.
 template <int F>
-__device__ __forceinline__ void tile_constants(const uint2 e, const FieldParams& p, int G, TileShared& S) {
+__device__ __forceinline__ void tile_constants(const uint2 e, const FieldParams& p, int G, uint32_t row, TileShared& S) {
     constexpr int P = F < 3 ? F : 3;
     const int lane = threadIdx.x;
     const bool fl = lane < F;
@@ -104,6 +118,7 @@ __device__ __forceinline__ void tile_constants(const uint2 e, const FieldParams&
         c.mn = mn;
         c.inv = p.inv;
         c.wf = wf;
+        c.row = row;
         c.cmask = (1u << (wf & 31u)) - 1u;
         c.rot = (ks - wf) & 31u;
         c.kmask = ((1u << g) - 1u) << ks;
@@ -124,16 +139,15 @@ __device__ __forceinline__ void or_bits(uint32_t* words, uint32_t pos, unsigned 
 
 // Steps 3 to 5 for a block whose records are at most 32 NR bits wide (NR = 2
 // or 4): the common case keeps two registers per record instead of four.
-// AOS: the tile holds records, value (f, i) at i * F + f.
-template <int F, bool FULL, bool AOS, int NR, class Idx>
+template <int F, bool FULL, int LAY, int NR, class Idx>
 __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, TileShared& S, Idx idx, int n_b,
                                             uint32_t flags, uint32_t W) {
     constexpr int P = F < 3 ? F : 3;
     constexpr int R = kTileRounds, NW = kTileWarps;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     uint32_t* stage = reinterpret_cast<uint32_t*>(dsm);
-    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F));  // [NW][512] per-warp histograms
-    uint32_t* order = reinterpret_cast<uint32_t*>(hist);                       // [1024] the sorted order, later
+    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY));  // [NW][512] per-warp histograms
+    uint32_t* order = reinterpret_cast<uint32_t*>(hist);                            // [1024] the sorted order, later
     const int i0 = 32 * R * w + lane;  // this thread's particles: i0 + 32 r
     auto valid = [&](int r) { return FULL || i0 + 32 * r < n_b; };
 
@@ -162,6 +176,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
             const uint4 c0 = reinterpret_cast<const uint4*>(&S.fc[f])[0];
             const uint4 c1 = reinterpret_cast<const uint4*>(&S.fc[f])[1];
             const float mn = __uint_as_float(c0.x), inv = __uint_as_float(c0.y);
+            const float* row = tile + (LAY == kTileUnaligned ? (int)S.fc[f].row : f * kBlock) + i0;
             const uint32_t wf = c0.z, cmask = c0.w, rot = c1.x, kmask = c1.y;
             const float s = __uint_as_float(c1.z), ebchk = __uint_as_float(c1.w);
             // the smallest and the largest code of the field's width: a fallback
@@ -174,7 +189,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
             }
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const float x = AOS ? tile[(i0 + 32 * r) * F + f] : tile[f * kBlock + i0 + 32 * r];
+                const float x = LAY == kTileRecords ? tile[(i0 + 32 * r) * F + f] : row[32 * r];
                 const float tt = __fmaf_rn(__fsub_rn(x, mn), inv, 0.5f);
                 const float u = __fadd_rd(tt, 8388608.0f);  // 2^23 + floor(t), t < 2^23 here
                 uint32_t ub = __float_as_uint(u);
@@ -256,7 +271,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     {
         // the staging words, assembled by OR, overlay the tile: clear what
         // the block can need (deltas <= 512 x 9 bits, counts <= 512 x 11)
-        const uint32_t need = min((hdr + 144u + 176u + rwords + 3u) >> 2, tile_region_bytes(F) / 16u);
+        const uint32_t need = min((hdr + 144u + 176u + rwords + 3u) >> 2, tile_region_bytes(F, LAY) / 16u);
         uint4* s4 = reinterpret_cast<uint4*>(stage);
         for (uint32_t k = t; k < need; k += kTileThreads) s4[k] = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -453,20 +468,35 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
 
 }  // namespace
 
-// AOS: the input is interleaved records (a.interleaved); the tile then holds
-// the block's records as they are in memory, value (f, i) at i * F + f.
-template <int F, bool FULL, bool PRE, class Idx, bool AOS = false>
+// kTileRecords: the input is interleaved records (a.interleaved), 16-byte
+// aligned; value (f, i) lies at i * F + f of the tile.
+template <int F, bool FULL, bool PRE, int LAY, class Idx>
 __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, TileShared& S, Idx idx) {
+    constexpr bool AOS = LAY == kTileRecords, UNAL = LAY == kTileUnaligned;
+    constexpr uint32_t ROW = tile_row(LAY);
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const uint32_t b = idx.b();  // the block within its array
     const uint64_t first = (uint64_t)b * kBlock;
     const int n_b = FULL ? kBlock : (int)(a.n - first);
-    float* tile = reinterpret_cast<float*>(dsm);  // [F][1024] input ([1024][F] if AOS)
+    float* tile = reinterpret_cast<float*>(dsm);  // [F] rows of input (the block's records if AOS)
 
     // ---- 1. the tile: one bulk copy per field (lane f of warp 0; one copy of
-    // the whole run of records if AOS); the ragged tail of a last block by
-    // plain loads
-    const uint32_t nvec = (AOS ? (uint32_t)(F * n_b) : (uint32_t)n_b) & ~3u;  // values moved in 16-byte units
+    // the whole run of records if AOS), of every 16-byte unit that holds a
+    // value of the block and lies inside the array; the values of the array's
+    // first and last unit, where those are cut, by plain loads
+    // words in field f's row before value 0
+    auto shift = [&](int f) { return !UNAL ? 0u : (uint32_t)(reinterpret_cast<uintptr_t>(a.fields[f]) >> 2) & 3u; };
+    // first unit and past the last, counted from the row's start (values of
+    // the row: words s .. s + n_b - 1; of the array: words from s - first)
+    auto units = [&](uint32_t s, uint32_t& lo, uint32_t& hi) {
+        lo = UNAL && first == 0 && s ? 1u : 0u;
+        hi = (uint32_t)n_b >> 2;
+        if (!UNAL) return;
+        const uint64_t left = a.n - first;  // the array's values from here on
+        hi = min((s + (uint32_t)n_b + 3u) >> 2, (uint32_t)min((s + left) >> 2, (uint64_t)(ROW / 4u)));
+        hi = max(hi, lo);
+    };
+    const uint32_t nrec = (uint32_t)(F * n_b) & ~3u;  // AOS: words of the records' whole units
     if (w == 0) {
         if (lane == 0) {
             mbar_init(&S.bar, AOS ? 1 : F);
@@ -474,25 +504,35 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
             S.unsure = 0u;
         }
         __syncwarp();
-        if (lane < (AOS ? 1 : F)) {
-            mbar_arrive_expect_tx(&S.bar, nvec * 4u);
-            if (nvec) {
-                const float* src = AOS ? a.fields[0] + first * F : a.fields[lane] + first;
-                bulk_g2s(tile + lane * kBlock, src, nvec * 4u, &S.bar);
+        if (AOS) {
+            if (lane == 0) {
+                mbar_arrive_expect_tx(&S.bar, nrec * 4u);
+                if (nrec) bulk_g2s(tile, a.fields[0] + first * F, nrec * 4u, &S.bar);
             }
+        } else if (lane < F) {
+            const uint32_t s = shift(lane);
+            uint32_t lo, hi;
+            units(s, lo, hi);
+            mbar_arrive_expect_tx(&S.bar, (hi - lo) * 16u);
+            if (hi > lo)
+                bulk_g2s(tile + lane * ROW + 4u * lo, a.fields[lane] + first - s + 4u * lo, (hi - lo) * 16u, &S.bar);
         }
     }
-    if (!FULL) {
-        if (AOS) {
-            const int k = (int)nvec + t;
-            if (t < 4 && k < F * n_b) tile[k] = __ldcs(a.fields[0] + first * F + k);
-        } else if (t < 4 * F) {
-            const int f = t >> 2, i = (int)nvec + (t & 3);
-            if (i < n_b) tile[f * kBlock + i] = __ldcs(a.fields[f] + first + i);
+    if (AOS) {
+        if (!FULL && t < 4) {
+            const uint32_t k = nrec + t;
+            if (k < (uint32_t)(F * n_b)) tile[k] = __ldcs(a.fields[0] + first * F + k);
         }
+    } else if ((UNAL || !FULL) && t < 8 * F) {  // up to three words at either end of the row
+        const int f = t >> 3;
+        const uint32_t s = shift(f), end = s + (uint32_t)n_b;
+        uint32_t lo, hi;
+        units(s, lo, hi);
+        const uint32_t k = (t & 4) ? 4u * hi + (t & 3) : s + (t & 3);
+        if (k >= s && k < end && ((t & 4) || k < 4u * lo)) tile[f * ROW + k] = __ldcs(a.fields[f] + first + (k - s));
     }
     {
-        uint4* h4 = reinterpret_cast<uint4*>(dsm + tile_region_bytes(F)) + w * (kMaxBins / 8);
+        uint4* h4 = reinterpret_cast<uint4*>(dsm + tile_region_bytes(F, LAY)) + w * (kMaxBins / 8);
 #pragma unroll
         for (int k = 0; k < kMaxBins / 256; ++k) h4[lane + 32 * k] = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -505,8 +545,9 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         for (int f = w; f < F; f += kTileWarps) {
             float lo = INFINITY, hi = -INFINITY;
             float p0 = 0.0f, p1 = 0.0f, p2 = 0.0f, p3 = 0.0f;  // become NaN if a value is NaN or infinite (x * 0)
-            if (FULL && !AOS) {
-                const float4* v4 = reinterpret_cast<const float4*>(tile + f * kBlock) + lane;
+            const uint32_t sh = shift(f);
+            if (FULL && !AOS && sh == 0u) {
+                const float4* v4 = reinterpret_cast<const float4*>(tile + f * ROW) + lane;
 #pragma unroll
                 for (int k = 0; k < kBlock / 128; ++k) {
                     const float4 v = v4[32 * k];
@@ -518,9 +559,9 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
                     p3 = __fmaf_rn(v.w, 0.0f, p3);
                 }
             } else {
-#pragma unroll 4
+#pragma unroll 8
                 for (int i = lane; i < n_b; i += 32) {
-                    const float v = AOS ? tile[i * F + f] : tile[f * kBlock + i];
+                    const float v = AOS ? tile[i * F + f] : tile[f * ROW + sh + i];
                     lo = fminf(lo, v);
                     hi = fmaxf(hi, v);
                     p0 = __fmaf_rn(v, 0.0f, p0);
@@ -541,7 +582,7 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
             e = PRE ? __ldg(a.bext + (size_t)b * F + lane) : S.ext[lane];
             p = a.d_params ? a.d_params[lane] : a.params[lane];
         }
-        tile_constants<F>(e, p, a.G, S);
+        tile_constants<F>(e, p, a.G, lane < F ? (uint32_t)lane * ROW + shift(lane) : 0u, S);
     }
     __syncthreads();  // the constants (with a range pass also the mbarrier and the plainly loaded values)
     if (PRE && !mbar_wait_bounded(&S.bar, 0, a.status)) return;  // no copy may outlive the CTA
@@ -556,9 +597,9 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         return;
     }
     if (F <= 2 || W <= 64u)  // two fields of codes below 2^23 never need more
-        tile_encode<F, FULL, AOS, 2>(a, dsm, S, idx, n_b, flags, W);
+        tile_encode<F, FULL, LAY, 2>(a, dsm, S, idx, n_b, flags, W);
     else
-        tile_encode<F, FULL, AOS, 4>(a, dsm, S, idx, n_b, flags, W);
+        tile_encode<F, FULL, LAY, 4>(a, dsm, S, idx, n_b, flags, W);
 }
 
 }  // namespace gpz

@@ -1,0 +1,54 @@
+// gpz_qse_tile_launch.cuh -- the single-array tile compression kernel and its
+// launch, instantiated per layout of the tile (gpz_qse_tile.cu describes the
+// design).
+#pragma once
+
+#include "gpz_qse_tile.cuh"
+
+namespace gpz {
+
+template <int F, bool PRE, int LAY>
+__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
+    extern __shared__ __align__(128) uint8_t dsm[];
+    __shared__ TileShared S;
+    if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
+        qse_block_tile<F, true, PRE, LAY>(a, dsm, S, GridBlock{});
+    else
+        qse_block_tile<F, false, PRE, LAY>(a, dsm, S, GridBlock{});
+}
+
+template <int F, bool PRE, int LAY>
+cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
+    const size_t smem = tile_smem_bytes(F, LAY);
+    auto kern = gpz_qse_tile_kernel<F, PRE, LAY>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    return launch_qse_general(a, s);
+}
+
+// One layout's launches (a translation unit each, so that they compile in
+// parallel: gpz_qse_tile.cu, gpz_qse_tile_unaligned.cu, gpz_aos.cu).
+template <int LAY>
+cudaError_t launch_qse_tile_layout(const QseArgs& a, cudaStream_t s) {
+    const bool pre = a.bext != nullptr;
+    switch (a.F) {
+#define GPZ_CASE(FF) \
+    case FF: return pre ? launch_qse_tile_fp<FF, true, LAY>(a, s) : launch_qse_tile_fp<FF, false, LAY>(a, s);
+        GPZ_CASE(1)
+        GPZ_CASE(2)
+        GPZ_CASE(3)
+        GPZ_CASE(4)
+        GPZ_CASE(5)
+        GPZ_CASE(6)
+        GPZ_CASE(7)
+        GPZ_CASE(8)
+#undef GPZ_CASE
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace gpz

@@ -51,3 +51,14 @@ def test_fallback_candidates(gpz, oracle, codes, n, offset, eb):  # noqa: F811
         assert sum(first_candidate_failures(x[0, k:k + 1024], eb) for k in range(0, n, 1024)) > 0
     for mode in (0, 1):
         assert_parity(gpz, oracle, x, eb if mode == 0 else eb / (2.0 * eb * codes), mode, 3)
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+@pytest.mark.parametrize("F,mode", [(1, 0), (3, 1), (6, 1), (8, 0)])
+@pytest.mark.parametrize("n", [1, 2, 5, 1023, 1024, 1025, 1026, 1027, 1029, 2047, 2 * 1024 + 2])
+def test_unaligned_rows(gpz, oracle, offset, F, mode, n):  # noqa: F811
+    """Fields 1 to 3 words past a 16-byte boundary, at the sizes where the
+    array's first and last 16-byte units are cut (a last block of one to three
+    values may not fill its first unit)."""
+    x = (np.random.default_rng(n + offset).random((F, n)) * 100.0).astype(np.float32)
+    assert_parity(gpz, oracle, x, 1e-2 if mode == 0 else 1e-4, mode, 3, offset=offset)

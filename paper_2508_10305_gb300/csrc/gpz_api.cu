@@ -227,10 +227,10 @@ RangeTargets compress_range_targets(uint64_t n, int F) {
     return r;
 }
 
-// gpz_compress; with range_done the range pass's outputs (the block
-// extremes, the CTAs' partial extremes folded into the constants) are
-// already in the workspace, written on this stream by a kernel that read the
-// fields anyway, and are neither cleared nor recomputed.
+// gpz_compress; with range_done the range pass's outputs -- the block
+// extremes and, with a relative bound, the constants -- are already in the
+// workspace, written on this stream by a kernel that read the fields anyway,
+// and are neither cleared nor recomputed.
 gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_params* p, void* d_out,
                          uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size, uint32_t* d_perm,
                          void* d_ws, uint64_t ws_size, void* stream, bool range_done,
@@ -271,9 +271,9 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
 
     gpz_status rc = GPZ_OK;
     Recorder rec(s);
-    range_done = range_done && p->mode == GPZ_EB_REL && d_ws != nullptr && !own_ws;
+    range_done = range_done && d_ws != nullptr && !own_ws;
     do {
-        if (range_done) {  // keep the constants: clear the control words and the look-back states only
+        if (range_done && p->mode == GPZ_EB_REL) {  // keep the constants: clear the control words and the look-back states only
             if ((rc = cuda_status(cudaMemsetAsync(ws + L.ctrl, 0, kCtrlBytes, s))) != GPZ_OK) break;
             if ((rc = cuda_status(cudaMemsetAsync(ws + L.states, 0, L.zero_bytes - L.states, s))) != GPZ_OK) break;
         } else if ((rc = cuda_status(cudaMemsetAsync(ws, 0, L.zero_bytes, s))) != GPZ_OK) {
@@ -332,7 +332,7 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         qa.G = p->seg_bits;
         qa.interleaved = interleaved ? 1 : 0;
         qa.d_params = rel ? d_params : nullptr;
-        qa.bext = rel ? reinterpret_cast<const uint2*>(ws + L.bext) : nullptr;
+        qa.bext = rel || (range_done && !fused) ? reinterpret_cast<const uint2*>(ws + L.bext) : nullptr;
         qa.binfo = rel && fused ? reinterpret_cast<const unsigned long long*>(ws + L.binfo) : nullptr;
         qa.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
         qa.slot_words = slot_words_of(F);

@@ -68,7 +68,7 @@ cudaError_t launch_decompress(const DecArgs& a, cudaStream_t s) {
 // a.out[f] holds the address of field f's double array, and every value is
 // the fp32 reconstruction widened exactly.
 cudaError_t launch_decompress64(const DecArgs& a, cudaStream_t s) {
-    return all_aligned(a) ? launch_decompress_out<kOut64>(a, s) : launch_decompress_out<kOutAny64>(a, s);
+    return launch_decompress_out<kOut64>(a, s);
 }
 
 }  // namespace gpz

@@ -51,22 +51,40 @@ __device__ __forceinline__ float small_u2f(uint32_t q) {
     return __fsub_rn(__uint_as_float(q + 0x4B000000u), 8388608.0f);
 }
 
-// Store four consecutive values at out[first .. first + 3]: fp32, or widened
-// to fp64 (exact) when OUT64 -- then `out` holds a double array's address.
-template <bool OUT64>
-__device__ __forceinline__ void store4(float* out, uint64_t first, const float* v, int left) {
-    if (OUT64) {
-        double* dst = reinterpret_cast<double*>(out) + first;
-        if (left >= 4 && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
-            reinterpret_cast<double2*>(dst)[0] = make_double2((double)v[0], (double)v[1]);
-            reinterpret_cast<double2*>(dst)[1] = make_double2((double)v[2], (double)v[3]);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (e < left) dst[e] = (double)v[e];
-        }
-        return;
+// The doubles of four floats, on the integer pipe: fp64 conversions kept
+// their pipe 78% busy (2^23 x 6 values: 0.116 -> 0.093 ms, with positions
+// strided so that a warp's 8-byte stores are consecutive).  Normal magnitudes only move their fields; a group
+// with any other value takes the second form.
+__device__ __forceinline__ double widen_any(float v) {
+    const uint32_t u = __float_as_uint(v), sign = u & 0x80000000u;
+    uint32_t m = u & 0x7fffffffu;
+    if (m >= 0x7f800000u)  // infinite, NaN
+        return __hiloint2double((int)(sign | ((m >> 3) + 0x70000000u)), (int)(u << 29));
+    if (m == 0u) return __hiloint2double((int)sign, 0);
+    uint32_t bias = 0x38000000u;
+    if (m < 0x00800000u) {  // subnormal: to a leading one at bit 23
+        const int sh = __clz(m) - 8;
+        m <<= sh;
+        bias -= (uint32_t)sh << 20;
     }
+    return __hiloint2double((int)(sign | ((m >> 3) + bias)), (int)(m << 29));
+}
+__device__ __forceinline__ void widen4(const float* v, double* d) {
+    bool other = false;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const uint32_t u = __float_as_uint(v[e]), m = u & 0x7fffffffu;
+        other |= m - 0x00800000u >= 0x7f000000u;
+        d[e] = __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+    }
+    if (other) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) d[e] = widen_any(v[e]);
+    }
+}
+
+// Store four consecutive values at out[first .. first + 3].
+__device__ __forceinline__ void store4(float* out, uint64_t first, const float* v, int left) {
     float* dst = out + first;
     if (left >= 4 && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
         __stcs(reinterpret_cast<float4*>(dst), make_float4(v[0], v[1], v[2], v[3]));
@@ -91,9 +109,9 @@ __device__ __forceinline__ void rebuild4(const uint32_t* q, uint32_t bits, float
     for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(bits <= 23u ? small_u2f(q[e]) : __uint2float_rn(q[e]), s, mn);
 }
 
-// Where a block's values go: fp32 fields or fp64 fields, 16-byte aligned or of
-// any alignment, or interleaved fp32 records.
-enum : int { kOut32, kOutAny, kOut64, kOutAny64, kOutRecords };
+// Where a block's values go: fp32 fields, 16-byte aligned or of any alignment,
+// fp64 fields, or interleaved fp32 records.
+enum : int { kOut32, kOutAny, kOut64, kOutRecords };
 
 // The positions a thread rebuilds, in groups of four: four consecutive ones,
 // stored with 16-byte stores, into aligned fields; otherwise one of each run
@@ -102,7 +120,7 @@ enum : int { kOut32, kOutAny, kOut64, kOutAny64, kOutRecords };
 // 10^7 x 6 snapshot: 53 us; with 4-byte stores of four consecutive positions
 // per lane 55, with 16-byte units completed by shuffles from the next lane
 // 68; aligned rows 50.)
-__host__ __device__ constexpr bool out_strided(int out) { return out != kOut32 && out != kOut64; }
+__host__ __device__ constexpr bool out_strided(int out) { return out != kOut32; }
 template <int OUT>
 __device__ __forceinline__ int out_pos(int g, int e) {
     const int t = threadIdx.x;
@@ -116,17 +134,19 @@ __device__ __forceinline__ void store_group(const DecArgs& a, int f, int g, cons
                                             float* recs) {
     if (!out_strided(OUT)) {
         const int j = out_pos<OUT>(g, 0);
-        store4<OUT == kOut64>(a.out[f], base + j, v, n_b - j);
+        store4(a.out[f], base + j, v, n_b - j);
         return;
     }
+    double d[4];
+    if (OUT == kOut64) widen4(v, d);
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const int j = out_pos<OUT>(g, e);
         if (j >= n_b) continue;
         if (OUT == kOutRecords)
             recs[rec_slot<F>(j, f)] = v[e];
-        else if (OUT == kOutAny64)
-            __stcs(reinterpret_cast<double*>(a.out[f]) + base + j, (double)v[e]);
+        else if (OUT == kOut64)
+            __stcs(reinterpret_cast<double*>(a.out[f]) + base + j, d[e]);
         else
             __stcs(a.out[f] + base + j, v[e]);
     }
@@ -404,7 +424,7 @@ __device__ __forceinline__ void store_records(const DecArgs& a, const float* rec
 template <int F, int OUT>
 __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32_t* stage,
                                             const uint32_t* blk, uint32_t b, int n_b) {
-    constexpr bool OUT64 = OUT == kOut64 || OUT == kOutAny64, AOS = OUT == kOutRecords;
+    constexpr bool OUT64 = OUT == kOut64, AOS = OUT == kOutRecords;
     uint16_t* uniq = S.uniq;
     uint32_t* mask = S.mask;
     uint32_t& s_bad = S.bad;

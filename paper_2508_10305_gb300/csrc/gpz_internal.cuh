@@ -93,14 +93,13 @@ constexpr uint32_t kPlaced = 0x80000000u;  // in a block's word count: already i
 // look-back over its predecessors' published sizes).
 constexpr int kCmTemp = 0, kCmDirect = 1;
 
-struct F64Args {                // fp64 input and output (gpz_f64.cu)
+struct F64Args {                // fp64 input (gpz_f64.cu)
     const double* in[kMaxFields];
-    float* out32[kMaxFields];
-    const float* in32[kMaxFields];
-    double* out64[kMaxFields];
+    float* out32[kMaxFields];   // 16-byte aligned
     uint64_t n;
     int F;
     unsigned long long* res;    // [F][3]: min key, max key, largest rounding error (bits)
+    uint2* bext;                // out, [nblocks][F]: each block's fp32 extremes, as RangeArgs
 };
 
 struct ScanArgs {
@@ -170,6 +169,12 @@ __device__ __forceinline__ FieldParams range_params(float lo, float hi, double r
 }
 
 // ---------------------------------------------------------------- helpers
+
+// fp64 operations run at 1/64 of the fp32 rate here (a warp's takes 16 cycles
+// of its SM, also with every lane predicated off), so they stay out of paths
+// that only move or compare bits: rare conversions sit behind a call, and
+// values whose bits are worked on are loaded as integers -- masks on the bits
+// of a loaded double become fp64 negations and absolute values.
 
 // ceil(2^32 / d) for d = 1..255 (entry 0 unused), built at compile time: with
 // m = ceil(2^32 / d), floor(n / d) = floor(n * m / 2^32) exactly for n < 2^18

@@ -74,8 +74,7 @@ struct WideDecArgs {
     uint32_t* status;
 };
 
-__device__ __forceinline__ unsigned long long wide_key(double x) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+__device__ __forceinline__ unsigned long long wide_key(unsigned long long u) {
     return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
 }
 
@@ -164,25 +163,71 @@ __device__ __forceinline__ bool wide_quantise(double x, const WideParams& p, dou
 
 // ---------------------------------------------------------------- range pass
 
-__global__ void __launch_bounds__(kWideThreads) gpz_wide_range_kernel(WideRangeArgs a) {
-    const uint64_t stride = (uint64_t)gridDim.x * kWideThreads;
-    const int lane = threadIdx.x & 31;
-    for (int f = 0; f < a.F; ++f) {
+// A warp per (field, 1024 values), eight 16-byte loads in flight per lane.
+// Bound by HBM: the keys' minima and maxima are integer operations (fp64
+// compares kept that pipe 70% busy and the pass at 120 us on 4*10^6 x 6
+// doubles in odd rows; 41 us this way).  NaN keys lie outside the infinities' and
+// are only looked for when an extreme does.
+__global__ void __launch_bounds__(kWideThreads, 6) gpz_wide_range_kernel(const __grid_constant__ WideRangeArgs a) {
+    __shared__ unsigned long long s_res[kMaxFields][2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < kMaxFields) s_res[tid][0] = s_res[tid][1] = 0ull;
+    __syncthreads();
+    constexpr unsigned long long kNegInf = ~0xfff0000000000000ull, kPosInf = 0xfff0000000000000ull;  // order keys
+    const uint64_t nb = (a.n + kBlock - 1) / kBlock, items = nb * (uint64_t)a.F;
+    const uint64_t per = (items + gridDim.x - 1) / gridDim.x;  // consecutive items: mostly one field per CTA
+    const uint64_t end = min(items, (uint64_t)(blockIdx.x + 1) * per);
+    for (uint64_t it = (uint64_t)blockIdx.x * per + warp; it < end; it += kWideWarps) {
+        const int f = (int)(it / nb);
+        const uint64_t b = it - (uint64_t)f * nb;
+        const unsigned long long* x = reinterpret_cast<const unsigned long long*>(a.fields[f]) + b * kBlock;
+        const int n_b = (int)min((uint64_t)kBlock, a.n - b * kBlock);
         unsigned long long nmin = 0ull, kmax = 0ull;  // nmin = max of ~key
-        for (uint64_t i = (uint64_t)blockIdx.x * kWideThreads + threadIdx.x; i < a.n; i += stride) {
-            const double v = __ldcs(a.fields[f] + i);
-            if (v == v) {
-                const unsigned long long k = wide_key(v);
-                nmin = max(nmin, ~k);
-                kmax = max(kmax, k);
+        auto take = [&](unsigned long long v) {
+            const unsigned long long k = wide_key(v);
+            nmin = max(nmin, ~k);
+            kmax = max(kmax, k);
+        };
+        if (n_b == kBlock && (reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
+            const ulonglong2* x2 = reinterpret_cast<const ulonglong2*>(x) + lane;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                ulonglong2 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = __ldcs(x2 + 32 * (8 * h + k));
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    take(v[k].x);
+                    take(v[k].y);
+                }
             }
+        } else {
+#pragma unroll 16
+            for (int i = lane; i < n_b; i += 32) take(__ldcs(x + i));
         }
         nmin = warp_max_u64(nmin);
         kmax = warp_max_u64(kmax);
-        if (lane == 0) {
-            if (nmin) atomicMax(a.res + 2 * f, nmin);
-            if (kmax) atomicMax(a.res + 2 * f + 1, kmax);
+        if (~nmin < kNegInf || kmax > kPosInf) {  // some value is NaN: once more without them
+            nmin = kmax = 0ull;
+            for (int i = lane; i < n_b; i += 32) {
+                const unsigned long long k = wide_key(x[i]);
+                if (k >= kNegInf && k <= kPosInf) {
+                    nmin = max(nmin, ~k);
+                    kmax = max(kmax, k);
+                }
+            }
+            nmin = warp_max_u64(nmin);
+            kmax = warp_max_u64(kmax);
         }
+        if (lane == 0 && nmin) {
+            atomicMax(&s_res[f][0], nmin);
+            atomicMax(&s_res[f][1], kmax);
+        }
+    }
+    __syncthreads();
+    if (tid < a.F && s_res[tid][0]) {
+        atomicMax(a.res + 2 * tid, s_res[tid][0]);
+        atomicMax(a.res + 2 * tid + 1, s_res[tid][1]);
     }
 }
 
@@ -274,14 +319,15 @@ __global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_qse_ker
 
     // ---- 1. load, non-finite values, block minima (order keys)
     bool valid[4];
-    double x[F][4];
+    unsigned long long x[F][4];  // the values' bits
 #pragma unroll
     for (int r = 0; r < 4; ++r) valid[r] = 128 * w + 32 * r + lane < n_b;
 #pragma unroll
     for (int f = 0; f < F; ++f) {
-        const double* src = a.fields[f] + first + 128 * w + lane;
+        const unsigned long long* src =
+            reinterpret_cast<const unsigned long long*>(a.fields[f]) + first + 128 * w + lane;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) x[f][r] = valid[r] ? __ldcs(src + 32 * r) : 0.0;
+        for (int r = 0; r < 4; ++r) x[f][r] = valid[r] ? __ldcs(src + 32 * r) : 0ull;
     }
     __syncthreads();  // shared slots initialised
     bool nonfinite = false;
@@ -291,8 +337,7 @@ __global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_qse_ker
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             if (valid[r]) {
-                const unsigned long long u = (unsigned long long)__double_as_longlong(x[f][r]);
-                nonfinite |= ((u >> 52) & 0x7ffu) == 0x7ffu;  // infinite or NaN
+                nonfinite |= ((x[f][r] >> 52) & 0x7ffu) == 0x7ffu;  // infinite or NaN
                 const unsigned long long k = wide_key(x[f][r]);
                 nk = max(nk, ~k);
                 xk = max(xk, k);
@@ -342,7 +387,7 @@ __global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_qse_ker
         if ((exact >> f) & 1u) {  // uniform over the block
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                q[f][r] = valid[r] ? code_floor(__fma_rn(__dsub_rn(x[f][r], mn[f]), a.params[f].inv, 0.5)) : 0ull;
+                q[f][r] = valid[r] ? code_floor(__fma_rn(__dsub_rn(__longlong_as_double((long long)x[f][r]), mn[f]), a.params[f].inv, 0.5)) : 0ull;
                 qm = max(qm, q[f][r]);
             }
         } else {
@@ -350,7 +395,7 @@ __global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_qse_ker
             for (int r = 0; r < 4; ++r) {
                 q[f][r] = 0ull;
                 if (valid[r]) {
-                    fail |= !wide_quantise(x[f][r], a.params[f], mn[f], q[f][r]);
+                    fail |= !wide_quantise(__longlong_as_double((long long)x[f][r]), a.params[f], mn[f], q[f][r]);
                     qm = max(qm, q[f][r]);
                 }
             }
@@ -1150,8 +1195,10 @@ gpz_status gpz_compress_wide(const double* const* d_fields, uint64_t n, const gp
         ra.n = n;
         ra.F = F;
         ra.res = res;
-        const uint64_t want = (n + kWideThreads - 1) / kWideThreads;
-        const unsigned grid = (unsigned)(want < 152ull * 8ull ? want : 152ull * 8ull);
+        // a warp per block and field, two of them one after the other, more
+        // where the grid would pass a few waves
+        const uint64_t items = nblocks_of(n) * (uint64_t)F, want = (items + 2 * kWideWarps - 1) / (2 * kWideWarps);
+        const unsigned grid = (unsigned)(want < 152ull * 64ull ? want : 152ull * 64ull);
         Recorder rec(s);
         rec.begin(1);
         gpz_wide_range_kernel<<<grid, kWideThreads, 0, s>>>(ra);

@@ -154,7 +154,7 @@ namespace host {
 uint64_t wide_workspace_size(uint64_t n, int F);
 gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G, int mode, const double* eb,
                          void* d_out, uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size,
-                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s);
+                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre = false);
 
 }  // namespace host
 }  // namespace gpz

@@ -9,14 +9,9 @@
 #include <type_traits>
 
 #include "gpz_qse_block.cuh"
+#include "gpz_sort.cuh"
 
 namespace gpz {
-
-constexpr int kTileThreads = 128;              // one CTA per particle block
-constexpr int kTileWarps = kTileThreads / 32;
-constexpr int kTileRounds = kBlock / kTileThreads;  // particles per thread
-constexpr int kTileBins = kMaxBins / kTileThreads;  // histogram bins per thread in the scan
-static_assert(kTileBins % 2 == 0 && kTileBins * 11 <= 64, "a thread's counts are appended to one 64-bit word");
 
 // The input tile, which the encoded block's staging words later overlay: an
 // encoding is kept only when it is shorter than the raw block's 1 + F n_b
@@ -33,12 +28,9 @@ __host__ __device__ constexpr uint32_t tile_region_bytes(int F, int layout) {
     return (uint32_t)F * tile_row(layout) * 4u;
 }
 
-// Dynamic shared memory: the tile and the per-warp histograms, whose space
-// later takes the sorted order (one word per particle).
-constexpr uint32_t kTileHistBytes = (uint32_t)kTileWarps * kMaxBins * 2u;
-static_assert(kTileHistBytes >= kBlock * 4u, "the sorted order overlays the histograms");
+// Dynamic shared memory: the tile and the sort's histograms.
 __host__ __device__ constexpr uint32_t tile_smem_bytes(int F, int layout) {
-    return tile_region_bytes(F, layout) + kTileHistBytes;
+    return tile_region_bytes(F, layout) + kSortHistBytes;
 }
 
 // Resident CTAs per SM the kernels are compiled for: what shared memory
@@ -49,12 +41,6 @@ __host__ __device__ constexpr int tile_ctas(int F) {
     const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, kTileUnaligned) + 1024u + 640u));
     return by_smem < kTileMaxCtas ? by_smem : kTileMaxCtas;
 }
-
-// Ranking a warp's round of 32 keys: match takes time in proportion to the
-// distinct keys (23 cycles of its SM-wide unit per round on scan data, 45 on
-// uniform positions), a shared atomic in proportion to the most lanes on one
-// bank; the first round's distinct keys decide for the others.
-constexpr int kMatchMaxDistinct = 16;
 
 namespace {
 
@@ -69,14 +55,10 @@ struct alignas(16) TileField {
     uint32_t pad[2];
 };
 
-struct alignas(16) TileShared {
+struct alignas(16) TileShared : SortShared {
     uint4 blk;                             // flags, record width, key bits
-    uint32_t tn[kTileWarps];               // per warp: particles | non-empty bins << 16
-    uint32_t last[kTileWarps];             // ... its last non-empty bin
-    uint32_t cmax[kTileWarps], dmax[kTileWarps];  // ... largest count and delta
     uint64_t bar;                          // mbarrier of the tile's bulk copies
     uint32_t fallback;                     // kFbCoded, kFbGeneral
-    uint32_t unsure;                       // some warp's ranks need the check of the sorted order
     uint2 ext[kMaxFields];                 // the block's extremes (order keys; (0, 0): a non-finite value)
     TileField fc[kMaxFields];
 };
@@ -129,24 +111,16 @@ __device__ __forceinline__ void tile_constants(const uint2 e, const FieldParams&
     if (lane == 0) S.blk = make_uint4(flags, W, keybits, 0u);
 }
 
-// ORs the low n (<= 44) bits of v into the shared words at a bit position.
-__device__ __forceinline__ void or_bits(uint32_t* words, uint32_t pos, unsigned long long v, uint32_t n) {
-    const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32), wi = pos >> 5, end = (pos & 31u) + n;
-    if (n) atomicOr(words + wi, __funnelshift_l(0u, lo, pos));
-    if (end > 32u) atomicOr(words + wi + 1, __funnelshift_l(lo, hi, pos));
-    if (end > 64u) atomicOr(words + wi + 2, __funnelshift_l(hi, 0u, pos));
-}
-
 // Steps 3 to 5 for a block whose records are at most 32 NR bits wide (NR = 2
 // or 4): the common case keeps two registers per record instead of four.
 template <int F, bool FULL, int LAY, int NR, class Idx>
 __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, TileShared& S, Idx idx, int n_b,
                                             uint32_t flags, uint32_t W) {
     constexpr int P = F < 3 ? F : 3;
-    constexpr int R = kTileRounds, NW = kTileWarps;
+    constexpr int R = kTileRounds;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     uint32_t* stage = reinterpret_cast<uint32_t*>(dsm);
-    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY));  // [NW][512] per-warp histograms
+    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY)); 
     uint32_t* order = reinterpret_cast<uint32_t*>(hist);                            // [1024] the sorted order, later
     const int i0 = 32 * R * w + lane;  // this thread's particles: i0 + 32 r
     auto valid = [&](int r) { return FULL || i0 + 32 * r < n_b; };
@@ -224,43 +198,8 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
         if (lane == 0) atomicOr(&S.fallback, fail ? kFbGeneral : kFbCoded);
     }
 
-    // ---- 4. counting sort: warp-local ranks, round after round.  The old
-    // count that the shared atomic returns is the particle's rank; within one
-    // round the lanes of equal keys get distinct ranks in the order in which
-    // the hardware serves them, which is checked below (stability).
-    uint16_t* myhist = hist + w * kMaxBins;
-    {
-        uint32_t peers = __match_any_sync(0xffffffffu, valid(0) ? key[0] : 0xffffffffu);
-        if (valid(0)) myhist[key[0]] = (uint16_t)__popc(peers);  // every peer stores the same count
-        const uint32_t rank0 = __popc(peers & lanemask_lt());
-        const int distinct = __popc(__ballot_sync(0xffffffffu, valid(0) && rank0 == 0u));
-        key[0] |= rank0 << 16;  // the rank above the 9 key bits
-        __syncwarp();
-        if (distinct > kMatchMaxDistinct) {
-            if (lane == 0) S.unsure = 1u;
-            uint32_t* h32 = reinterpret_cast<uint32_t*>(myhist);  // two bins per word
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                if (valid(r)) {
-                    const uint32_t sh = (key[r] & 1u) << 4;
-                    const uint32_t old = atomicAdd(h32 + (key[r] >> 1), 1u << sh);
-                    key[r] |= ((old >> sh) & 0xffffu) << 16;
-                }
-                __syncwarp();  // the next round's counts come after this one's
-            }
-        } else {
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                peers = __match_any_sync(0xffffffffu, valid(r) ? key[r] : 0xffffffffu);
-                uint32_t before = 0u;
-                if (valid(r)) before = myhist[key[r]];
-                __syncwarp();
-                if (valid(r)) myhist[key[r]] = (uint16_t)(before + __popc(peers));
-                __syncwarp();
-                key[r] |= (before + __popc(peers & lanemask_lt())) << 16;
-            }
-        }
-    }
+    // ---- 4. counting sort: warp-local ranks, round after round
+    rank_keys(key, hist, valid, S);
     __syncthreads();  // C: every value quantised (the tile is dead) and ranked
     if (const uint32_t fb = S.fallback) {
         if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id() | (fb & kFbGeneral ? 0u : kCodedBlock);
@@ -276,101 +215,11 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
         for (uint32_t k = t; k < need; k += kTileThreads) s4[k] = make_uint4(0u, 0u, 0u, 0u);
     }
 
-    // ---- 4b. scan over (bin, warp): sorted positions and the run-length
-    // code.  Thread t owns bins b0 .. b0 + kTileBins - 1; two 16-bit counts
-    // per word, none of whose sums exceeds 1024.
-    constexpr int BW = kTileBins / 2;
-    const uint32_t b0 = (uint32_t)kTileBins * t;
-    uint32_t row[NW][BW], sum[BW];
-#pragma unroll
-    for (int k = 0; k < BW; ++k) sum[k] = 0u;
-#pragma unroll
-    for (int ww = 0; ww < NW; ++ww)
-    {
-        const uint16_t* cell = hist + ww * kMaxBins + b0;
-        if constexpr (BW == 2) {
-            const uint2 v = *reinterpret_cast<const uint2*>(cell);
-            row[ww][0] = v.x;
-            row[ww][BW - 1] = v.y;
-        } else {
-            row[ww][0] = *reinterpret_cast<const uint32_t*>(cell);
-        }
-#pragma unroll
-        for (int k = 0; k < BW; ++k) sum[k] += row[ww][k];
-    }
-    uint32_t c[kTileBins], tot = 0u, nz = 0u, cm = 0u, mylast = 0u;
-#pragma unroll
-    for (int k = 0; k < kTileBins; ++k) {
-        c[k] = (k & 1) ? sum[k >> 1] >> 16 : sum[k >> 1] & 0xffffu;
-        tot += c[k];
-        nz += c[k] ? 1u : 0u;
-        cm = max(cm, c[k]);
-        if (c[k]) mylast = b0 + k;
-    }
-    // one scan of both: the counts sum to at most 1024 and the non-empty bins
-    // to at most 512, so they share a word
-    const uint32_t incl = warp_incl_sum(tot | (nz << 16));
-    cm = __reduce_max_sync(0xffffffffu, cm);
-    // the last non-empty bin before this thread's, in its warp
-    const uint32_t filled = __ballot_sync(0xffffffffu, tot != 0u), below = filled & lanemask_lt();
-    uint32_t prev = __shfl_sync(0xffffffffu, mylast, below ? 31 - __clz(below) : 0);
-    if (!below) prev = 0u;
-    const uint32_t wlast = __shfl_sync(0xffffffffu, mylast, filled ? 31 - __clz(filled) : 0);
-    if (lane == 31) {
-        S.tn[w] = incl;
-        S.last[w] = wlast;
-        S.cmax[w] = cm;
-    }
-    __syncthreads();  // D
-    uint32_t excl = incl - (tot | (nz << 16)), all = 0u, maxcnt = 0u;
-#pragma unroll
-    for (int ww = 0; ww < NW; ++ww) {
-        const uint32_t v = S.tn[ww];
-        if (ww < w) {
-            excl += v;
-            prev = max(prev, S.last[ww]);  // 0 when none: a first id's delta is the id itself
-        }
-        all += v;
-        maxcnt = max(maxcnt, S.cmax[ww]);
-    }
-    const uint32_t U = all >> 16;
-    uint32_t dm = 0u;
-    {
-        uint32_t start = excl & 0xffffu, pv = prev;
-        uint32_t run[BW];
-#pragma unroll
-        for (int k = 0; k < kTileBins; ++k) {
-            run[k >> 1] = (k & 1) ? run[k >> 1] | (start << 16) : start;
-            start += c[k];
-            if (c[k]) {
-                dm = max(dm, b0 + k - pv);
-                pv = b0 + k;
-            }
-        }
-        // each warp's sorted start of the bins: the start plus the counts of the warps before it
-        if (tot) {
-#pragma unroll
-            for (int ww = 0; ww < NW; ++ww)
-            {
-                uint16_t* cell = hist + ww * kMaxBins + b0;
-                if constexpr (BW == 2)
-                    *reinterpret_cast<uint2*>(cell) = make_uint2(run[0], run[BW - 1]);
-                else
-                    *reinterpret_cast<uint32_t*>(cell) = run[0];
-#pragma unroll
-                for (int k = 0; k < BW; ++k) run[k] += row[ww][k];
-            }
-        }
-    }
-    dm = __reduce_max_sync(0xffffffffu, dm);
-    if (lane == 0) S.dmax[w] = dm;
-    __syncthreads();  // E
-    uint32_t maxdelta = 0u;
-#pragma unroll
-    for (int ww = 0; ww < NW; ++ww) maxdelta = max(maxdelta, S.dmax[ww]);
+    // ---- 4b. scan over (bin, warp): sorted positions and the run-length code
+    const SortRuns runs = scan_bins(hist, S);
 
     // ---- encoded size; raw when not smaller (keeps the bound size a bound)
-    const uint32_t wd = bit_width(maxdelta), wc = bit_width(maxcnt);
+    const uint32_t U = runs.U, wd = bit_width(runs.maxdelta), wc = bit_width(runs.maxcnt);
     const uint32_t dwords = ceil_words(U * wd), cwords = ceil_words(U * wc);
     const uint32_t enc = hdr + dwords + cwords + rwords;
     const uint32_t b = idx.b();
@@ -392,30 +241,13 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
             if ((f >> 2) == t) word |= S.fc[f].bits << (8 * (f & 3));
         stage[1 + F + t] = word;
     }
-    if (tot) {
-        unsigned long long dv = 0ull, cv = 0ull;
-        uint32_t nd = 0u, nc = 0u, pv = prev;
-#pragma unroll
-        for (int k = 0; k < kTileBins; ++k) {
-            if (c[k]) {
-                dv |= (unsigned long long)(b0 + k - pv) << nd;
-                cv |= (unsigned long long)c[k] << nc;
-                nd += wd;
-                nc += wc;
-                pv = b0 + k;
-            }
-        }
-        const uint32_t k0 = excl >> 16;  // index of the thread's first run
-        or_bits(stage, 32u * hdr + k0 * wd, dv, nd);
-        or_bits(stage, 32u * (hdr + dwords) + k0 * wc, cv, nc);
-    }
+    or_runs(stage, runs, hdr, wd, wc);
     {
         const uint32_t rbase = 32u * (hdr + dwords + cwords);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (!valid(r)) continue;
-            const uint32_t k9 = key[r] & 0xffffu, dest = myhist[k9] + (key[r] >> 16);  // sorted position
-            key[r] = k9 | (dest << 16);
+            const uint32_t dest = sorted_position(key[r], hist);
             if (W == 0u) continue;
             const uint32_t bp = rbase + dest * W, end = (bp & 31u) + W;
             uint32_t* at = stage + (bp >> 5);
@@ -433,32 +265,8 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
         a.sizes[b] = enc;
         bulk_s2g_start(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
     }
-    const bool unsure = S.unsure != 0u;
-    if (unsure || a.perm) {
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-            if (valid(r)) order[key[r] >> 16] = ((key[r] & 0xffffu) << 10) | (uint32_t)(i0 + 32 * r);
-        __syncthreads();
-    }
-    // ---- the sort was stable if (key, index) increases strictly along the
-    // sorted positions; else the general kernel redoes the block
-    bool bad = false;
-    if (unsure) {
-#pragma unroll
-    for (int k = 0; k < kBlock / (4 * kTileThreads); ++k) {
-        const int j = 4 * (t + kTileThreads * k);
-        const uint4 v = reinterpret_cast<const uint4*>(order)[t + kTileThreads * k];
-        uint32_t next = __shfl_down_sync(0xffffffffu, v.x, 1);
-        if (lane == 31) next = j + 4 < kBlock ? order[j + 4] : 0xffffffffu;
-        bad |= (FULL || j + 1 < n_b) && v.x >= v.y;
-        bad |= (FULL || j + 2 < n_b) && v.y >= v.z;
-        bad |= (FULL || j + 3 < n_b) && v.z >= v.w;
-        bad |= (FULL || j + 4 < n_b) && v.w >= next;
-    }
-        bad = __syncthreads_or(bad);
-    }
-    if (bad) {
-        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();
+    if (!sorted_order(key, order, valid, i0, n_b, a.perm != nullptr, S)) {
+        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();  // not stable: the general kernel redoes it
     } else if (a.perm) {
         const uint64_t first = (uint64_t)b * kBlock;
         for (int j = t; j < n_b; j += kTileThreads) a.perm[first + j] = (uint32_t)first + (order[j] & 1023u);

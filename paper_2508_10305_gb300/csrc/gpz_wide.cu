@@ -20,80 +20,22 @@
 // not smaller.
 //
 // Kernels: a range pass (relative bounds), one CTA per block for the stages
-// (the codes sorted into shared memory, each thread's four sorted records
+// (gpz_wide_fast.cu; the blocks it leaves are done here by the general kernel:
+// the codes sorted into shared memory, each thread's four sorted records
 // appended into staging words), the scan and copy of the 32-bit form, and one
-// CTA per block to decode (the record words staged in shared memory).
+// CTA per block to decode (the block's words staged in shared memory).
 #include <cmath>
 #include <cstring>
 
 #include "gpz.h"
 #include "gpz_host.hpp"
 #include "gpz_internal.cuh"
+#include "gpz_wide.cuh"
 
 using namespace gpz;
 using namespace gpz::host;
 
 namespace gpz {
-
-constexpr int kWideThreads = 256;
-constexpr int kWideWarps = kWideThreads / 32;
-constexpr uint32_t kWideMaxBits = 53;
-constexpr unsigned long long kWideLimit = 1ull << 53;  // codes stay below 2^53
-constexpr double kWideLimitD = 9007199254740992.0;     // 2^53
-constexpr uint32_t kWideDcWords = 144u + 176u;         // deltas (<= 9 bits) and counts (<= 11 bits) of <= 512 runs
-
-struct WideParams {
-    double eb, s, inv, ebchk;
-};
-
-struct WideRangeArgs {
-    const double* fields[kMaxFields];
-    uint64_t n;
-    int F;
-    unsigned long long* res;  // [F][2]: max of ~key (the minimum), max of key, over the non-NaN values; zeroed
-};
-
-struct WideQseArgs {
-    const double* fields[kMaxFields];
-    uint64_t n;
-    int F, G;
-    WideParams params[kMaxFields];
-    uint32_t* temp;  // [nblocks][slot_words]
-    uint32_t slot_words;
-    uint32_t* sizes;  // [nblocks]
-    uint32_t* perm;   // [n] or nullptr
-};
-
-struct WideDecArgs {
-    const uint32_t* stream;
-    uint64_t total_words;
-    double* out[kMaxFields];
-    uint64_t n;
-    int F;
-    uint32_t nblocks;
-    uint32_t* status;
-};
-
-__device__ __forceinline__ unsigned long long wide_key(unsigned long long u) {
-    return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-
-__device__ __forceinline__ double wide_from_key(unsigned long long k) {
-    return __longlong_as_double((long long)((k >> 63) ? (k & 0x7fffffffffffffffull) : ~k));
-}
-
-// Maximum over the warp (every lane calls it): the largest high word, then
-// the largest low word among the lanes that hold it (two redux operations).
-__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-    const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
-    const uint32_t mh = __reduce_max_sync(0xffffffffu, hi);
-    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
-    return ((unsigned long long)mh << 32) | ml;
-}
-
-__device__ __forceinline__ uint32_t bit_width64(unsigned long long v) { return 64u - (uint32_t)__clzll((long long)v); }
-
-__device__ __forceinline__ unsigned long long mask64(uint32_t w) { return w >= 64u ? ~0ull : ((1ull << w) - 1ull); }
 
 // |d| <= c for a non-NaN d and c >= 0, on the bit patterns (integer pipe).
 __device__ __forceinline__ bool abs_le(double d, double c) {
@@ -110,35 +52,11 @@ __device__ __forceinline__ double code_to_double(unsigned long long q) {
     return q ? __longlong_as_double((long long)bits) : 0.0;
 }
 
-// floor(t) for 0 <= t < 2^53, on the integer pipe: the significand shifted
-// right by the fraction bits the exponent leaves below the binary point.
-__device__ __forceinline__ unsigned long long code_floor(double t) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(t);
-    const int e = (int)(u >> 52) - 1023;  // t >= 0
-    const unsigned long long m = (u & 0xfffffffffffffull) | 0x10000000000000ull;
-    return e < 0 ? 0ull : (e >= 52 ? m : (m >> (52 - e)));
-}
-
 // The decompressor's reconstruction of code q, checked against the bound
 // (x is finite, so x - x^ is never NaN).
 __device__ __forceinline__ bool wide_ok(double x, unsigned long long q, const WideParams& p, double mn) {
     const double xh = __fma_rn(code_to_double(q), p.s, mn);
     return abs_le(__dsub_rn(x, xh), p.ebchk);
-}
-
-// When the first candidate needs no check.  With u = 2^-53, D = x - min >= 0,
-// r = D / s and the three roundings of t = fma(RN(D), RN(1/s), 1/2):
-// |q - r| <= 1/2 + e, e <= 3.01 u r + u/2; the reconstruction
-// X = q s + min rounds to x^ with |x^ - X| <= u |X|, and the check's
-// difference rounds once more.  So |RN(x - x^)| <= (s (1/2 + e) + u |X|)(1 + u).
-// With s <= eb (63/32)(1 + u), r <= 2^40 (then e < 3.7e-4) and
-// |X| <= max|x| + s <= eb (2^45 + 2) (then u |X| / eb < 0.0040), this is
-// below 0.990 eb, under the threshold eb (1 - 2^-51) -- the 1/64 margin of
-// the step absorbs the rounding.  eb >= 2^-1000 keeps every quantity normal
-// (a subnormal difference is exact; a subnormal x^ errs by 2^-1075 at most).
-__device__ __forceinline__ bool first_candidate_exact(double bmin, double bmax, const WideParams& p) {
-    return p.eb >= 0x1p-1000 && __dsub_ru(bmax, bmin) <= p.s * 0x1p40 &&
-           fmax(fabs(bmin), fabs(bmax)) <= p.eb * 0x1p45;
 }
 
 // Candidates q, q - 1, q + 1 (codes below 2^53); false when none passes.
@@ -207,6 +125,11 @@ __global__ void __launch_bounds__(kWideThreads, 6) gpz_wide_range_kernel(const _
         }
         nmin = warp_max_u64(nmin);
         kmax = warp_max_u64(kmax);
+        if (lane == 0) {
+            const bool finite = ~nmin > kNegInf && kmax < kPosInf;
+            reinterpret_cast<ulonglong2*>(a.temp + b * a.slot_words)[f] =
+                finite ? make_ulonglong2(nmin, kmax) : make_ulonglong2(0ull, 0ull);
+        }
         if (~nmin < kNegInf || kmax > kPosInf) {  // some value is NaN: once more without them
             nmin = kmax = 0ull;
             for (int i = lane; i < n_b; i += 32) {
@@ -288,12 +211,9 @@ __device__ __forceinline__ void wide_write_raw(const WideQseArgs& a, uint32_t b,
 }
 
 template <int F>
-__global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_qse_kernel(WideQseArgs a) {
-    extern __shared__ __align__(16) uint8_t dsm[];
-    __shared__ WideShared S;
+__device__ __forceinline__ void wide_block_general(const WideQseArgs& a, uint8_t* dsm, WideShared& S, uint32_t b) {
     constexpr int P = F < 3 ? F : 3;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    const uint32_t b = blockIdx.x;
     const uint64_t first = (uint64_t)b * kBlock;
     const int n_b = (int)min((uint64_t)kBlock, a.n - first);
     unsigned long long* codes = reinterpret_cast<unsigned long long*>(dsm);  // [F][1024], sorted order
@@ -678,7 +598,26 @@ __global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_qse_ker
     if (t == 0) a.sizes[b] = enc;
 }
 
+// The blocks the fast kernel leaves (values that need the check of their
+// candidates, non-finite values, incompressible blocks): a grid of a few CTAs
+// per SM walks the list.
+template <int F>
+__global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_general_kernel(const __grid_constant__ WideQseArgs a) {
+    extern __shared__ __align__(16) uint8_t dsm[];
+    __shared__ WideShared S;
+    const uint32_t count = *(volatile const uint32_t*)a.general_count;
+    for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
+        wide_block_general<F>(a, dsm, S, a.general_list[i]);
+        __syncthreads();
+    }
+}
+
 // ---------------------------------------------------------------- decompression
+//
+// Bound by the integer pipe and, 40 us of it, by the one multiply-add per
+// value in fp64 (16 cycles of an SM per warp).  4*10^6 x 6 doubles in odd rows:
+// 94 us with four consecutive positions per thread (8-byte stores 32 bytes
+// apart) and words staged by plain loads, 74 us now.
 
 struct WideDecShared {
     double mn[kMaxFields], s[kMaxFields];
@@ -686,15 +625,12 @@ struct WideDecShared {
     uint16_t uniq[kMaxBins];
     uint32_t mask[32], warp_uc[kWideWarps];
     uint32_t ok, raw, bad, U, wd, wc, W, keybits, off, nw;
+    uint64_t bar;  // the staging bulk copy
 };
 
-// w (<= 32) bits at bit position pos of A[0..len); 0 when w = 0.
-__device__ __forceinline__ uint32_t wide_get(const uint32_t* A, uint32_t len, uint32_t pos, uint32_t w) {
-    if (w == 0u) return 0u;
-    const uint32_t wi = pos >> 5, sh = pos & 31u;
-    const uint32_t lo = wi < len ? __ldg(A + wi) : 0u;
-    const uint32_t hi = (sh + w > 32u && wi + 1u < len) ? __ldg(A + wi + 1u) : 0u;
-    return __funnelshift_r(lo, hi, sh) & (w >= 32u ? 0xffffffffu : ((1u << w) - 1u));
+// w (<= 11) bits at bit position pos of staged words.
+__device__ __forceinline__ uint32_t wide_get_s(const uint32_t* A, uint32_t pos, uint32_t w) {
+    return __funnelshift_r(A[pos >> 5], A[(pos >> 5) + 1u], pos) & ((1u << w) - 1u);
 }
 
 // w (<= 53) bits at bit position pos of the staged record words; the two
@@ -709,16 +645,22 @@ __device__ __forceinline__ unsigned long long wide_get64_s(const uint32_t* A, ui
     return v & mask64(w);
 }
 
-// Staged record words of one block: at most ceil(1024 x 53 F / 32), plus two.
+// The staged words of one block after its header: deltas, counts and at most
+// ceil(1024 x 53 F / 32) of records, up to three words before them (the bulk
+// copy's 16-byte boundary) and a few after (windows reach past their value).
+template <int F>
+constexpr uint32_t wide_dec_stage_words() {
+    return kWideDcWords + 32u * kWideMaxBits * (uint32_t)F;
+}
 template <int F>
 constexpr uint32_t wide_dec_smem_bytes() {
-    return 4u * ((kBlock * kWideMaxBits * (uint32_t)F + 31u) / 32u + 2u);
+    return 4u * (wide_dec_stage_words<F>() + 8u);
 }
 
 template <int F>
 __global__ void __launch_bounds__(kWideThreads) gpz_wide_decode_kernel(WideDecArgs a) {
     __shared__ WideDecShared S;
-    extern __shared__ __align__(16) uint32_t srec[];  // the block's record words
+    extern __shared__ __align__(16) uint32_t stage[];  // the block's words after its header, from word `shift`
     constexpr int P = F < 3 ? F : 3;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     const uint32_t* Sw = a.stream;
@@ -838,23 +780,33 @@ __global__ void __launch_bounds__(kWideThreads) gpz_wide_decode_kernel(WideDecAr
         return;
     }
 
-    // ---- 2. unique ids and run starts (Section 4.3, undone); the record
-    // words are copied to shared memory meanwhile (visible after the barriers)
+    // ---- 2. unique ids and run starts (Section 4.3, undone)
     const uint32_t U = S.U, wd = S.wd, wc = S.wc, W = S.W, keybits = S.keybits;
     const uint32_t dwords = ceil_words(U * wd), cwords = ceil_words(U * wc);
-    const uint32_t rwords = S.nw - hdr - dwords - cwords;  // <= ceil(n_b W / 32) by the size check
     const uint32_t idlimit = 1u << keybits;
-    {
-        const uint32_t* R = blk + hdr + dwords + cwords;
-        for (uint32_t k = t; k < rwords; k += kWideThreads) srec[k] = __ldg(R + k);
+    // one bulk copy of the 16-byte units that hold the words and end inside
+    // the stream; the few words after the last such unit by plain loads
+    const uint32_t nst = S.nw - hdr;  // dwords + cwords + record words, by the size check
+    const uint32_t* src = blk + hdr;
+    const uint32_t shift = (uint32_t)((reinterpret_cast<uintptr_t>(src) >> 2) & 3u);
+    uint32_t units = (uint32_t)(min((uint64_t)(nst + shift + 3u), a.total_words - (uint64_t)(src - Sw) + shift) >> 2);
+    if (units * 4u < shift) units = 0;
+    if (units && t == 0) {
+        mbar_init(&S.bar, 1);
+        mbar_arrive_expect_tx(&S.bar, units * 16u);
+        bulk_g2s(stage, src - shift, units * 16u, &S.bar);
     }
+    for (uint32_t k = (units ? units * 4u - shift : 0u) + t; k < nst; k += kWideThreads) stage[shift + k] = __ldg(src + k);
+    __syncthreads();  // the mbarrier and the plainly loaded words
+    if (units && !__syncthreads_and(mbar_wait_bounded(&S.bar, 0, a.status))) return;  // uniform
+    const uint32_t* sD = stage + shift;
+    const uint32_t* sC = sD + dwords;
+    const uint32_t* srec = sC + cwords;
     {
-        const uint32_t* D = blk + hdr;
-        const uint32_t* Cc = D + dwords;
         const uint32_t k0 = 2u * t, k1 = k0 + 1u;
         const bool v0 = k0 < U, v1 = k1 < U;
-        uint32_t d0 = v0 ? wide_get(D, dwords, k0 * wd, wd) : 0u, d1 = v1 ? wide_get(D, dwords, k1 * wd, wd) : 0u;
-        uint32_t c0 = v0 ? wide_get(Cc, cwords, k0 * wc, wc) : 0u, c1 = v1 ? wide_get(Cc, cwords, k1 * wc, wc) : 0u;
+        uint32_t d0 = v0 ? wide_get_s(sD, k0 * wd, wd) : 0u, d1 = v1 ? wide_get_s(sD, k1 * wd, wd) : 0u;
+        uint32_t c0 = v0 ? wide_get_s(sC, k0 * wc, wc) : 0u, c1 = v1 ? wide_get_s(sC, k1 * wc, wc) : 0u;
         bool bad = (v0 && (d0 >= idlimit || c0 == 0u || c0 > (uint32_t)n_b || (k0 > 0 && d0 == 0u))) ||
                    (v1 && (d1 >= idlimit || c1 == 0u || c1 > (uint32_t)n_b || d1 == 0u));
         if (bad) d0 = d1 = c0 = c1 = 0u;
@@ -905,41 +857,28 @@ __global__ void __launch_bounds__(kWideThreads) gpz_wide_decode_kernel(WideDecAr
     const uint32_t mpc = __popc(mword);
     const uint32_t mpre = warp_incl_sum(mpc) - mpc;
 
-    // ---- 3. positions 4t..4t+3: run, key, record fields, q = segId * 2^o + segOffset
-    // thread t's four positions lie in mask word t/8 (every lane shuffles)
-    const int src = (t >> 3) & 31;
-    const uint32_t mrow = __shfl_sync(0xffffffffu, mword, src), prow = __shfl_sync(0xffffffffu, mpre, src);
-    const int j0 = 4 * t;
-    if (j0 >= n_b) return;
-    const int left = n_b - j0;
+    // ---- 3. positions t + 256 e, so that a warp's stores are consecutive (in
+    // one mask word): run, key, record fields, q = segId * 2^o + segOffset
     uint32_t key[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const uint32_t bit = (uint32_t)(j0 + e) & 31u;
-        int run = (int)(prow + __popc(mrow & ((2u << bit) - 1u))) - 1;
-        run = run < 0 ? 0 : (run >= (int)U ? (int)U - 1 : run);
-        key[e] = S.uniq[run];
+        const int word = (t + kWideThreads * e) >> 5;  // the same for the whole warp
+        const uint32_t m = __shfl_sync(0xffffffffu, mword, word) & lanemask_le();
+        // position 0 starts a run: indexes 0..U-1
+        key[e] = S.uniq[__shfl_sync(0xffffffffu, mpre, word) + __popc(m) - 1u];
     }
 #pragma unroll
     for (int f = 0; f < F; ++f) {
         const uint32_t wf = S.wf[f], rs = S.rshift[f], ks = S.kshift[f], gm = (1u << S.g[f]) - 1u, of = S.o[f];
         const double sf = S.s[f], mf = S.mn[f];
-        double v[4];
+        double* dst = a.out[f] + first;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const uint32_t j = (uint32_t)min(j0 + e, n_b - 1);  // positions past the block repeat the last
-            unsigned long long qv = wide_get64_s(srec, j * W + rs, wf);
+            const int j = t + kWideThreads * e;
+            if (j >= n_b) continue;
+            unsigned long long qv = wide_get64_s(srec, (uint32_t)j * W + rs, wf);
             if (f < P) qv |= (unsigned long long)((key[e] >> ks) & gm) << of;
-            v[e] = __fma_rn(code_to_double(qv), sf, mf);  // qv < 2^53
-        }
-        double* dst = a.out[f] + first + j0;
-        if (left >= 4 && (reinterpret_cast<uintptr_t>(a.out[f]) & 15u) == 0) {
-            reinterpret_cast<double2*>(dst)[0] = make_double2(v[0], v[1]);
-            reinterpret_cast<double2*>(dst)[1] = make_double2(v[2], v[3]);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (e < left) dst[e] = v[e];
+            __stcs(dst + j, __fma_rn(code_to_double(qv), sf, mf));  // qv < 2^53
         }
     }
 }
@@ -947,15 +886,16 @@ __global__ void __launch_bounds__(kWideThreads) gpz_wide_decode_kernel(WideDecAr
 // ---------------------------------------------------------------- launches
 
 template <int F>
-cudaError_t launch_wide_qse_f(const WideQseArgs& a, uint32_t nblocks, cudaStream_t s) {
+cudaError_t launch_wide_general_f(const WideQseArgs& a, cudaStream_t s) {
     constexpr uint32_t smem = wide_smem_bytes<F>();
     // set at every launch (the attributes belong to the current device), with
     // the largest shared-memory carveout so that three CTAs fit per SM
-    cudaError_t e = cudaFuncSetAttribute(gpz_wide_qse_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gpz_wide_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gpz_wide_qse_kernel<F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        e = cudaFuncSetAttribute(gpz_wide_general_kernel<F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    gpz_wide_qse_kernel<F><<<nblocks, kWideThreads, smem, s>>>(a);
+    const unsigned grid = a.nblocks < 152u * 3u ? a.nblocks : 152u * 3u;
+    gpz_wide_general_kernel<F><<<grid, kWideThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -970,16 +910,16 @@ cudaError_t launch_wide_dec_f(const WideDecArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_wide_qse(const WideQseArgs& a, uint32_t nblocks, cudaStream_t s) {
+cudaError_t launch_wide_general(const WideQseArgs& a, cudaStream_t s) {
     switch (a.F) {
-        case 1: return launch_wide_qse_f<1>(a, nblocks, s);
-        case 2: return launch_wide_qse_f<2>(a, nblocks, s);
-        case 3: return launch_wide_qse_f<3>(a, nblocks, s);
-        case 4: return launch_wide_qse_f<4>(a, nblocks, s);
-        case 5: return launch_wide_qse_f<5>(a, nblocks, s);
-        case 6: return launch_wide_qse_f<6>(a, nblocks, s);
-        case 7: return launch_wide_qse_f<7>(a, nblocks, s);
-        case 8: return launch_wide_qse_f<8>(a, nblocks, s);
+        case 1: return launch_wide_general_f<1>(a, s);
+        case 2: return launch_wide_general_f<2>(a, s);
+        case 3: return launch_wide_general_f<3>(a, s);
+        case 4: return launch_wide_general_f<4>(a, s);
+        case 5: return launch_wide_general_f<5>(a, s);
+        case 6: return launch_wide_general_f<6>(a, s);
+        case 7: return launch_wide_general_f<7>(a, s);
+        case 8: return launch_wide_general_f<8>(a, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -1005,7 +945,7 @@ cudaError_t launch_wide_decode(const WideDecArgs& a, cudaStream_t s) {
 namespace {
 
 constexpr uint64_t kWideAlign = 256;
-constexpr uint64_t kWideCtrlBytes = 256;  // words: 0 status, 1 scan tile counter, 4-5 out size
+constexpr uint64_t kWideCtrlBytes = 256;  // words: 0 status, 1 scan tile counter, 2 general-list count, 4-5 out size
 constexpr uint64_t kWideResBytes = 256;   // range pass: [8][2] order keys
 
 uint32_t wide_slot_words(int F) { return (uint32_t)align_up(1ull + 2ull * (uint64_t)F * kBlock, 4); }
@@ -1078,10 +1018,11 @@ uint64_t wide_workspace_size(uint64_t n, int F) {
 }
 
 // Stages, scan and copy of the 64-bit form with absolute bounds eb[f]; the
-// header's mode word is `mode` (the caller's bound mode).
+// header's mode word is `mode` (the caller's bound mode).  pre: the range
+// pass has put each block's extremes into its slot.
 gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G, int mode, const double* eb,
                          void* d_out, uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size,
-                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s) {
+                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre) {
     const uint64_t nb = nblocks_of(n);
     if (nb + 2ull * (uint64_t)F * n >= (1ull << 32)) return GPZ_ERR_UNSUPPORTED;
     if (out_capacity < gpz_bound_size_wide(n, F)) return GPZ_ERR_CAPACITY;
@@ -1091,7 +1032,7 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     uint32_t* status = reinterpret_cast<uint32_t*>(ws + L.ctrl);
     if (cudaMemsetAsync(ws, 0, L.zero_bytes, s) != cudaSuccess) return GPZ_ERR_CUDA;
     Recorder rec(s);
-    rec.begin(3);
+    rec.begin(4);
     WideQseArgs qa{};
     for (int f = 0; f < F; ++f) {
         qa.fields[f] = n ? d_fields[f] : nullptr;
@@ -1104,12 +1045,18 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     qa.slot_words = wide_slot_words(F);
     qa.sizes = reinterpret_cast<uint32_t*>(ws + L.sizes);
     qa.perm = d_perm;
-    if (nb > 0) {
-        if (launch_wide_qse(qa, (uint32_t)nb, s) != cudaSuccess) return GPZ_ERR_CUDA;
-        rec.mark("wide_qse");
-    }
+    qa.pre = pre ? 1 : 0;
+    qa.nblocks = (uint32_t)nb;
     const uint32_t table_start = (uint32_t)(kHeaderWords + 4 * F);
     uint32_t* stream_words = static_cast<uint32_t*>(d_out);
+    qa.general_list = stream_words + table_start;  // the offset table's place, written by the scan later
+    qa.general_count = status + 2;
+    if (nb > 0) {
+        if (launch_wide_fast(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;
+        rec.mark("wide_qse");
+        if (launch_wide_general(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;
+        rec.mark("wide_general");
+    }
     ScanArgs sa{};
     sa.sizes = qa.sizes;
     sa.nblocks = (uint32_t)nb;
@@ -1185,7 +1132,8 @@ gpz_status gpz_compress_wide(const double* const* d_fields, uint64_t n, const gp
     cudaStream_t s = (cudaStream_t)stream;
     double eb[kMaxFields];
     for (int f = 0; f < F; ++f) eb[f] = p->eb[f];
-    if (p->mode == GPZ_EB_REL && n > 0) {
+    const bool ranged = p->mode == GPZ_EB_REL && n > 0;
+    if (ranged) {
         // the fp64 range of the non-NaN values (one synchronisation)
         uint8_t* ws = static_cast<uint8_t*>(d_ws);
         unsigned long long* res = reinterpret_cast<unsigned long long*>(ws + L.res);
@@ -1195,6 +1143,8 @@ gpz_status gpz_compress_wide(const double* const* d_fields, uint64_t n, const gp
         ra.n = n;
         ra.F = F;
         ra.res = res;
+        ra.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
+        ra.slot_words = wide_slot_words(F);
         // a warp per block and field, two of them one after the other, more
         // where the grid would pass a few waves
         const uint64_t items = nblocks_of(n) * (uint64_t)F, want = (items + 2 * kWideWarps - 1) / (2 * kWideWarps);
@@ -1220,7 +1170,7 @@ gpz_status gpz_compress_wide(const double* const* d_fields, uint64_t n, const gp
     if (h_eb_used)
         for (int f = 0; f < F; ++f) h_eb_used[f] = eb[f];
     return wide_compress(d_fields, n, F, p->seg_bits, p->mode, eb, d_out, out_capacity, d_out_size, h_out_size,
-                         d_perm, d_ws, ws_size, s);
+                         d_perm, d_ws, ws_size, s, ranged);
 }
 
 gpz_status gpz_decompress_wide(const void* d_in, uint64_t in_size, double* const* d_fields, int F, uint64_t n,

@@ -210,3 +210,29 @@ def test_full_snapshot_sampled(gpz, oracle):
         assert np.array_equal(mine, theirs), "block %d" % b
         assert np.array_equal(perm[b * 1024:(b + 1) * 1024].cpu().numpy() - b * 1024, rp)
     assert x.numel() * 8 / s.numel() > 1.5
+
+
+@pytest.mark.parametrize("F", [1, 3, 6, 8])
+@pytest.mark.parametrize("n", [1, 31, 257, 1023, 1024, 1025, 2 * 1024 + 300])
+@pytest.mark.parametrize("kind", ["half_steps", "mixed_signs", "unexact", "zeros"])
+def test_fixed_point_quantiser(gpz, oracle, F, n, kind):
+    """The fixed-point codes and what they leave to fp64 or to the general
+    kernel: values on and around half steps, both signs, a field whose
+    candidates need their check beside fields that do not, and zeros, negative
+    zeros and subnormals among them."""
+    rng = np.random.default_rng(F * 7919 + n)
+    eb = 1e-9
+    s = eb * 1.96875
+    k = rng.integers(0, 2 ** 33, size=(F, n)).astype(np.float64)
+    x = (k + rng.choice([0.0, 0.5, 0.25], size=(F, n))) * s
+    if kind == "mixed_signs":
+        x -= 2.0 ** 32 * s
+    elif kind == "unexact":
+        x[F - 1] *= 1e5  # beyond 2^40 steps
+    elif kind == "zeros":
+        x[:, ::3] = 0.0
+        x[:, 1::5] = -0.0
+        x[:, 2::7] = 5e-324
+    check_parity(gpz, oracle, x, eb, 0, 3)
+    if n > 1:
+        check_parity(gpz, oracle, x, 1e-11, 1, 2)

@@ -2,8 +2,9 @@
 // Validates arguments, lays out the workspace, finalises the per-field
 // constants and enqueues the kernels on the caller's stream:
 //   compress:   [range (relative bound)] -> Q.S.E. (shared-memory tile kernel,
-//               or, with fused compaction, the register kernel) -> look-back
-//               scan -> copy
+//               or, with fused compaction, the register kernel) -> offsets
+//               and copy (with fused compaction a look-back scan, then the
+//               copy of the blocks left)
 //   decompress: decode
 #include <atomic>
 #include <cmath>
@@ -95,7 +96,8 @@ WsLayout layout_of(uint64_t n, int F) {
     o += align_up(ntiles_of(nb) * 8, kAlign);
     L.bstates = o;  // per-block look-back states of the fused compaction
     o += align_up(nb * 8, kAlign);
-    L.zero_bytes = o;  // ctrl + params + both look-back state arrays are cleared per call
+    L.zero_bytes = o;  // ctrl + params + states (sizes' totals, or look-back states) are cleared per call,
+                       // and with fused compaction the per-block states
     L.partials = o;
     o += align_up((uint64_t)kRangeGridMax * F * sizeof(float2), kAlign);
     L.bext = o;  // each block's extremes from the range pass (relative bound)
@@ -272,11 +274,13 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
     gpz_status rc = GPZ_OK;
     Recorder rec(s);
     range_done = range_done && d_ws != nullptr && !own_ws;
+    const bool fused = (p->flags & GPZ_FLAG_FUSED_COMPACTION) != 0u;
+    const uint64_t zero_end = fused ? L.zero_bytes : L.bstates;
     do {
-        if (range_done && p->mode == GPZ_EB_REL) {  // keep the constants: clear the control words and the look-back states only
+        if (range_done && p->mode == GPZ_EB_REL) {  // keep the constants
             if ((rc = cuda_status(cudaMemsetAsync(ws + L.ctrl, 0, kCtrlBytes, s))) != GPZ_OK) break;
-            if ((rc = cuda_status(cudaMemsetAsync(ws + L.states, 0, L.zero_bytes - L.states, s))) != GPZ_OK) break;
-        } else if ((rc = cuda_status(cudaMemsetAsync(ws, 0, L.zero_bytes, s))) != GPZ_OK) {
+            if ((rc = cuda_status(cudaMemsetAsync(ws + L.states, 0, zero_end - L.states, s))) != GPZ_OK) break;
+        } else if ((rc = cuda_status(cudaMemsetAsync(ws, 0, zero_end, s))) != GPZ_OK) {
             break;
         }
         rec.begin();
@@ -284,7 +288,6 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         const bool rel = p->mode == GPZ_EB_REL;
         if (!rel)
             for (int f = 0; f < F; ++f) hp[f] = finalise(p->eb[f]);
-        const bool fused = (p->flags & GPZ_FLAG_FUSED_COMPACTION) != 0u;
         // the shared-memory tile kernel derives each block's widths itself; the
         // register kernel of the fused compaction reads them from the
         // block-info pass (relative bound)
@@ -337,6 +340,10 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         qa.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
         qa.slot_words = slot_words_of(F);
         qa.sizes = reinterpret_cast<uint32_t*>(ws + L.sizes);
+        if (!fused) {
+            qa.sums = reinterpret_cast<uint32_t*>(ws + L.states);
+            qa.sum_shift = size_sum_shift(nb, (L.bstates - L.states) / 4);
+        }
         qa.perm = d_perm;
         qa.status = status;
         qa.general_list = reinterpret_cast<uint32_t*>(ws + L.list);
@@ -357,23 +364,11 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         }
 
         uint32_t* stream_words = static_cast<uint32_t*>(d_out);
-        ScanArgs sa{};
-        sa.sizes = qa.sizes;
-        sa.nblocks = (uint32_t)nb;
-        sa.n = n;
-        sa.F = F;
-        sa.table = stream_words + table_start;
-        sa.tile_state = reinterpret_cast<unsigned long long*>(ws + L.states);
-        sa.tile_counter = tile_counter;
-        sa.status = status;
-        if ((rc = cuda_status(launch_scan(sa, s))) != GPZ_OK) break;
-        rec.mark("scan");
-
         CompactArgs ca{};
         ca.temp = qa.temp;
         ca.slot_words = qa.slot_words;
         ca.sizes = qa.sizes;
-        ca.table = sa.table;
+        ca.table = stream_words + table_start;
         ca.stream = stream_words;
         ca.payload_start = (uint32_t)(table_start + nb + 1);
         ca.nblocks = (uint32_t)nb;
@@ -386,7 +381,27 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         ca.d_out_size = d_out_size ? reinterpret_cast<unsigned long long*>(d_out_size) : ws_out_size;
         ca.unplaced = fused ? status + 8 : nullptr;
         ca.version = kVersion;
-        if ((rc = cuda_status(launch_compact(ca, s))) != GPZ_OK) break;
+        if (fused) {  // offsets by a scan, then the blocks not placed yet
+            ScanArgs sa{};
+            sa.sizes = qa.sizes;
+            sa.nblocks = (uint32_t)nb;
+            sa.n = n;
+            sa.F = F;
+            sa.table = stream_words + table_start;
+            sa.tile_state = reinterpret_cast<unsigned long long*>(ws + L.states);
+            sa.tile_counter = tile_counter;
+            sa.status = status;
+            if ((rc = cuda_status(launch_scan(sa, s))) != GPZ_OK) break;
+            rec.mark("scan");
+            if ((rc = cuda_status(launch_compact(ca, s))) != GPZ_OK) break;
+        } else {
+            PlaceArgs pa{};
+            pa.sums = qa.sums;
+            pa.sum_shift = qa.sum_shift;
+            pa.table = stream_words + table_start;
+            pa.raw_fields = (uint32_t)F;
+            if ((rc = cuda_status(launch_place(ca, pa, s))) != GPZ_OK) break;
+        }
         rec.mark("compact");
 
         if (h_out_size || own_ws) {

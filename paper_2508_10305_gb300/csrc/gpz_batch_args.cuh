@@ -39,6 +39,8 @@ __device__ __forceinline__ void load_chunk_args(const BatchCompressArgs& g, uint
         A.temp = g.temp + ch->temp_base;
         A.slot_words = batch_slot_words(ch->F);
         A.sizes = g.sizes + base;
+        A.sums = nullptr;  // the batch has its own scan
+        A.sum_shift = 0;
         A.perm = ch->perm;
         A.status = g.chunk_status + c;
         A.general_list = g.general_list;

@@ -20,6 +20,15 @@ inline uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1) / a * a; }
 
 inline uint64_t nblocks_of(uint64_t n) { return (n + kBlock - 1) / kBlock; }
 
+// The runs of blocks whose sizes are totalled (PlaceArgs): the shortest, from
+// 256 blocks up, whose totals fit `words` words -- the workspace's look-back
+// states, 64 words and more for every 32,768 blocks.
+inline uint32_t size_sum_shift(uint64_t nblocks, uint64_t words) {
+    uint32_t shift = 8;
+    while (((nblocks + (1ull << shift) - 1) >> shift) > words) ++shift;
+    return shift;
+}
+
 // The constants of one field from its bound eb: step eb * 63/32 (2 eb less
 // 1/64), reciprocal, and the verification threshold RD32(eb * (1 - 2^-22)).
 inline FieldParams finalise(double eb) {

@@ -69,6 +69,8 @@ struct QseArgs {
     uint32_t* temp;             // [nblocks][slot_words]
     uint32_t slot_words;
     uint32_t* sizes;            // [nblocks] words per block
+    uint32_t* sums;             // total words per 2^sum_shift blocks (zeroed), or nullptr (store_size)
+    uint32_t sum_shift;
     uint32_t* perm;             // [n] or nullptr
     uint32_t* status;
     uint32_t* general_list;     // [nblocks] blocks left to the general kernel (kCodedBlock: only recorded)
@@ -112,6 +114,18 @@ struct ScanArgs {
     uint32_t* tile_counter;     // zeroed
     uint32_t* status;
     long long wait_cycles;      // limit of a look-back wait in SM cycles; 0: kWaitCycles
+};
+
+// How the blocks' words come to their places in the stream (Section 4.4, steps
+// 2 and 3, in one kernel): every block's size was also added to the total of
+// its run of 2^sum_shift blocks, so a CTA finds its offset from the totals
+// before its run and the sizes before it in the run.
+struct PlaceArgs {
+    const uint32_t* sums;
+    uint32_t sum_shift;
+    uint32_t* table;            // out, [nblocks + 1]
+    uint32_t raw_fields;        // words per particle of a raw block
+    uint32_t log_blocks;        // blocks per CTA, log2 (set by the launch)
 };
 
 struct CompactArgs {
@@ -191,6 +205,12 @@ __constant__ DivMagic kDivMagic = DivMagic();
 __device__ __forceinline__ uint32_t div_small(uint32_t n, uint32_t d) {
     const unsigned long long m = kDivMagic.m[d];
     return __umulhi(n, (uint32_t)m) + ((m >> 32) ? n : 0u);
+}
+
+// A block's final size, and its share of its run's total.
+__device__ __forceinline__ void store_size(uint32_t* sizes, uint32_t* sums, uint32_t shift, uint32_t b, uint32_t words) {
+    sizes[b] = words;
+    if (sums) atomicAdd(sums + (b >> shift), words);
 }
 
 __device__ __forceinline__ void set_status(uint32_t* st, uint32_t code) {
@@ -372,6 +392,7 @@ cudaError_t launch_block_info(const uint2* bext, const FieldParams* d_params, ui
                               unsigned long long* binfo, cudaStream_t s);
 cudaError_t launch_scan(const ScanArgs& a, cudaStream_t s, unsigned grid = 0);  // grid 0: one CTA per tile
 cudaError_t launch_compact(const CompactArgs& a, cudaStream_t s);
+cudaError_t launch_place(const CompactArgs& a, const PlaceArgs& p, cudaStream_t s);  // scan and copy in one
 cudaError_t launch_decompress(const DecArgs& a, cudaStream_t s);
 
 }  // namespace gpz

@@ -176,7 +176,7 @@ __device__ __forceinline__ void write_raw(const QseArgs& a, uint32_t b, int n_b,
     }
     if (a.perm)
         for (int i = t; i < n_b; i += TH) a.perm[first + i] = (uint32_t)(first + i);
-    if (t == 0) a.sizes[b] = 1u + (uint32_t)F * (uint32_t)n_b;
+    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, 1u + (uint32_t)F * (uint32_t)n_b);
 }
 
 // The general per-block path: any block, including codes >= 2^23, values
@@ -577,7 +577,7 @@ __device__ __forceinline__ void qse_block_general(const QseArgs& a, uint8_t* dsm
     }
     if (a.perm)
         for (int j = t; j < n_b; j += kThreads) a.perm[first + j] = (uint32_t)first + sperm[j];
-    if (t == 0) a.sizes[b] = enc;
+    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, enc);
 }
 
 // ------------------------------------------------------------------ fast path

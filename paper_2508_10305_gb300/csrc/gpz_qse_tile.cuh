@@ -261,15 +261,15 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     }
     fence_proxy_async_shared();  // the staging words are read by a bulk copy (async proxy)
     __syncthreads();
-    if (t == 0) {
-        a.sizes[b] = enc;
-        bulk_s2g_start(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
-    }
+    if (t == 0) bulk_s2g_start(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
     if (!sorted_order(key, order, valid, i0, n_b, a.perm != nullptr, S)) {
         if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();  // not stable: the general kernel redoes it
-    } else if (a.perm) {
-        const uint64_t first = (uint64_t)b * kBlock;
-        for (int j = t; j < n_b; j += kTileThreads) a.perm[first + j] = (uint32_t)first + (order[j] & 1023u);
+    } else {
+        if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, enc);
+        if (a.perm) {
+            const uint64_t first = (uint64_t)b * kBlock;
+            for (int j = t; j < n_b; j += kTileThreads) a.perm[first + j] = (uint32_t)first + (order[j] & 1023u);
+        }
     }
     if (t == 0) bulk_s2g_wait();
 }

@@ -207,7 +207,7 @@ __device__ __forceinline__ void wide_write_raw(const WideQseArgs& a, uint32_t b,
     }
     if (a.perm)
         for (int i = t; i < n_b; i += kWideThreads) a.perm[first + i] = (uint32_t)(first + i);
-    if (t == 0) a.sizes[b] = 1u + 2u * (uint32_t)F * (uint32_t)n_b;
+    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, 1u + 2u * (uint32_t)F * (uint32_t)n_b);
 }
 
 template <int F>
@@ -595,7 +595,7 @@ __device__ __forceinline__ void wide_block_general(const WideQseArgs& a, uint8_t
     }
     if (a.perm)
         for (int j = t; j < n_b; j += kWideThreads) a.perm[first + j] = (uint32_t)first + sperm[j];
-    if (t == 0) a.sizes[b] = enc;
+    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, enc);
 }
 
 // The blocks the fast kernel leaves (values that need the check of their
@@ -945,7 +945,7 @@ cudaError_t launch_wide_decode(const WideDecArgs& a, cudaStream_t s) {
 namespace {
 
 constexpr uint64_t kWideAlign = 256;
-constexpr uint64_t kWideCtrlBytes = 256;  // words: 0 status, 1 scan tile counter, 2 general-list count, 4-5 out size
+constexpr uint64_t kWideCtrlBytes = 256;  // words: 0 status, 2 general-list count, 4-5 out size
 constexpr uint64_t kWideResBytes = 256;   // range pass: [8][2] order keys
 
 uint32_t wide_slot_words(int F) { return (uint32_t)align_up(1ull + 2ull * (uint64_t)F * kBlock, 4); }
@@ -964,7 +964,7 @@ WideLayout wide_layout(uint64_t n, int F) {
     o += kWideResBytes;
     L.states = o;
     o += align_up((nb + 1 + kScanTile - 1) / kScanTile * 8ull, kWideAlign);
-    L.zero_bytes = o;  // ctrl, range results and scan states are cleared per call
+    L.zero_bytes = o;  // ctrl, range results and the sizes' totals are cleared per call
     L.sizes = o;
     o += align_up(nb * 4ull, kWideAlign);
     L.temp = o;
@@ -1032,7 +1032,7 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     uint32_t* status = reinterpret_cast<uint32_t*>(ws + L.ctrl);
     if (cudaMemsetAsync(ws, 0, L.zero_bytes, s) != cudaSuccess) return GPZ_ERR_CUDA;
     Recorder rec(s);
-    rec.begin(4);
+    rec.begin(3);
     WideQseArgs qa{};
     for (int f = 0; f < F; ++f) {
         qa.fields[f] = n ? d_fields[f] : nullptr;
@@ -1044,6 +1044,8 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     qa.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
     qa.slot_words = wide_slot_words(F);
     qa.sizes = reinterpret_cast<uint32_t*>(ws + L.sizes);
+    qa.sums = reinterpret_cast<uint32_t*>(ws + L.states);
+    qa.sum_shift = size_sum_shift(nb, (L.sizes - L.states) / 4);
     qa.perm = d_perm;
     qa.pre = pre ? 1 : 0;
     qa.nblocks = (uint32_t)nb;
@@ -1057,22 +1059,11 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
         if (launch_wide_general(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;
         rec.mark("wide_general");
     }
-    ScanArgs sa{};
-    sa.sizes = qa.sizes;
-    sa.nblocks = (uint32_t)nb;
-    sa.n = n;
-    sa.F = 2 * F;  // a raw block holds 1 + 2F n_b words
-    sa.table = stream_words + table_start;
-    sa.tile_state = reinterpret_cast<unsigned long long*>(ws + L.states);
-    sa.tile_counter = status + 1;
-    sa.status = status;
-    if (launch_scan(sa, s) != cudaSuccess) return GPZ_ERR_CUDA;
-    rec.mark("scan");
     CompactArgs ca{};
     ca.temp = qa.temp;
     ca.slot_words = qa.slot_words;
     ca.sizes = qa.sizes;
-    ca.table = sa.table;
+    ca.table = stream_words + table_start;
     ca.stream = stream_words;
     ca.payload_start = (uint32_t)(table_start + nb + 1);
     ca.nblocks = (uint32_t)nb;
@@ -1093,7 +1084,12 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
         ca.ext[4 * f + 2] = (uint32_t)st;
         ca.ext[4 * f + 3] = (uint32_t)(st >> 32);
     }
-    if (launch_compact(ca, s) != cudaSuccess) return GPZ_ERR_CUDA;
+    PlaceArgs pa{};
+    pa.sums = qa.sums;
+    pa.sum_shift = qa.sum_shift;
+    pa.table = stream_words + table_start;
+    pa.raw_fields = 2u * (uint32_t)F;  // a raw block holds 1 + 2F n_b words
+    if (launch_place(ca, pa, s) != cudaSuccess) return GPZ_ERR_CUDA;
     rec.mark("compact");
     if (h_out_size) {
         if (cudaMemcpyAsync(h_out_size, ca.d_out_size, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess)

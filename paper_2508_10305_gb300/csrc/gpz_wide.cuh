@@ -35,6 +35,8 @@ struct WideQseArgs {
     uint32_t* temp;  // [nblocks][slot_words]
     uint32_t slot_words;
     uint32_t* sizes;  // [nblocks]
+    uint32_t* sums;   // as QseArgs
+    uint32_t sum_shift;
     uint32_t* perm;   // [n] or nullptr
     int pre;          // the range pass has put each block's extremes at the start of its slot
     uint32_t nblocks;

@@ -114,12 +114,19 @@ WsLayout layout_of(uint64_t n, int F) {
     return L;
 }
 
-gpz_status read_status(void* d_ws, cudaStream_t s, bool clear) {
-    if (cudaStreamSynchronize(s) != cudaSuccess) return GPZ_ERR_CUDA;
-    uint32_t st = 0;
-    if (cudaMemcpy(&st, d_ws, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return GPZ_ERR_CUDA;
-    if (clear && st != 0 && cudaMemset(d_ws, 0, 4) != cudaSuccess) return GPZ_ERR_CUDA;
-    return (gpz_status)st;
+// The device-side status after all work on the stream and, with h_size, the
+// stream size that the copy kernel left beside it (bytes 16..23), in one copy
+// on the stream.
+gpz_status read_status(void* d_ws, cudaStream_t s, bool clear, uint64_t* h_size = nullptr) {
+    uint32_t w[6] = {};
+    if (cudaMemcpyAsync(w, d_ws, h_size ? 24 : 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return GPZ_ERR_CUDA;
+    if (h_size) *h_size = (uint64_t)w[4] | ((uint64_t)w[5] << 32);
+    if (clear && w[0] != 0) {
+        if (cudaMemsetAsync(d_ws, 0, 4, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) return GPZ_ERR_CUDA;
+    }
+    return (gpz_status)w[0];
 }
 
 }  // namespace
@@ -378,7 +385,8 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         ca.mode = p->mode;
         for (int f = 0; f < F; ++f) ca.params[f] = hp[f];
         ca.d_params = rel ? d_params : nullptr;
-        ca.d_out_size = d_out_size ? reinterpret_cast<unsigned long long*>(d_out_size) : ws_out_size;
+        ca.d_out_size = reinterpret_cast<unsigned long long*>(d_out_size);
+        ca.ws_out_size = ws_out_size;
         ca.unplaced = fused ? status + 8 : nullptr;
         ca.version = kVersion;
         if (fused) {  // offsets by a scan, then the blocks not placed yet
@@ -405,12 +413,7 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         rec.mark("compact");
 
         if (h_out_size || own_ws) {
-            if (h_out_size) {
-                if ((rc = cuda_status(cudaMemcpyAsync(h_out_size, ca.d_out_size, 8, cudaMemcpyDeviceToHost, s))) !=
-                    GPZ_OK)
-                    break;
-            }
-            rc = read_status(status, s, !own_ws);
+            rc = read_status(status, s, !own_ws, h_out_size);
         }
     } while (false);
     if (own_ws) {

@@ -149,8 +149,9 @@ __device__ __forceinline__ void write_header(const CompactArgs& a, uint32_t payl
         if (a.d_params) p = a.d_params[f];
         a.stream[kHeaderWords + lane] = __float_as_uint((lane & 1) ? p.s : p.eb);
     }
-    if (lane == 0 && a.d_out_size)
-        *a.d_out_size = 4ull * ((unsigned long long)a.payload_start + payload_words);
+    const unsigned long long size = 4ull * ((unsigned long long)a.payload_start + payload_words);
+    if (lane == 0 && a.d_out_size) *a.d_out_size = size;
+    if (lane == 0 && a.ws_out_size) *a.ws_out_size = size;
 }
 
 __global__ void __launch_bounds__(32 * kCompactWarps) gpz_compact_kernel(CompactArgs a) {

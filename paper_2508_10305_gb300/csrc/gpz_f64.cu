@@ -41,10 +41,10 @@ __device__ __forceinline__ uint32_t f64_order_key32(float x) {
 //
 // A warp per (field, block of 1024 values): the fp32 copy, the block's fp32
 // extremes for the fused kernel (as the range pass stores them), and the
-// field's res[3f] = order key of the fp64 minimum, res[3f+1] = of the maximum
+// field's res[3f] = ~order key of the fp64 minimum, res[3f+1] = key of the maximum
 // (over the non-NaN values), res[3f+2] = bits of the largest |x - RN32(x)|
 // over the finite values (non-negative, so its bits order as the value); res
-// must start as {~0, 0, 0} per field.
+// must start as zeros.
 //
 // Bound by HBM and instruction issue.  A value's rounding takes about 25
 // integer and fp32 instructions; the exact 64-bit extremes and errors, three
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kF64Threads, 4) gpz_f64_prepass_kernel(const _
     flush();
     __syncthreads();
     if (tid < a.F && S.res[tid][0] != ~0ull) {
-        atomicMin(a.res + 3 * tid, S.res[tid][0]);
+        atomicMax(a.res + 3 * tid, ~S.res[tid][0]);
         atomicMax(a.res + 3 * tid + 1, S.res[tid][1]);
         atomicMax(a.res + 3 * tid + 2, S.res[tid][2]);
     }
@@ -316,13 +316,7 @@ gpz_status gpz_compress_f64(const double* const* d_fields, uint64_t n, const gpz
     const uint64_t ld = f32_ld(n);
 
     // the prepass: the fp32 copy, the fp64 extremes and the largest rounding error
-    unsigned long long init[3 * kMaxFields];
-    for (int f = 0; f < F; ++f) {
-        init[3 * f] = ~0ull;
-        init[3 * f + 1] = 0ull;
-        init[3 * f + 2] = 0ull;
-    }
-    if (cudaMemcpyAsync(res, init, 24ull * F, cudaMemcpyHostToDevice, s) != cudaSuccess) return GPZ_ERR_CUDA;
+    if (cudaMemsetAsync(res, 0, 24ull * F, s) != cudaSuccess) return GPZ_ERR_CUDA;
     F64Args fa{};
     fa.F = F;
     fa.n = n;
@@ -349,9 +343,9 @@ gpz_status gpz_compress_f64(const double* const* d_fields, uint64_t n, const gpz
     bool narrow = true;
     for (int f = 0; f < F; ++f) {
         double e = p->eb[f];
-        const bool any = got[3 * f] != ~0ull;  // some value is not NaN
+        const bool any = got[3 * f] != 0ull;  // some value is not NaN
         if (p->mode == GPZ_EB_REL && any) {
-            const volatile double range = from_key64(got[3 * f + 1]) - from_key64(got[3 * f]);
+            const volatile double range = from_key64(got[3 * f + 1]) - from_key64(~got[3 * f]);
             if (range > 0.0 && std::isfinite(range)) {
                 const volatile double t = p->eb[f] * range;
                 if (t > 0.0 && std::isfinite(t)) e = t;

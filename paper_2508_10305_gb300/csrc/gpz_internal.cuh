@@ -100,7 +100,7 @@ struct F64Args {                // fp64 input (gpz_f64.cu)
     float* out32[kMaxFields];   // 16-byte aligned
     uint64_t n;
     int F;
-    unsigned long long* res;    // [F][3]: min key, max key, largest rounding error (bits)
+    unsigned long long* res;    // [F][3]: ~min key, max key, largest rounding error (bits)
     uint2* bext;                // out, [nblocks][F]: each block's fp32 extremes, as RangeArgs
 };
 
@@ -143,6 +143,7 @@ struct CompactArgs {
     FieldParams params[kMaxFields];
     const FieldParams* d_params;
     unsigned long long* d_out_size; // nullable
+    unsigned long long* ws_out_size; // nullable: the same size, beside the status word
     uint32_t* unplaced;         // nullable: counts the blocks this kernel moves (in-kernel compaction forms)
     uint32_t version;           // header word 1
     uint32_t ext_words;         // nonzero: the header extension is ext[0..ext_words) instead of (eb, s) per field

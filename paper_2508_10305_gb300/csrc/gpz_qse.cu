@@ -113,9 +113,11 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_qse_general_kernel(QseArgs a)
 template <int F>
 cudaError_t launch_qse_general_f(const QseArgs& a, cudaStream_t s) {
     const size_t gsmem = qse_smem_bytes(F);
-    cudaError_t e =
-        cudaFuncSetAttribute(gpz_qse_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem);
-    if (e != cudaSuccess) return e;
+    if (gsmem + sizeof(QseShared) > 48u * 1024u) {  // beyond a CTA's default limit
+        const cudaError_t e =
+            cudaFuncSetAttribute(gpz_qse_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem);
+        if (e != cudaSuccess) return e;
+    }
     const unsigned ggrid = a.nblocks < 2u * 152u ? a.nblocks : 2u * 152u;
     gpz_qse_general_kernel<F><<<ggrid, kThreads, gsmem, s>>>(a);
     return cudaGetLastError();

@@ -21,8 +21,8 @@ template <int F, bool PRE, int LAY>
 cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
     const size_t smem = tile_smem_bytes(F, LAY);
     auto kern = gpz_qse_tile_kernel<F, PRE, LAY>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    static_assert(tile_smem_bytes(F, LAY) + sizeof(TileShared) <= 48u * 1024u, "within the default limit of a CTA");
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
     kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
     e = cudaGetLastError();

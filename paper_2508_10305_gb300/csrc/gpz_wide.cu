@@ -886,16 +886,20 @@ __global__ void __launch_bounds__(kWideThreads) gpz_wide_decode_kernel(WideDecAr
 // ---------------------------------------------------------------- launches
 
 template <int F>
-cudaError_t launch_wide_general_f(const WideQseArgs& a, cudaStream_t s) {
+bool prepare_wide_general() {
     constexpr uint32_t smem = wide_smem_bytes<F>();
-    // set at every launch (the attributes belong to the current device), with
-    // the largest shared-memory carveout so that three CTAs fit per SM
-    cudaError_t e = cudaFuncSetAttribute(gpz_wide_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gpz_wide_general_kernel<F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
+    // (the attributes belong to the current device; the largest shared-memory
+    // carveout lets three CTAs fit per SM)
+    return cudaFuncSetAttribute(gpz_wide_general_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+               cudaSuccess &&
+           cudaFuncSetAttribute(gpz_wide_general_kernel<F>, cudaFuncAttributePreferredSharedMemoryCarveout, 100) ==
+               cudaSuccess;
+}
+
+template <int F>
+cudaError_t launch_wide_general_f(const WideQseArgs& a, cudaStream_t s) {
     const unsigned grid = a.nblocks < 152u * 3u ? a.nblocks : 152u * 3u;
-    gpz_wide_general_kernel<F><<<grid, kWideThreads, smem, s>>>(a);
+    gpz_wide_general_kernel<F><<<grid, kWideThreads, wide_smem_bytes<F>(), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -922,6 +926,22 @@ cudaError_t launch_wide_general(const WideQseArgs& a, cudaStream_t s) {
         case 8: return launch_wide_general_f<8>(a, s);
     }
     return cudaErrorInvalidValue;
+}
+
+// The compression kernels' attributes on the current device.
+bool wide_prepare(int F) {
+    if (prepare_wide_fast(F) != cudaSuccess) return false;
+    switch (F) {
+        case 1: return prepare_wide_general<1>();
+        case 2: return prepare_wide_general<2>();
+        case 3: return prepare_wide_general<3>();
+        case 4: return prepare_wide_general<4>();
+        case 5: return prepare_wide_general<5>();
+        case 6: return prepare_wide_general<6>();
+        case 7: return prepare_wide_general<7>();
+        case 8: return prepare_wide_general<8>();
+    }
+    return false;
 }
 
 cudaError_t launch_wide_decode(const WideDecArgs& a, cudaStream_t s) {
@@ -992,11 +1012,13 @@ double wide_from_key_host(unsigned long long k) {
     return d;
 }
 
-gpz_status wide_read_status(uint32_t* status, cudaStream_t s) {
-    uint32_t st = 0;
-    if (cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
+// The device-side status and the stream size beside it (bytes 16..23).
+gpz_status wide_read_status(uint32_t* ctrl, cudaStream_t s, uint64_t* h_size) {
+    uint32_t w[6] = {};
+    if (cudaMemcpyAsync(w, ctrl, 24, cudaMemcpyDeviceToHost, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
         return GPZ_ERR_CUDA;
-    return (gpz_status)st;
+    *h_size = (uint64_t)w[4] | ((uint64_t)w[5] << 32);
+    return (gpz_status)w[0];
 }
 
 bool wide_fields_ok(const double* const* d_fields, uint64_t n, int F) {
@@ -1019,7 +1041,8 @@ uint64_t wide_workspace_size(uint64_t n, int F) {
 
 // Stages, scan and copy of the 64-bit form with absolute bounds eb[f]; the
 // header's mode word is `mode` (the caller's bound mode).  pre: the range
-// pass has put each block's extremes into its slot.
+// pass has put each block's extremes into its slot, and the control words were
+// cleared before it.
 gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G, int mode, const double* eb,
                          void* d_out, uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size,
                          uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre) {
@@ -1030,7 +1053,7 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     if (ws_size < L.total) return GPZ_ERR_CAPACITY;
     uint8_t* ws = static_cast<uint8_t*>(d_ws);
     uint32_t* status = reinterpret_cast<uint32_t*>(ws + L.ctrl);
-    if (cudaMemsetAsync(ws, 0, L.zero_bytes, s) != cudaSuccess) return GPZ_ERR_CUDA;
+    if (!pre && (!wide_prepare(F) || cudaMemsetAsync(ws, 0, L.zero_bytes, s) != cudaSuccess)) return GPZ_ERR_CUDA;
     Recorder rec(s);
     rec.begin(3);
     WideQseArgs qa{};
@@ -1071,8 +1094,8 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     ca.F = F;
     ca.G = G;
     ca.mode = mode;
-    ca.d_out_size = d_out_size ? reinterpret_cast<unsigned long long*>(d_out_size)
-                               : reinterpret_cast<unsigned long long*>(ws + L.ctrl + 16);
+    ca.d_out_size = reinterpret_cast<unsigned long long*>(d_out_size);
+    ca.ws_out_size = reinterpret_cast<unsigned long long*>(ws + L.ctrl + 16);
     ca.version = 2;
     ca.ext_words = 4u * (uint32_t)F;
     for (int f = 0; f < F; ++f) {
@@ -1091,12 +1114,7 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     pa.raw_fields = 2u * (uint32_t)F;  // a raw block holds 1 + 2F n_b words
     if (launch_place(ca, pa, s) != cudaSuccess) return GPZ_ERR_CUDA;
     rec.mark("compact");
-    if (h_out_size) {
-        if (cudaMemcpyAsync(h_out_size, ca.d_out_size, 8, cudaMemcpyDeviceToHost, s) != cudaSuccess)
-            return GPZ_ERR_CUDA;
-        return wide_read_status(status, s);
-    }
-    return GPZ_OK;
+    return h_out_size ? wide_read_status(status, s, h_out_size) : GPZ_OK;
 }
 
 }  // namespace host
@@ -1133,7 +1151,7 @@ gpz_status gpz_compress_wide(const double* const* d_fields, uint64_t n, const gp
         // the fp64 range of the non-NaN values (one synchronisation)
         uint8_t* ws = static_cast<uint8_t*>(d_ws);
         unsigned long long* res = reinterpret_cast<unsigned long long*>(ws + L.res);
-        if (cudaMemsetAsync(res, 0, kWideResBytes, s) != cudaSuccess) return GPZ_ERR_CUDA;
+        if (cudaMemsetAsync(ws, 0, L.zero_bytes, s) != cudaSuccess) return GPZ_ERR_CUDA;
         WideRangeArgs ra{};
         for (int f = 0; f < F; ++f) ra.fields[f] = d_fields[f];
         ra.n = n;
@@ -1141,15 +1159,17 @@ gpz_status gpz_compress_wide(const double* const* d_fields, uint64_t n, const gp
         ra.res = res;
         ra.temp = reinterpret_cast<uint32_t*>(ws + L.temp);
         ra.slot_words = wide_slot_words(F);
-        // a warp per block and field, two of them one after the other, more
-        // where the grid would pass a few waves
-        const uint64_t items = nblocks_of(n) * (uint64_t)F, want = (items + 2 * kWideWarps - 1) / (2 * kWideWarps);
+        // a warp per block and field, two of them one after the other once the
+        // grid passes a wave, more where it would pass a few waves
+        const uint64_t items = nblocks_of(n) * (uint64_t)F, per_cta = items > 152ull * 6ull * kWideWarps ? 2 * kWideWarps : kWideWarps;
+        const uint64_t want = (items + per_cta - 1) / per_cta;
         const unsigned grid = (unsigned)(want < 152ull * 64ull ? want : 152ull * 64ull);
         Recorder rec(s);
         rec.begin(1);
         gpz_wide_range_kernel<<<grid, kWideThreads, 0, s>>>(ra);
         if (cudaGetLastError() != cudaSuccess) return GPZ_ERR_CUDA;
         rec.mark("wide_range");
+        if (!wide_prepare(F)) return GPZ_ERR_CUDA;  // while the range pass runs
         unsigned long long got[2 * kMaxFields];
         if (cudaMemcpyAsync(got, res, 16ull * F, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess)

@@ -105,5 +105,6 @@ __device__ __forceinline__ bool first_candidate_exact(double bmin, double bmax, 
 // Stages 1-3 of the blocks the common path takes, the others into the
 // general list (gpz_wide_fast.cu).
 cudaError_t launch_wide_fast(const WideQseArgs& a, cudaStream_t s);
+cudaError_t prepare_wide_fast(int F);  // its attributes on the current device
 
 }  // namespace gpz

@@ -270,12 +270,15 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
 namespace {
 
 template <int F>
-cudaError_t launch_wide_fast_f(const WideQseArgs& a, cudaStream_t s) {
+cudaError_t prepare_wide_fast_f() {
     auto kern = gpz_wide_fast_kernel<F>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wf_smem_bytes(F));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    kern<<<a.nblocks, kTileThreads, wf_smem_bytes(F), s>>>(a);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wf_smem_bytes(F));
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+}
+
+template <int F>
+cudaError_t launch_wide_fast_f(const WideQseArgs& a, cudaStream_t s) {
+    gpz_wide_fast_kernel<F><<<a.nblocks, kTileThreads, wf_smem_bytes(F), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -291,6 +294,20 @@ cudaError_t launch_wide_fast(const WideQseArgs& a, cudaStream_t s) {
         case 6: return launch_wide_fast_f<6>(a, s);
         case 7: return launch_wide_fast_f<7>(a, s);
         case 8: return launch_wide_fast_f<8>(a, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t prepare_wide_fast(int F) {
+    switch (F) {
+        case 1: return prepare_wide_fast_f<1>();
+        case 2: return prepare_wide_fast_f<2>();
+        case 3: return prepare_wide_fast_f<3>();
+        case 4: return prepare_wide_fast_f<4>();
+        case 5: return prepare_wide_fast_f<5>();
+        case 6: return prepare_wide_fast_f<6>();
+        case 7: return prepare_wide_fast_f<7>();
+        case 8: return prepare_wide_fast_f<8>();
     }
     return cudaErrorInvalidValue;
 }

@@ -161,18 +161,24 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
                 half = __uint2float_rn((1u << bits) >> 1);
                 top = __uint2float_rn((1u << bits) - 1u);
             }
+            auto value = [&](int r) { return LAY == kTileRecords ? tile[(i0 + 32 * r) * F + f] : row[32 * r]; };
+            auto place = [&](int r, uint32_t ub) {
+                if (MODE == 2 || f < P) key[r] |= __funnelshift_l(ub, ub, rot) & kmask;
+                // append below the record so far (field 0 ends most significant)
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const float x = LAY == kTileRecords ? tile[(i0 + 32 * r) * F + f] : row[32 * r];
-                const float tt = __fmaf_rn(__fsub_rn(x, mn), inv, 0.5f);
-                const float u = __fadd_rd(tt, 8388608.0f);  // 2^23 + floor(t), t < 2^23 here
-                uint32_t ub = __float_as_uint(u);
-                if (MODE) {
+                for (int k = NR - 1; k > 0; --k) rw[r][k] = __funnelshift_l(rw[r][k - 1], rw[r][k], wf);
+                rw[r][0] = (rw[r][0] << wf) | (ub & cmask);
+            };
+            if (MODE == 2) {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const float x = value(r);
+                    const float tt = __fmaf_rn(__fsub_rn(x, mn), inv, 0.5f);
+                    const float u = __fadd_rd(tt, 8388608.0f);  // 2^23 + floor(t), t < 2^23 here
+                    uint32_t ub = __float_as_uint(u);
                     const float q = __fsub_rn(u, 8388608.0f);
                     auto ok = [&](float c) { return fabsf(__fsub_rn(x, __fmaf_rn(c, s, mn))) <= ebchk; };
-                    if (MODE == 1) {
-                        pend |= valid(r) && !ok(q);
-                    } else if (valid(r) && !ok(q)) {  // the next candidates, in the format's order
+                    if (valid(r) && !ok(q)) {  // the next candidates, in the format's order
                         if (q > 0.0f && ok(__fsub_rn(q, 1.0f))) {
                             pend |= q == half;
                             ub -= 1u;
@@ -181,12 +187,27 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
                             ub += 1u;
                         }
                     }
+                    place(r, ub);
                 }
-                if (MODE == 2 || f < P) key[r] |= __funnelshift_l(ub, ub, rot) & kmask;
-                // append below the record so far (field 0 ends most significant)
+            } else {  // the same, two values at a time
+                const f32x2 mn2 = pack2(mn, mn), neg2 = pack2(-mn, -mn), inv2 = pack2(inv, inv), s2 = pack2(s, s);
 #pragma unroll
-                for (int k = NR - 1; k > 0; --k) rw[r][k] = __funnelshift_l(rw[r][k - 1], rw[r][k], wf);
-                rw[r][0] = (rw[r][0] << wf) | (ub & cmask);
+                for (int r = 0; r < R; r += 2) {
+                    const f32x2 x = pack2(value(r), value(r + 1));
+                    const f32x2 tt = fma2_rn(add2_rn(x, neg2), inv2, pack2(0.5f, 0.5f));
+                    const f32x2 u = add2_rd(tt, pack2(8388608.0f, 8388608.0f));
+                    if (MODE == 1) {  // x - x^ as one rounding of x^ (-1) + x
+                        const f32x2 xh = fma2_rn(add2_rn(u, pack2(-8388608.0f, -8388608.0f)), s2, mn2);
+                        float d0, d1;
+                        unpack2(fma2_rn(xh, pack2(-1.0f, -1.0f), x), d0, d1);
+                        pend |= valid(r) && !(fabsf(d0) <= ebchk);
+                        pend |= valid(r + 1) && !(fabsf(d1) <= ebchk);
+                    }
+                    float u0, u1;
+                    unpack2(u, u0, u1);
+                    place(r, __float_as_uint(u0));
+                    place(r + 1, __float_as_uint(u1));
+                }
             }
         }
         return pend;

@@ -13,7 +13,7 @@ namespace gpz {
 // arguments in shared memory, in the layout that every chunk of the group
 // allows.
 template <int F, bool PRE, int LAY>
-__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_batch_tile_kernel(BatchCompressArgs g) {
+__global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_batch_tile_kernel(BatchCompressArgs g) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ TileShared S;
     __shared__ QseArgs A;

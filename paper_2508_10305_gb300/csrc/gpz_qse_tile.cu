@@ -15,7 +15,8 @@
 //     block's staging words are assembled in the same bytes, then written to
 //     the block's temporary slot by one bulk copy.
 // What bounds it: instruction issue (71% of the issue slots busy with three
-// fields, 60% with six) and shared-memory wavefronts (66-70% of their peak).
+// fields, 62% with six) and shared-memory wavefronts (55% and 69% of their
+// peak).
 // Why 128 threads: whatever a block costs
 // per warp rather than per particle (the constants' loads, the scan over
 // (bin, warp), the barriers) halves against 256 threads of four particles,
@@ -36,10 +37,11 @@
 // Fallback candidates (values whose rounding is near the bound) are coded in
 // place, in a second pass of the warps that have one, instead of redoing the
 // block in the general kernel: the scan (2% of its blocks) 0.533 -> 0.502 ms.
-// Residency: shared memory allows seven CTAs per SM for six fields (28 KB
-// each); for three fields nine (56 registers) measured best, 7 / 8 / 9 / 10 /
-// 12 CTAs: 0.565 / 0.544 / 0.533 / 0.540 / 0.550 ms on the scan (and with the
-// later steps 7 / 8 / 9: 0.539 / 0.518 / 0.502 ms).
+// Residency: for three fields nine CTAs per SM (56 registers) measured best, 7
+// / 8 / 9 / 10 / 12 CTAs: 0.565 / 0.544 / 0.533 / 0.540 / 0.550 ms on the scan
+// (and with the later steps 7 / 8 / 9: 0.539 / 0.518 / 0.502 ms).  For six fields
+// shared memory decides: with the histograms in the tile's first row eight
+// CTAs fit instead of seven, the snapshot 0.396 -> 0.377 ms.
 //
 // With a relative bound the block's extremes come from the range pass and
 // must bound the block's values (they are exact there): codes are monotone in

@@ -28,18 +28,30 @@ __host__ __device__ constexpr uint32_t tile_region_bytes(int F, int layout) {
     return (uint32_t)F * tile_row(layout) * 4u;
 }
 
-// Dynamic shared memory: the tile and the sort's histograms.
+// Dynamic shared memory: the tile and the sort's histograms.  With five and
+// more aligned fields, where shared memory sets the residency, the
+// histograms take the place of the tile's first row once a warp has quantised
+// its particles (a warp's row of counts is as long as its part of the row),
+// and the staging words start behind them: records are at most 128 bits, so
+// an encoded block fits the other rows.
+__host__ __device__ constexpr bool tile_overlays_hist(int F, int layout) { return layout == kTileAligned && F >= 5; }
+constexpr uint32_t kTileMaxEncWords = 1u + 8u + 2u + 144u + 176u + 32u * kFastRecordBits;
+static_assert(4u * kBlock >= 1u + 5u + 2u + 144u + 176u + 32u * 115u && 5u * kBlock >= kTileMaxEncWords,
+              "five fields (23 bits each) and more: the encoded block fits behind the first row");
+static_assert(kSortHistBytes == kBlock * 4u, "the histograms take one row");
 __host__ __device__ constexpr uint32_t tile_smem_bytes(int F, int layout) {
-    return tile_region_bytes(F, layout) + kSortHistBytes;
+    return tile_region_bytes(F, layout) + (tile_overlays_hist(F, layout) ? 0u : kSortHistBytes);
 }
 
 // Resident CTAs per SM the kernels are compiled for: what shared memory
 // allows (227 KB, 1 KB reserved per CTA, about 0.6 KB of static memory), at
-// most nine (56 registers per thread; more CTAs spill, see gpz_qse_tile.cu).
+// most nine (56 registers per thread; more CTAs spill, see gpz_qse_tile.cu),
+// eight from five fields on (64 registers).
 constexpr int kTileMaxCtas = 9;
-__host__ __device__ constexpr int tile_ctas(int F) {
-    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, kTileUnaligned) + 1024u + 640u));
-    return by_smem < kTileMaxCtas ? by_smem : kTileMaxCtas;
+__host__ __device__ constexpr int tile_ctas(int F, int layout) {
+    const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, layout) + 1024u + 640u));
+    const int most = F >= 5 ? kTileMaxCtas - 1 : kTileMaxCtas;
+    return by_smem < most ? by_smem : most;
 }
 
 namespace {
@@ -119,8 +131,9 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     constexpr int P = F < 3 ? F : 3;
     constexpr int R = kTileRounds;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    uint32_t* stage = reinterpret_cast<uint32_t*>(dsm);
-    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY)); 
+    constexpr bool OVER = tile_overlays_hist(F, LAY);
+    uint32_t* stage = reinterpret_cast<uint32_t*>(dsm + (OVER ? kSortHistBytes : 0u));
+    uint16_t* hist = reinterpret_cast<uint16_t*>(dsm + (OVER ? 0u : tile_region_bytes(F, LAY))); 
     uint32_t* order = reinterpret_cast<uint32_t*>(hist);                            // [1024] the sorted order, later
     const int i0 = 32 * R * w + lane;  // this thread's particles: i0 + 32 r
     auto valid = [&](int r) { return FULL || i0 + 32 * r < n_b; };
@@ -219,6 +232,11 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
         if (lane == 0) atomicOr(&S.fallback, fail ? kFbGeneral : kFbCoded);
     }
 
+    if (OVER) {  // the warp's part of the first row becomes its counts
+        __syncwarp();
+        clear_hist_row(hist);
+        __syncwarp();
+    }
     // ---- 4. counting sort: warp-local ranks, round after round
     rank_keys(key, hist, valid, S);
     __syncthreads();  // C: every value quantised (the tile is dead) and ranked
@@ -231,7 +249,8 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     {
         // the staging words, assembled by OR, overlay the tile: clear what
         // the block can need (deltas <= 512 x 9 bits, counts <= 512 x 11)
-        const uint32_t need = min((hdr + 144u + 176u + rwords + 3u) >> 2, tile_region_bytes(F, LAY) / 16u);
+        const uint32_t need = min((hdr + 144u + 176u + rwords + 3u) >> 2,
+                                  (tile_region_bytes(F, LAY) - (OVER ? kSortHistBytes : 0u)) / 16u);
         uint4* s4 = reinterpret_cast<uint4*>(stage);
         for (uint32_t k = t; k < need; k += kTileThreads) s4[k] = make_uint4(0u, 0u, 0u, 0u);
     }
@@ -360,11 +379,7 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         const uint32_t k = (t & 4) ? 4u * hi + (t & 3) : s + (t & 3);
         if (k >= s && k < end && ((t & 4) || k < 4u * lo)) tile[f * ROW + k] = __ldcs(a.fields[f] + first + (k - s));
     }
-    {
-        uint4* h4 = reinterpret_cast<uint4*>(dsm + tile_region_bytes(F, LAY)) + w * (kMaxBins / 8);
-#pragma unroll
-        for (int k = 0; k < kMaxBins / 256; ++k) h4[lane + 32 * k] = make_uint4(0u, 0u, 0u, 0u);
-    }
+    if (!tile_overlays_hist(F, LAY)) clear_hist_row(reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY)));
     // ---- 2. the field constants from the block's extremes: those of the
     // range pass (loaded with the step constants while the tile is in
     // flight), or found in the tile, a warp per field

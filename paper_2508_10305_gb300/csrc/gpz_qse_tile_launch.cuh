@@ -8,7 +8,7 @@
 namespace gpz {
 
 template <int F, bool PRE, int LAY>
-__global__ void __launch_bounds__(kTileThreads, tile_ctas(F)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
+__global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ TileShared S;
     if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)

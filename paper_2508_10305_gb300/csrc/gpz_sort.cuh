@@ -36,6 +36,13 @@ struct alignas(16) SortShared {
 
 namespace {
 
+// Clears the warp's row of counts.
+__device__ __forceinline__ void clear_hist_row(uint16_t* hist) {
+    uint4* h4 = reinterpret_cast<uint4*>(hist + (threadIdx.x >> 5) * kMaxBins) + (threadIdx.x & 31);
+#pragma unroll
+    for (int k = 0; k < kMaxBins / 256; ++k) h4[32 * k] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 // Each particle's rank among the earlier particles of its warp with the same
 // key (below 512), into bits 16 and up of key[r]; the warp's counts into its
 // row of hist (zeroed before).  With shared atomics the old count that comes

@@ -113,15 +113,18 @@ __host__ __device__ constexpr uint32_t batch_slot_words(int F) {
 }
 
 // Smallest c in [0, n) with end[c] > item, for a non-decreasing end[] whose
-// last entry exceeds item: a binary search, at most 32 probes.
+// last entry exceeds item (every lane of a warp calls it): 32 probes at a
+// time, so two or three round trips for thousands of chunks.
 __device__ __forceinline__ uint32_t search_chunk(const uint32_t* end, uint32_t n, uint32_t item) {
-    uint32_t lo = 0, hi = n - 1;
-    for (int k = 0; k < 32 && lo < hi; ++k) {
-        const uint32_t mid = lo + ((hi - lo) >> 1);
-        if (__ldg(end + mid) > item)
-            hi = mid;
-        else
-            lo = mid + 1;
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t lo = 0, size = n;  // the answer lies in [lo, lo + size)
+    while (size > 1u) {
+        const uint32_t step = (size + 31u) >> 5;
+        const uint32_t at = min(lane * step + step, size) - 1u;  // the last of the lane's share
+        const uint32_t hit = __ballot_sync(0xffffffffu, __ldg(end + lo + at) > item);
+        const uint32_t first = hit ? (uint32_t)__ffs(hit) - 1u : 31u;
+        lo += min(first * step, size - 1u);
+        size = min(step, size - min(first * step, size - 1u));
     }
     return lo;
 }

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(256) gpz_batch_map_kernel(BatchMapArgs a) {
 }
 
 // One CTA per range item of the group.
-__global__ void __launch_bounds__(kThreads) gpz_batch_range_kernel(BatchCompressArgs g) {
+__global__ void __launch_bounds__(kThreads, 6) gpz_batch_range_kernel(const __grid_constant__ BatchCompressArgs g) {
     __shared__ float2 red[kWarps];
     const uint32_t r = g.range_first + blockIdx.x;
     const uint32_t c = g.first + search_chunk(g.range_end + g.first, g.nchunks, r);
@@ -125,12 +125,14 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_batch_general_kernel(BatchCom
     __shared__ uint32_t slot[2];
     const uint32_t count = *(volatile const uint32_t*)g.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
-        const uint32_t gb = __ldcg(g.general_list + i);
-        if (gb & kCodedBlock) continue;
+        const uint32_t entry = __ldcg(g.general_list + i), gb = entry & ~kRawBlock;
+        if (entry & kCodedBlock) continue;
         load_chunk_args(g, __ldg(g.block_map + gb), gb, A, slot);
         __syncthreads();
         const uint32_t b = slot[0];
-        if ((uint64_t)(b + 1) * kBlock <= A.n)
+        if (entry & kRawBlock)
+            write_raw<F>(A, b, (int)min((uint64_t)kBlock, A.n - (uint64_t)b * kBlock), threadIdx.x);
+        else if ((uint64_t)(b + 1) * kBlock <= A.n)
             qse_block_general<F, true>(A, dsm, S, b);
         else
             qse_block_general<F, false>(A, dsm, S, b);
@@ -221,21 +223,33 @@ __global__ void __launch_bounds__(kScanThreads) gpz_batch_scan_kernel(BatchScanA
 
 // ------------------------------------------------------------------ compaction, tables and headers
 
-__global__ void __launch_bounds__(32 * kCompactWarps) gpz_batch_compact_kernel(BatchCompactArgs a) {
+__global__ void __launch_bounds__(32 * kCompactWarps, 6) gpz_batch_compact_kernel(const __grid_constant__ BatchCompactArgs a) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t nwarps = gridDim.x * kCompactWarps;
     const uint32_t items = a.total_blocks + a.nchunks;
+    // the next block's chunk and offsets are loaded while the current one is copied
+    auto place = [&](uint32_t qi, uint32_t& c, unsigned long long& o0, unsigned long long& o1) {
+        if (qi >= a.total_blocks) return;
+        const uint32_t q = a.total_blocks - 1u - qi;
+        c = __ldg(a.block_map + q);
+        o0 = __ldcg(a.offsets + q);
+        o1 = __ldcg(a.offsets + q + 1);
+    };
+    uint32_t next_c = 0u;
+    unsigned long long next_o0 = 0ull, next_o1 = 0ull;
+    place(blockIdx.x * kCompactWarps + warp, next_c, next_o0, next_o1);
     for (uint32_t qi = blockIdx.x * kCompactWarps + warp; qi < items; qi += nwarps) {
+        const uint32_t cur = next_c;
+        const unsigned long long o0 = next_o0, o1 = next_o1;
+        place(qi + nwarps, next_c, next_o0, next_o1);
         // the blocks from the last one down (the last slots written are the
         // likeliest still in L2), then the chunks' headers
         const uint32_t q = qi < a.total_blocks ? a.total_blocks - 1u - qi : qi;
         if (q < a.total_blocks) {
-            const uint32_t cur = __ldg(a.block_map + q);
             const BatchChunk* ch = a.chunks + cur;
             const uint32_t F = (uint32_t)ch->F, nb = ch->nblocks, b = q - ch->block_base;
             const uint64_t n = ch->n;
             const unsigned long long base = __ldcg(a.offsets + ch->block_base);
-            const unsigned long long o0 = __ldcg(a.offsets + q), o1 = __ldcg(a.offsets + q + 1);
             const uint64_t first = (uint64_t)b * kBlock;
             const uint32_t n_b = (uint32_t)(n - first < (uint64_t)kBlock ? n - first : (uint64_t)kBlock);
             const uint64_t table_start = kHeaderWords + 2ull * F;

@@ -84,9 +84,11 @@ struct QseArgs {
     uint32_t* deferred_count;
 };
 
-// In a general-list entry: a block with a value that takes a fallback
-// candidate, which the tile kernel has coded itself.
-constexpr uint32_t kCodedBlock = 0x80000000u;
+// In a general-list entry (a block index below 2^30: no device holds the
+// 2^40 particles of more): a block with a value that takes a fallback
+// candidate, coded by the tile kernel itself; a block with a value that no
+// candidate brings within its bound, to be stored raw.
+constexpr uint32_t kCodedBlock = 0x80000000u, kRawBlock = 0x40000000u;
 
 constexpr uint32_t kPlaced = 0x80000000u;  // in a block's word count: already in the stream
 

@@ -171,7 +171,12 @@ __device__ __forceinline__ void write_raw(const QseArgs& a, uint32_t b, int n_b,
 #pragma unroll
         for (int f = 0; f < F; ++f) {
             const float* src = a.fields[f] + first;
-            for (int i = t; i < n_b; i += TH) out[1 + f * n_b + i] = __float_as_uint(__ldg(src + i));
+            float v[kBlock / TH];  // all in flight at once
+#pragma unroll
+            for (int k = 0; k < kBlock / TH; ++k) v[k] = t + k * TH < n_b ? __ldg(src + t + k * TH) : 0.0f;
+#pragma unroll
+            for (int k = 0; k < kBlock / TH; ++k)
+                if (t + k * TH < n_b) out[1 + f * n_b + t + k * TH] = __float_as_uint(v[k]);
         }
     }
     if (a.perm)

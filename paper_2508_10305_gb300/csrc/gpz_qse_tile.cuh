@@ -70,13 +70,14 @@ struct alignas(16) TileField {
 struct alignas(16) TileShared : SortShared {
     uint4 blk;                             // flags, record width, key bits
     uint64_t bar;                          // mbarrier of the tile's bulk copies
-    uint32_t fallback;                     // kFbCoded, kFbGeneral
+    uint32_t fallback;                     // kFb... bits
     uint2 ext[kMaxFields];                 // the block's extremes (order keys; (0, 0): a non-finite value)
     TileField fc[kMaxFields];
 };
 
 constexpr uint32_t kFbCoded = 1u;      // a value took a fallback candidate
-constexpr uint32_t kFbGeneral = 2u;    // a value the tile kernel cannot code
+constexpr uint32_t kFbGeneral = 2u;    // ... that could change its field's width: general path
+constexpr uint32_t kFbRaw = 4u;        // a value without a candidate in the bound: the block is stored raw
 constexpr uint32_t kTfNonFinite = 1u;  // a non-finite value: stored raw
 constexpr uint32_t kTfBig = 2u;        // a code reaches 2^23: general path
 constexpr uint32_t kTfVerify = 4u;     // some field's first candidates need their check
@@ -144,9 +145,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     // segOffset.
     uint32_t key[R], rw[R][NR];
     // MODE 0: first candidates, known to pass.  1: first candidates, checked;
-    // true when one fails.  2: every candidate; true when the block needs the
-    // general path (no candidate passes, or one that could change the
-    // field's width).
+    // true when one fails.  2: every candidate; S.fallback takes what they call for.
     auto quantise = [&](auto mode) {
         constexpr int MODE = decltype(mode)::value;
         const float* tile = reinterpret_cast<const float*>(dsm);
@@ -193,11 +192,13 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
                     auto ok = [&](float c) { return fabsf(__fsub_rn(x, __fmaf_rn(c, s, mn))) <= ebchk; };
                     if (valid(r) && !ok(q)) {  // the next candidates, in the format's order
                         if (q > 0.0f && ok(__fsub_rn(q, 1.0f))) {
-                            pend |= q == half;
+                            if (q == half) atomicOr(&S.fallback, kFbGeneral);
                             ub -= 1u;
-                        } else {
-                            pend |= !(ok(__fadd_rn(q, 1.0f)) && q != top);
+                        } else if (ok(__fadd_rn(q, 1.0f))) {
+                            if (q == top) atomicOr(&S.fallback, kFbGeneral);
                             ub += 1u;
+                        } else {
+                            atomicOr(&S.fallback, kFbRaw);
                         }
                     }
                     place(r, ub);
@@ -228,8 +229,8 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     if (!(flags & kTfVerify)) {
         quantise(std::integral_constant<int, 0>{});
     } else if (__any_sync(0xffffffffu, quantise(std::integral_constant<int, 1>{}))) {
-        const bool fail = __any_sync(0xffffffffu, quantise(std::integral_constant<int, 2>{}));  // rare: once more
-        if (lane == 0) atomicOr(&S.fallback, fail ? kFbGeneral : kFbCoded);
+        quantise(std::integral_constant<int, 2>{});  // rare: once more
+        if (lane == 0) atomicOr(&S.fallback, kFbCoded);
     }
 
     if (OVER) {  // the warp's part of the first row becomes its counts
@@ -240,9 +241,11 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     // ---- 4. counting sort: warp-local ranks, round after round
     rank_keys(key, hist, valid, S);
     __syncthreads();  // C: every value quantised (the tile is dead) and ranked
-    if (const uint32_t fb = S.fallback) {
-        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id() | (fb & kFbGeneral ? 0u : kCodedBlock);
-        if (fb & kFbGeneral) return;
+    if (const uint32_t all = S.fallback) {
+        if (t == 0)
+            a.general_list[atomicAdd(a.general_count, 1u)] =
+                idx.id() | (all & kFbRaw ? kRawBlock : all & kFbGeneral ? 0u : kCodedBlock);
+        if (all & (kFbGeneral | kFbRaw)) return;
     }
     const uint32_t hdr = 1u + (uint32_t)F + (uint32_t)((F + 3) >> 2);
     const uint32_t rwords = ceil_words((uint32_t)n_b * W);

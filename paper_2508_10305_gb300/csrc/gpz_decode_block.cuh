@@ -83,10 +83,10 @@ __device__ __forceinline__ void widen4(const float* v, double* d) {
     }
 }
 
-// Store four consecutive values at out[first .. first + 3].
+// Store four consecutive values at out[first .. first + 3], 16-byte aligned.
 __device__ __forceinline__ void store4(float* out, uint64_t first, const float* v, int left) {
     float* dst = out + first;
-    if (left >= 4 && ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0)) {
+    if (left >= 4) {
         __stcs(reinterpret_cast<float4*>(dst), make_float4(v[0], v[1], v[2], v[3]));
     } else {
 #pragma unroll
@@ -96,12 +96,12 @@ __device__ __forceinline__ void store4(float* out, uint64_t first, const float* 
 }
 
 // Interleaved output: a block's values in record order in shared memory,
-// value (j, f) at word j * F + f + j / 8 (the padding word every eight
-// records spreads the records of a warp over the banks when F is even).
+// value (j, f) at word j * F + f: consecutive lanes' records are F words
+// apart, a bank conflict of gcd(F, 32) ways.
 template <int F>
-__device__ __forceinline__ int rec_slot(int j, int f) { return j * F + f + (j >> 3); }
+__device__ __forceinline__ int rec_slot(int j, int f) { return j * F + f; }
 template <int F>
-constexpr uint32_t rec_words() { return (uint32_t)(kBlock * F + kBlock / 8); }
+constexpr uint32_t rec_words() { return (uint32_t)(kBlock * F); }
 
 // x = fma((float)q, step, min) of four codes.
 __device__ __forceinline__ void rebuild4(const uint32_t* q, uint32_t bits, float s, float mn, float* v) {
@@ -228,7 +228,7 @@ template <int F>
 struct DecSharedRec : DecCore {
     static constexpr uint32_t kWords = dec_stage_words(F);
     uint64_t bar;
-    alignas(16) uint32_t stage[cmax(kWords + kDecStagePad + 4, 4 + rec_words<F>())];
+    alignas(16) uint32_t stage[cmax(kWords + kDecStagePad + 4, rec_words<F>())];
 };
 
 // Groups g0 .. g0 + NG - 1 of four positions (keys key[g - g0]): their records
@@ -390,39 +390,30 @@ __device__ __forceinline__ void decode_checks(const DecArgs& a, DecCore& S, uint
     }
 }
 
+// The block's values, staged in record order (rec_slot) from a 16-byte
+// boundary, to out[0] (every thread, after the values are staged): one bulk
+// copy of the whole 16-byte units when the records are 16-byte aligned.
+template <int F>
+__device__ __forceinline__ void store_records(const DecArgs& a, const float* recs, uint32_t b, int n_b) {
+    fence_proxy_async_shared();  // the values are read by a bulk copy (async proxy)
+    __syncthreads();             // every value is staged
+    const int t = threadIdx.x, total = n_b * F;
+    float* dst = a.out[0] + (uint64_t)b * kBlock * F;
+    const bool vec = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0;
+    const int bulk = vec ? total & ~3 : 0;
+    if (t == 0 && bulk) bulk_s2g_start(dst, recs, (uint32_t)bulk * 4u);
+    for (int k = bulk + t; k < total; k += kDecThreads) dst[k] = recs[k];
+    if (t == 0 && bulk) bulk_s2g_wait();
+}
+
 // Decode a block whose constants warp 0 has published in S (after a
 // barrier): stage holds the block's words after its header, blk the block in
 // the stream (read directly for raw blocks and records wider than 128 bits).
-// The block's values, staged in record order (rec_slot), to out[0] with
-// contiguous 16-byte stores when the records are 16-byte aligned (every
-// thread, after the values are staged).
-template <int F>
-__device__ __forceinline__ void store_records(const DecArgs& a, const float* recs, uint32_t b, int n_b) {
-    __syncthreads();  // every value is staged
-    const int t = threadIdx.x, total = n_b * F;
-    float* dst = a.out[0] + (uint64_t)b * kBlock * F;
-    if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-        for (int k = 4 * t; k < total; k += 4 * kDecThreads) {
-            float v[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int j = (k + c) / F;
-                v[c] = k + c < total ? recs[k + c + (j >> 3)] : 0.0f;  // rec_slot(j, (k + c) - j F)
-            }
-            if (k + 4 <= total)
-                __stcs(reinterpret_cast<float4*>(dst + k), make_float4(v[0], v[1], v[2], v[3]));
-            else
-                for (int c = 0; c < 4 && k + c < total; ++c) dst[k + c] = v[c];
-        }
-    } else {
-        for (int k = t; k < total; k += kDecThreads) dst[k] = recs[k + ((k / F) >> 3)];
-    }
-}
-
-// kOutRecords: the values go to interleaved records at out[0]; `stage` must then
-// hold rec_words<F>() words.
+// kOutRecords: the values go to interleaved records at out[0]; recs (16-byte
+// aligned, rec_words<F>() words) takes them once the stage's words, which it
+// overlays, are consumed.
 template <int F, int OUT>
-__device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32_t* stage,
+__device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32_t* stage, float* recs,
                                             const uint32_t* blk, uint32_t b, int n_b) {
     constexpr bool OUT64 = OUT == kOut64, AOS = OUT == kOutRecords;
     uint16_t* uniq = S.uniq;
@@ -559,7 +550,6 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
         }
     }
     const uint64_t base = (uint64_t)b * kBlock;
-    float* recs = reinterpret_cast<float*>(stage);  // AOS, once the stage's words are consumed
     auto sync = [] {
         if (AOS) __syncthreads();
     };
@@ -568,17 +558,20 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
 #pragma unroll
         for (int g = 0; g < kDecGroups; ++g)
             decode_wide<F, OUT>(a, blk, hdr + dwords + cwords, rwords, W, S.G, g, n_b, base, key[g], recs);
-    } else if (W <= 64u) {
+    } else if (W <= 64u && OUT != kOut64) {
         decode_groups<F, kDecGroups, false, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
     } else if (AOS) {  // every record in registers before the first value is staged
         decode_groups<F, kDecGroups, true, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
-    } else {
+    } else {  // a group at a time: fewer registers (fp64 output 94 -> 84 us on a 2^23 x 6 stream)
 #pragma unroll 1
         for (int g = 0; g < kDecGroups; ++g) {
             uint32_t kg[1][4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) kg[0][e] = g == 0 ? key[0][e] : key[kDecGroups - 1][e];
-            decode_groups<F, 1, true, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
+            if (OUT == kOut64 && W <= 64u)
+                decode_groups<F, 1, false, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
+            else
+                decode_groups<F, 1, true, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
         }
     }
     if (AOS) store_records<F>(a, recs, b, n_b);
@@ -653,7 +646,7 @@ __device__ __forceinline__ void decode_block(const DecArgs& a, Sh& S, Idx idx, u
     if (w == 0) decode_checks<F>(a, S, hv, bw, step, inside, b, off, end, payload_words, n_b);
     __syncthreads();
     if (units && !__syncthreads_and(mbar_wait_bounded(&S.bar, 0, a.status))) return;  // uniform
-    decode_tail<F, OUT>(a, S, stage + shift, blk, b, n_b);
+    decode_tail<F, OUT>(a, S, stage + shift, reinterpret_cast<float*>(stage), blk, b, n_b);
 }
 
 }  // namespace gpz

@@ -7,14 +7,28 @@
 
 namespace gpz {
 
+// The last block first: a ragged one runs code of its own (in the caches of
+// no SM yet) and would otherwise end the kernel alone; 1.7*10^7 x 3 records
+// with 43 in the last block: 102 -> 93 us.
+struct LastFirst {
+    __device__ __forceinline__ uint32_t b() const { return blockIdx.x ? blockIdx.x - 1u : gridDim.x - 1u; }  // block within its array
+    __device__ __forceinline__ uint32_t id() const { return b(); }  // entry for the general list
+};
+
+struct LastBlock {
+    __device__ __forceinline__ uint32_t b() const { return gridDim.x - 1u; }
+    __device__ __forceinline__ uint32_t id() const { return b(); }
+};
+
 template <int F, bool PRE, int LAY>
 __global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ TileShared S;
-    if ((uint64_t)(blockIdx.x + 1) * kBlock <= a.n)
-        qse_block_tile<F, true, PRE, LAY>(a, dsm, S, GridBlock{});
+    // the grid's last block may be ragged
+    if (blockIdx.x != 0u || (uint64_t)gridDim.x * kBlock == a.n)
+        qse_block_tile<F, true, PRE, LAY>(a, dsm, S, LastFirst{});
     else
-        qse_block_tile<F, false, PRE, LAY>(a, dsm, S, GridBlock{});
+        qse_block_tile<F, false, PRE, LAY>(a, dsm, S, LastBlock{});
 }
 
 template <int F, bool PRE, int LAY>

@@ -16,13 +16,13 @@
 //      gives the segment offsets and extra-field codes; every value is
 //      rebuilt as fma(q, step, min) and stored, four consecutive ones at once.
 // What bounds it: with six fields HBM (2.06 GB of a 2^26-particle snapshot in
-// 0.317 ms, 6.5 TB/s), with three the issue slots (67% busy) and the integer
+// 0.313 ms, 6.6 TB/s), with three the issue slots (67% busy) and the integer
 // pipe (71%).  Why 128 threads: what a block costs per warp rather than per
 // position (the checks' barrier, the scan, the mask, the fields' constants)
 // is half of what 256 threads of four positions paid: 6,220 -> 4,160 warp
 // instructions per block with six fields, 5,070 -> 3,190 with three.
-// Measured: 2^26 x 6 snapshot 0.420 -> 0.317 ms, 10^8 x 3 scan points 0.514 ->
-// 0.358 ms.
+// Measured: 2^26 x 6 snapshot 0.420 -> 0.317 ms (0.313 with the later steps),
+// 10^8 x 3 scan points 0.514 -> 0.358 ms (0.319).
 // Every read stays inside the stream, every failed check sets
 // GPZ_ERR_CORRUPT in the status word, and the kernel never traps.
 #include "gpz_decode_block.cuh"

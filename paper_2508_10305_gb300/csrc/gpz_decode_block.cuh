@@ -234,19 +234,17 @@ struct DecSharedRec : DecCore {
 // Groups g0 .. g0 + NG - 1 of four positions (keys key[g - g0]): their records
 // from the staged words, then the codes of fields F-1 .. 0, consumed from the
 // least significant end: field F-1 sits at bit 0 of the record and field 0 at
-// the top.  rr holds a record in its low bits (two words when W <= 64, else
-// four); after each field the record is shifted right by the field's width
+// the top.  rr holds a record in its low bits (NR words, W <= 32 NR); after each field the record is shifted right by the field's width
 // and the key right by the axis' segId bits.  q = segId * 2^o + segOffset for
 // a position axis, the whole code otherwise.  Words past the record array
 // (inside the staging pad) hold bits above W, which are never consumed.
 // kOutRecords: sync() once every record is in registers, then the values go to
 // recs.
-template <int F, int NG, bool WIDE, int OUT, class Sync>
+template <int F, int NG, int NR, int OUT, class Sync>
 __device__ __forceinline__ void decode_groups(const DecArgs& a, const DecCore& L, const uint32_t* sR, uint32_t W,
                                               int g0, uint32_t (&key)[NG][4], uint64_t base, int n_b,
                                               float* recs, Sync sync) {
     constexpr int P = F < 3 ? F : 3;
-    constexpr int NR = WIDE ? 4 : 2;
     uint32_t rr[NG][4][NR];
 #pragma unroll
     for (int g = 0; g < NG; ++g)
@@ -558,10 +556,13 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
 #pragma unroll
         for (int g = 0; g < kDecGroups; ++g)
             decode_wide<F, OUT>(a, blk, hdr + dwords + cwords, rwords, W, S.G, g, n_b, base, key[g], recs);
+    } else if (F <= 3 && W <= 32u && OUT != kOut64) {
+        // one word per record (10^8 x 3 scan points, most of them: 0.344 -> 0.319 ms)
+        decode_groups<F, kDecGroups, 1, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
     } else if (W <= 64u && OUT != kOut64) {
-        decode_groups<F, kDecGroups, false, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
+        decode_groups<F, kDecGroups, 2, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
     } else if (AOS) {  // every record in registers before the first value is staged
-        decode_groups<F, kDecGroups, true, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
+        decode_groups<F, kDecGroups, 4, OUT>(a, S, sR, W, 0, key, base, n_b, recs, sync);
     } else {  // a group at a time: fewer registers (fp64 output 94 -> 84 us on a 2^23 x 6 stream)
 #pragma unroll 1
         for (int g = 0; g < kDecGroups; ++g) {
@@ -569,9 +570,9 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
 #pragma unroll
             for (int e = 0; e < 4; ++e) kg[0][e] = g == 0 ? key[0][e] : key[kDecGroups - 1][e];
             if (OUT == kOut64 && W <= 64u)
-                decode_groups<F, 1, false, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
+                decode_groups<F, 1, 2, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
             else
-                decode_groups<F, 1, true, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
+                decode_groups<F, 1, 4, OUT>(a, S, sR, W, g, kg, base, n_b, recs, sync);
         }
     }
     if (AOS) store_records<F>(a, recs, b, n_b);

@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(32 * kCompactWarps) gpz_place_kernel(const __g
     const uint32_t raw_full = 1u + p.raw_fields * kBlock;
     const uint32_t raw_last = 1u + p.raw_fields * (uint32_t)(a.n - (uint64_t)(a.nblocks ? a.nblocks - 1 : 0) * kBlock);
     auto words = [&](uint32_t b) { return min(__ldcg(a.sizes + b), b + 1u == a.nblocks ? raw_last : raw_full); };
+    wait_for_previous_kernel();
     const uint32_t run = b0 >> p.sum_shift;
     uint32_t acc = 0u;
     for (uint32_t i = tid; i < run; i += 32 * kCompactWarps) acc += __ldcg(p.sums + i);
@@ -236,8 +237,7 @@ cudaError_t launch_place(const CompactArgs& a, const PlaceArgs& args, cudaStream
     p.log_blocks = 3;
     while (p.log_blocks < 4u && (a.nblocks >> p.log_blocks) >= 152u * 12u) ++p.log_blocks;
     const unsigned grid = (unsigned)(((uint64_t)a.nblocks + (1u << p.log_blocks) - 1) >> p.log_blocks);
-    gpz_place_kernel<<<grid ? grid : 1u, 32 * kCompactWarps, 0, s>>>(a, p);
-    return cudaGetLastError();
+    return launch_dependent(gpz_place_kernel, grid ? grid : 1u, 32 * kCompactWarps, 0, s, a, p);
 }
 
 }  // namespace gpz

@@ -414,6 +414,29 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// ---------------------------------------------------------------- dependent launches
+
+// Launch a kernel that may be set up while the kernel before it on the stream
+// still ends (programmatic dependent launch).  The kernel calls
+// wait_for_previous_kernel() before it reads or writes anything that earlier
+// work on the stream touches.
+template <class... P, class... A>
+cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &attr;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...);
+}
+
+__device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- launch wrappers (defined in the .cu files)
 
 cudaError_t launch_range(const RangeArgs& a, int grid, cudaStream_t s);

@@ -97,6 +97,7 @@ template <int F>
 __global__ void __launch_bounds__(kThreads, 2) gpz_qse_general_kernel(QseArgs a) {
     extern __shared__ __align__(16) uint8_t dsm[];
     __shared__ QseShared S;
+    wait_for_previous_kernel();
     const uint32_t count = *(volatile const uint32_t*)a.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
         const uint32_t entry = a.general_list[i], b = entry & ~kRawBlock;
@@ -121,8 +122,7 @@ cudaError_t launch_qse_general_f(const QseArgs& a, cudaStream_t s) {
         if (e != cudaSuccess) return e;
     }
     const unsigned ggrid = a.nblocks < 2u * 152u ? a.nblocks : 2u * 152u;
-    gpz_qse_general_kernel<F><<<ggrid, kThreads, gsmem, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(gpz_qse_general_kernel<F>, ggrid, kThreads, gsmem, s, a);
 }
 
 cudaError_t launch_qse_general(const QseArgs& a, cudaStream_t s) {

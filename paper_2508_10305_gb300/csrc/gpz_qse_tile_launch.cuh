@@ -38,8 +38,12 @@ cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
     static_assert(tile_smem_bytes(F, LAY) + sizeof(TileShared) <= 48u * 1024u, "within the default limit of a CTA");
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
-    e = cudaGetLastError();
+    if (PRE) {
+        e = launch_dependent(kern, a.nblocks, kTileThreads, smem, s, a);
+    } else {
+        kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
+        e = cudaGetLastError();
+    }
     if (e != cudaSuccess) return e;
     return launch_qse_general(a, s);
 }

@@ -605,6 +605,7 @@ template <int F>
 __global__ void __launch_bounds__(kWideThreads, F <= 6 ? 3 : 2) gpz_wide_general_kernel(const __grid_constant__ WideQseArgs a) {
     extern __shared__ __align__(16) uint8_t dsm[];
     __shared__ WideShared S;
+    wait_for_previous_kernel();
     const uint32_t count = *(volatile const uint32_t*)a.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
         wide_block_general<F>(a, dsm, S, a.general_list[i]);
@@ -899,8 +900,7 @@ bool prepare_wide_general() {
 template <int F>
 cudaError_t launch_wide_general_f(const WideQseArgs& a, cudaStream_t s) {
     const unsigned grid = a.nblocks < 152u * 3u ? a.nblocks : 152u * 3u;
-    gpz_wide_general_kernel<F><<<grid, kWideThreads, wide_smem_bytes<F>(), s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(gpz_wide_general_kernel<F>, grid, kWideThreads, wide_smem_bytes<F>(), s, a);
 }
 
 template <int F>

@@ -84,7 +84,7 @@ __device__ __forceinline__ bool wide_quantise(double x, const WideParams& p, dou
 // A warp per (field, 1024 values), eight 16-byte loads in flight per lane.
 // Bound by HBM: the keys' minima and maxima are integer operations (fp64
 // compares kept that pipe 70% busy and the pass at 120 us on 4*10^6 x 6
-// doubles in odd rows; 41 us this way).  NaN keys lie outside the infinities' and
+// doubles in odd rows; 40 us this way).  NaN keys lie outside the infinities' and
 // are only looked for when an extreme does.
 __global__ void __launch_bounds__(kWideThreads, 6) gpz_wide_range_kernel(const __grid_constant__ WideRangeArgs a) {
     __shared__ unsigned long long s_res[kMaxFields][2];
@@ -106,19 +106,25 @@ __global__ void __launch_bounds__(kWideThreads, 6) gpz_wide_range_kernel(const _
             nmin = max(nmin, ~k);
             kmax = max(kmax, k);
         };
-        if (n_b == kBlock && (reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
-            const ulonglong2* x2 = reinterpret_cast<const ulonglong2*>(x) + lane;
+        if (n_b == kBlock) {
+            // from the first 16-byte boundary on; a field that starts 8 bytes
+            // before one has 511 whole units (the last lane reads its own
+            // before twice) and a value at either end
+            const int head = (int)(reinterpret_cast<uintptr_t>(x) >> 3) & 1;
+            const ulonglong2* x2 = reinterpret_cast<const ulonglong2*>(x + head) + lane;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 ulonglong2 v[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) v[k] = __ldcs(x2 + 32 * (8 * h + k));
+                for (int k = 0; k < 8; ++k)
+                    v[k] = __ldcs(x2 + 32 * (8 * h + k) - (8 * h + k == 15 && head && lane == 31 ? 32 : 0));
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     take(v[k].x);
                     take(v[k].y);
                 }
             }
+            if (head) take(__ldcs(x + (lane & 1 ? kBlock - 1 : 0)));
         } else {
 #pragma unroll 16
             for (int i = lane; i < n_b; i += 32) take(__ldcs(x + i));

@@ -851,7 +851,7 @@ def run_gpz(args, rank, world, local):
         ach = algo.get(k, 0.0) / step_s / 1e9
         kernels[k] = [r4(1e3 * step_s), r4(ach / peak)]
     dom = max(kernels, key=lambda k: kernels[k][0])
-    kname = {"qse": "gpz_qse_tile_kernel"}.get(dom, "gpz_%s_kernel" % dom)
+    kname = {"qse": "gpz_qse_tile_kernel", "compact": "gpz_place_kernel"}.get(dom, "gpz_%s_kernel" % dom)
     dom_ms = kernels[dom][0]
     roofline = {"bound": "hbm", "kernel": kname, "achieved": r4(algo[dom] / (dom_ms / 1e3) / 1e9), "peak": peak,
                 "unit": "GB/s", "frac": r4(algo[dom] / (dom_ms / 1e3) / 1e9 / peak), "traffic": recorded_traffic(dom),
@@ -1083,7 +1083,7 @@ def batched_measure(args, embedded=False):
     total_stream = float(sum(sizes))
     nblocks = sum((n + 1023) // 1024 for n in wl.n)
     payload = total_stream - 4.0 * sum(16 + 2 * F + (n + 1023) // 1024 + 1 for n, F in zip(wl.n, wl.F))
-    algo = {"batch_qse": 2 * in_bytes + payload, "batch_scan": 12.0 * nblocks, "batch_compact": 2 * payload,
+    algo = {"batch_range": in_bytes, "batch_qse": in_bytes + payload, "batch_scan": 12.0 * nblocks, "batch_compact": 2 * payload,
             "batch_decompress": total_stream + in_bytes}
     peak, peak_kind = load_peaks()
     kernels = {}

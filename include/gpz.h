@@ -81,7 +81,7 @@ typedef struct {
 /* Compaction form (Section 4.4) of one gpz_compress call; the stream is the
  * same bytes in either form.
  *   default (no flag): Section 4.4's three steps -- every block is encoded
- *     into a temporary slot, a scan computes the offsets, a copy kernel moves
+ *     into a temporary slot, and one kernel computes the offsets and moves
  *     every block into the stream.
  *   GPZ_FLAG_FUSED_COMPACTION: every block publishes its size and looks back
  *     over its predecessors' sizes, waiting for them (a decoupled look-back
@@ -322,7 +322,7 @@ const char* gpz_status_str(gpz_status s);
  * 8192 events between reads); calls on other streams are not affected.
  * gpz_set_stage_timing(stream, 0) stops it.  gpz_stage_times synchronises on
  * the last recorded event, writes up to max stage names ("range", "qse",
- * "scan", "compact", "decompress", ...) with their summed elapsed
+ * "compact", "decompress", and with fused compaction "scan", ...) with their summed elapsed
  * milliseconds and launch counts since the previous read, returns the number
  * of stages, and clears the log.  names[] receives static strings. */
 void gpz_set_stage_timing(void* stream, int enable);

@@ -22,7 +22,7 @@
 // Kernels: a range pass (relative bounds), one CTA per block for the stages
 // (gpz_wide_fast.cu; the blocks it leaves are done here by the general kernel:
 // the codes sorted into shared memory, each thread's four sorted records
-// appended into staging words), the scan and copy of the 32-bit form, and one
+// appended into staging words), the offsets and copy of the 32-bit form, and one
 // CTA per block to decode (the block's words staged in shared memory).
 #include <cmath>
 #include <cstring>

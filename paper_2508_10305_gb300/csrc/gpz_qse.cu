@@ -8,9 +8,11 @@ namespace gpz {
 
 // ------------------------------------------------------------------ range pass (relative bound)
 //
-// Bound by HBM: 1.61 GB of a 2^26 x 6 snapshot in 0.262 ms (6.2 TB/s).  Fields
+// Bound by HBM: 1.61 GB of a 2^26 x 6 snapshot in 0.256 ms (6.3 TB/s; 0.263
+// before the fold at its end took all fields at once, finish_range).  Fields
 // of any alignment are read with 16-byte loads: a 10^7 x 6 snapshot with odd
-// rows 62 -> 56 us (55 aligned).
+// rows 62 -> 56 us, 49 with that fold.  As many CTAs as make rounds of equal
+// size instead of eight per SM: no change (49 us, 0.257 ms).
 
 // One warp per (block, field) item, field-major, so that consecutive warps
 // stream consecutive blocks of a field.  Each item yields the block's
@@ -18,7 +20,6 @@ namespace gpz {
 // NaN or an infinity in that field) and feeds the CTA's running extremes of
 // the field over its non-NaN values.
 __global__ void __launch_bounds__(kRangeThreads, 8) gpz_range_kernel(RangeArgs a) {
-    __shared__ float2 red[kRangeThreads / 32];
     __shared__ uint32_t s_lo[kMaxFields], s_hi[kMaxFields];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < kMaxFields) {
@@ -45,45 +46,7 @@ __global__ void __launch_bounds__(kRangeThreads, 8) gpz_range_kernel(RangeArgs a
         }
     }
     __syncthreads();
-    if (tid < a.F) {
-        const uint32_t kl = s_lo[tid], kh = s_hi[tid];
-        const bool any = kl != 0xffffffffu || kh != 0u;
-        a.partials[(size_t)blockIdx.x * a.F + tid] =
-            any ? make_float2(from_order_key(kl), from_order_key(kh)) : make_float2(INFINITY, -INFINITY);
-    }
-    // The last CTA to finish folds the partials and finalises the constants.
-    __shared__ bool last;
-    if (tid == 0) {
-        __threadfence();
-        last = atomicAdd(a.done_counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int f = 0; f < a.F; ++f) {  // all threads fold the CTAs' partials of field f
-        float lo = INFINITY, hi = -INFINITY;
-        for (unsigned c = tid; c < gridDim.x; c += blockDim.x) {
-            const float2 p = __ldcg(a.partials + (size_t)c * a.F + f);
-            lo = fminf(lo, p.x);
-            hi = fmaxf(hi, p.y);
-        }
-        lo = warp_min_f32(lo);
-        hi = warp_max_f32(hi);
-        if (lane == 0) red[warp] = make_float2(lo, hi);
-        __syncthreads();
-        if (tid == 0) {
-            for (int w = 1; w < kRangeThreads / 32; ++w) {
-                lo = fminf(lo, red[w].x);
-                hi = fmaxf(hi, red[w].y);
-            }
-            double rel = a.rel[0];
-#pragma unroll
-            for (int k = 1; k < kMaxFields; ++k)
-                if (k == f) rel = a.rel[k];
-            a.d_params[f] = range_params(lo, hi, rel);
-        }
-        __syncthreads();
-    }
+    finish_range<kRangeThreads>(a, s_lo, s_hi);
 }
 
 cudaError_t launch_range(const RangeArgs& a, int grid, cudaStream_t s) {

@@ -66,6 +66,58 @@ __device__ __forceinline__ float from_order_key(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
+// The end of a range pass: every CTA leaves its fields' extremes (order keys in
+// shared memory: 0xffffffff and 0 without a value) in partials, and the last one
+// to do so folds them and writes the constants.  All threads together, each
+// with one field (the stride is a multiple of F), so that the fold is one run
+// of independent loads and the constants' fp64 operations run side by side:
+// field after field, this was 6 us of every call with a relative bound and
+// six fields (the pass over 3*10^4 x 6 values 14.7 -> 8.9 us).
+template <int THREADS>
+__device__ __forceinline__ void finish_range(const RangeArgs& a, uint32_t* s_lo, uint32_t* s_hi) {
+    __shared__ bool last;
+    const int tid = threadIdx.x, F = a.F;
+    if (tid < F) {
+        const uint32_t kl = s_lo[tid], kh = s_hi[tid];
+        const bool any = kl != 0xffffffffu || kh != 0u;
+        a.partials[(size_t)blockIdx.x * F + tid] =
+            any ? make_float2(from_order_key(kl), from_order_key(kh)) : make_float2(INFINITY, -INFINITY);
+    }
+    if (tid < 32) __syncwarp();
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(a.done_counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    const uint32_t stride = (uint32_t)(THREADS / F * F), total = gridDim.x * (uint32_t)F;
+    if ((uint32_t)tid < stride) {
+        float lo = INFINITY, hi = -INFINITY;
+        for (uint32_t k0 = tid; k0 < total; k0 += 8u * stride) {
+            float2 p[8];
+#pragma unroll
+            for (uint32_t i = 0; i < 8u; ++i)
+                p[i] = k0 + i * stride < total ? __ldcg(a.partials + k0 + i * stride) : make_float2(INFINITY, -INFINITY);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                lo = fminf(lo, p[i].x);
+                hi = fmaxf(hi, p[i].y);
+            }
+        }
+        atomicMin(&s_lo[tid % F], order_key(lo));
+        atomicMax(&s_hi[tid % F], order_key(hi));
+    }
+    __syncthreads();
+    if (tid < F) {
+        double rel = a.rel[0];
+#pragma unroll
+        for (int k = 1; k < kMaxFields; ++k)
+            if (k == tid) rel = a.rel[k];
+        a.d_params[tid] = range_params(from_order_key(s_lo[tid]), from_order_key(s_hi[tid]), rel);
+    }
+}
+
 // The extremes of one block's n_b values of a field over its non-NaN values
 // (lo > hi when there are none), and whether a value is NaN or infinite (one
 // warp; every lane returns the same).  A whole block is read as 16-byte words,

@@ -86,6 +86,8 @@ __global__ void __launch_bounds__(kAosThreads) gpz_aos_range_kernel(const float*
                                                                     uint64_t ld, bool vec, RangeArgs ra) {
     __shared__ float tile[(kAosTile + 1) * F];
     __shared__ uint32_t s_lo[kMaxFields], s_hi[kMaxFields];
+    __shared__ float2 red[kAosThreads / 32];
+    __shared__ bool last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < kMaxFields) {
         s_lo[tid] = 0xffffffffu;
@@ -155,7 +157,43 @@ __global__ void __launch_bounds__(kAosThreads) gpz_aos_range_kernel(const float*
         }
         __syncthreads();
     }
-    finish_range<kAosThreads>(ra, s_lo, s_hi);
+    if (tid < F) {
+        const uint32_t kl = s_lo[tid], kh = s_hi[tid];
+        const bool any = kl != 0xffffffffu || kh != 0u;
+        ra.partials[(size_t)blockIdx.x * F + tid] =
+            any ? make_float2(from_order_key(kl), from_order_key(kh)) : make_float2(INFINITY, -INFINITY);
+    }
+    if (tid == 0) {
+        __threadfence();
+        last = atomicAdd(ra.done_counter, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // The last CTA folds every CTA's partial extremes of field f.  (All fields
+    // at once, as finish_range does, saves 2 us here but takes registers the
+    // pass over the tiles then runs without: 2^26 records of 3 fields 185 ->
+    // 275 us, of 6 fields 316 -> 369.)
+    for (int f = 0; f < F; ++f) {
+        float lo = INFINITY, hi = -INFINITY;
+        for (unsigned c = tid; c < gridDim.x; c += kAosThreads) {
+            const float2 pp = __ldcg(ra.partials + (size_t)c * F + f);
+            lo = fminf(lo, pp.x);
+            hi = fmaxf(hi, pp.y);
+        }
+        lo = warp_min_f32(lo);
+        hi = warp_max_f32(hi);
+        if (lane == 0) red[warp] = make_float2(lo, hi);
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < kAosThreads / 32; ++w) {
+                lo = fminf(lo, red[w].x);
+                hi = fmaxf(hi, red[w].y);
+            }
+            ra.d_params[f] = range_params(lo, hi, ra.rel[f]);
+        }
+        __syncthreads();
+    }
 }
 
 // Compression straight from 16-byte aligned interleaved records: the tile

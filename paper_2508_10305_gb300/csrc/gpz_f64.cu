@@ -294,7 +294,11 @@ uint64_t gpz_decompress_f64_workspace_size(uint64_t n, int n_fields) {
 gpz_status gpz_compress_f64(const double* const* d_fields, uint64_t n, const gpz_params* p, void* d_out,
                             uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size, uint32_t* d_perm,
                             void* d_ws, uint64_t ws_size, double* h_eb_used, void* stream) {
-    if (!p || p->n_fields < 1 || p->n_fields > kMaxFields || (p->mode != GPZ_EB_ABS && p->mode != GPZ_EB_REL))
+    // everything that either form checks: wide_compress takes its arguments as
+    // checked, and the data decides which form runs
+    if (!p || p->n_fields < 1 || p->n_fields > kMaxFields || p->seg_bits < 0 || p->seg_bits > kMaxSegBits ||
+        (p->mode != GPZ_EB_ABS && p->mode != GPZ_EB_REL) || !d_out || !aligned(d_out, 4) ||
+        (d_perm && !aligned(d_perm, 4)))
         return GPZ_ERR_INVALID_ARG;
     const int F = p->n_fields;
     for (int f = 0; f < F; ++f)

@@ -71,8 +71,9 @@ namespace {
 constexpr uint64_t kAlign = 256;
 constexpr int kRangeGridMax = 152 * 8;  // range-pass CTAs: 8 per SM of a GB300 (full occupancy)
 constexpr uint64_t kCtrlBytes = 256;    // words: 0 status, 1 scan tile counter, 2 range counter,
-                                        // 3 general-list count, 4-5 out size, 8 blocks left to the
-                                        // copy kernel (fused compaction)
+                                        // 3 warps of the tile kernel that took fallback
+                                        // candidates, 4-5 out size, 6 general-list count, 8 blocks
+                                        // left to the copy kernel (fused compaction)
 constexpr uint64_t kParamBytes = 256;   // FieldParams[8]
 constexpr unsigned kKnownFlags = GPZ_FLAG_FUSED_COMPACTION;
 
@@ -354,7 +355,8 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
         qa.perm = d_perm;
         qa.status = status;
         qa.general_list = reinterpret_cast<uint32_t*>(ws + L.list);
-        qa.general_count = status + 3;
+        qa.general_count = status + 6;
+        qa.fallback_count = status + 3;
         const uint32_t table_start = (uint32_t)(kHeaderWords + 2 * F);
         if (fused) {
             const uint64_t payload_start = table_start + nb + 1;

@@ -126,7 +126,6 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_batch_general_kernel(BatchCom
     const uint32_t count = *(volatile const uint32_t*)g.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
         const uint32_t entry = __ldcg(g.general_list + i), gb = entry & ~kRawBlock;
-        if (entry & kCodedBlock) continue;
         load_chunk_args(g, __ldg(g.block_map + gb), gb, A, slot);
         __syncthreads();
         const uint32_t b = slot[0];

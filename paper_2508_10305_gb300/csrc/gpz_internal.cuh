@@ -73,8 +73,9 @@ struct QseArgs {
     uint32_t sum_shift;
     uint32_t* perm;             // [n] or nullptr
     uint32_t* status;
-    uint32_t* general_list;     // [nblocks] blocks left to the general kernel (kCodedBlock: only recorded)
+    uint32_t* general_list;     // [nblocks] blocks left to the general kernel, each at most once
     uint32_t* general_count;    // zeroed
+    uint32_t* fallback_count;   // nullable: warps of the tile kernel that took fallback candidates (a measure, not read here)
     // Fused compaction only (gpz_qse_direct_kernel): the stream's payload,
     // the words it can hold, the per-block look-back states (zeroed) and a
     // count of the blocks that could not be placed directly.
@@ -85,10 +86,11 @@ struct QseArgs {
 };
 
 // In a general-list entry (a block index below 2^30: no device holds the
-// 2^40 particles of more): a block with a value that takes a fallback
-// candidate, coded by the tile kernel itself; a block with a value that no
-// candidate brings within its bound, to be stored raw.
-constexpr uint32_t kCodedBlock = 0x80000000u, kRawBlock = 0x40000000u;
+// 2^40 particles of more): a block with a value that no candidate brings
+// within its bound, to be stored raw.  A block is entered at most once, so the
+// list of one word per block cannot overrun: by the kernel that leaves it
+// before its sort, or by the check of the sorted order.
+constexpr uint32_t kRawBlock = 0x40000000u;
 
 constexpr uint32_t kPlaced = 0x80000000u;  // in a block's word count: already in the stream
 

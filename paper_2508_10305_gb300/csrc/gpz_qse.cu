@@ -64,7 +64,6 @@ __global__ void __launch_bounds__(kThreads, 2) gpz_qse_general_kernel(QseArgs a)
     const uint32_t count = *(volatile const uint32_t*)a.general_count;
     for (uint32_t i = blockIdx.x; i < count; i += gridDim.x) {
         const uint32_t entry = a.general_list[i], b = entry & ~kRawBlock;
-        if (entry & kCodedBlock) continue;
         if (entry & kRawBlock)
             write_raw<F>(a, b, (int)min((uint64_t)kBlock, a.n - (uint64_t)b * kBlock), threadIdx.x);
         else if ((uint64_t)(b + 1) * kBlock <= a.n)

@@ -75,9 +75,8 @@ struct alignas(16) TileShared : SortShared {
     TileField fc[kMaxFields];
 };
 
-constexpr uint32_t kFbCoded = 1u;      // a value took a fallback candidate
-constexpr uint32_t kFbGeneral = 2u;    // ... that could change its field's width: general path
-constexpr uint32_t kFbRaw = 4u;        // a value without a candidate in the bound: the block is stored raw
+constexpr uint32_t kFbGeneral = 1u;    // a fallback candidate that could change its field's width: general path
+constexpr uint32_t kFbRaw = 2u;        // a value without a candidate in the bound: the block is stored raw
 constexpr uint32_t kTfNonFinite = 1u;  // a non-finite value: stored raw
 constexpr uint32_t kTfBig = 2u;        // a code reaches 2^23: general path
 constexpr uint32_t kTfVerify = 4u;     // some field's first candidates need their check
@@ -230,7 +229,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
         quantise(std::integral_constant<int, 0>{});
     } else if (__any_sync(0xffffffffu, quantise(std::integral_constant<int, 1>{}))) {
         quantise(std::integral_constant<int, 2>{});  // rare: once more
-        if (lane == 0) atomicOr(&S.fallback, kFbCoded);
+        if (lane == 0 && a.fallback_count) atomicAdd(a.fallback_count, 1u);
     }
 
     if (OVER) {  // the warp's part of the first row becomes its counts
@@ -242,10 +241,8 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     rank_keys(key, hist, valid, S);
     __syncthreads();  // C: every value quantised (the tile is dead) and ranked
     if (const uint32_t all = S.fallback) {
-        if (t == 0)
-            a.general_list[atomicAdd(a.general_count, 1u)] =
-                idx.id() | (all & kFbRaw ? kRawBlock : all & kFbGeneral ? 0u : kCodedBlock);
-        if (all & (kFbGeneral | kFbRaw)) return;
+        if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id() | (all & kFbRaw ? kRawBlock : 0u);
+        return;
     }
     const uint32_t hdr = 1u + (uint32_t)F + (uint32_t)((F + 3) >> 2);
     const uint32_t rwords = ceil_words((uint32_t)n_b * W);

@@ -199,7 +199,9 @@ __global__ void __launch_bounds__(kAosThreads) gpz_aos_range_kernel(const float*
 // Compression straight from 16-byte aligned interleaved records: the tile
 // kernel's body with the block's records as its tile (one bulk copy of
 // 1024 F contiguous values), so no structure-of-arrays copy is made.
-cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s) { return launch_qse_tile_layout<kTileRecords>(a, s); }
+cudaError_t launch_qse_tile_aos(const QseArgs& a, bool early, cudaStream_t s) {
+    return launch_qse_tile_layout<kTileRecords>(a, early, s);
+}
 
 // Decompression into interleaved records: the block decoder stages the
 // block's values in record order in shared memory and writes the block's

@@ -366,7 +366,10 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
             qa.deferred_count = status + 8;
         }
         if (nb > 0) {
-            const cudaError_t e = fused ? launch_qse_direct(qa, s) : launch_qse_tile(qa, s);
+            // with range_done the fields may have been written by a kernel of this
+            // call (a transpose, the rounding of doubles)
+            const bool early = rel && !range_done;
+            const cudaError_t e = fused ? launch_qse_direct(qa, s) : launch_qse_tile(qa, early, s);
             if ((rc = cuda_status(e)) != GPZ_OK) break;
             rec.mark("qse");
             ++g_launches;  // two kernels: the fast path and the general list

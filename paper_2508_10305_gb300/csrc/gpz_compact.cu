@@ -199,11 +199,11 @@ __global__ void __launch_bounds__(32 * kCompactWarps) gpz_place_kernel(const __g
     // keeps the copy inside the bound even if a size were corrupt.
     const uint32_t raw_full = 1u + p.raw_fields * kBlock;
     const uint32_t raw_last = 1u + p.raw_fields * (uint32_t)(a.n - (uint64_t)(a.nblocks ? a.nblocks - 1 : 0) * kBlock);
-    auto words = [&](uint32_t b) { return min(__ldcg(a.sizes + b), b + 1u == a.nblocks ? raw_last : raw_full); };
+    auto words = [&](uint32_t b) { return min(load_after_wait(a.sizes + b), b + 1u == a.nblocks ? raw_last : raw_full); };
     wait_for_previous_kernel();
     const uint32_t run = b0 >> p.sum_shift;
     uint32_t acc = 0u;
-    for (uint32_t i = tid; i < run; i += 32 * kCompactWarps) acc += __ldcg(p.sums + i);
+    for (uint32_t i = tid; i < run; i += 32 * kCompactWarps) acc += load_after_wait(p.sums + i);
     for (uint32_t b = (run << p.sum_shift) + tid; b < b0; b += 32 * kCompactWarps) acc += words(b);
     uint32_t v = 0u;
     if (warp == 0 && (uint32_t)lane < cnt) v = words(b0 + lane);

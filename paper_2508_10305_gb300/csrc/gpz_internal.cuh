@@ -420,8 +420,12 @@ __device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned l
 
 // Launch a kernel that may be set up while the kernel before it on the stream
 // still ends (programmatic dependent launch).  The kernel calls
-// wait_for_previous_kernel() before it reads or writes anything that earlier
-// work on the stream touches.
+// wait_for_previous_kernel() before it writes anything and before it reads
+// anything that the kernel before it, or one that this one may in turn have
+// overtaken, writes; what the wait guards is read with load_after_wait (or
+// plain loads), never through the read-only path, whose data must not change
+// while a kernel runs.  Launched ordinarily, the same kernel's wait returns at
+// once.
 template <class... P, class... A>
 cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
     cudaLaunchConfig_t c = {};
@@ -438,15 +442,28 @@ cudaError_t launch_dependent(void (*kern)(P...), unsigned grid, unsigned threads
 }
 
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ uint32_t load_after_wait(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 load_after_wait(const uint2* p) {
+    uint2 v;
+    asm volatile("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
 
 // ---------------------------------------------------------------- launch wrappers (defined in the .cu files)
 
 cudaError_t launch_range(const RangeArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_qse_direct(const QseArgs& a, cudaStream_t s);  // register kernel placing blocks directly, then the general list
 cudaError_t launch_qse_general(const QseArgs& a, cudaStream_t s);
-cudaError_t launch_qse_tile(const QseArgs& a, cudaStream_t s);    // shared-memory tile kernel, then the general list
-cudaError_t launch_qse_tile_unaligned(const QseArgs& a, cudaStream_t s);  // the same on 4-byte aligned fields
-cudaError_t launch_qse_tile_aos(const QseArgs& a, cudaStream_t s); // the same on interleaved records (16-byte aligned)
+// Shared-memory tile kernel, then the general list.  early: the kernel before on
+// the stream is the range pass over the same fields, and nothing that this call
+// enqueued writes them, so the tile may be loaded while that pass still ends.
+cudaError_t launch_qse_tile(const QseArgs& a, bool early, cudaStream_t s);
+cudaError_t launch_qse_tile_unaligned(const QseArgs& a, bool early, cudaStream_t s);  // the same on 4-byte aligned fields
+cudaError_t launch_qse_tile_aos(const QseArgs& a, bool early, cudaStream_t s); // the same on interleaved records (16-byte aligned)
 cudaError_t launch_decompress_aos(const DecArgs& a, cudaStream_t s); // decompression into interleaved records
 cudaError_t launch_block_info(const uint2* bext, const FieldParams* d_params, uint32_t nblocks, int F,
                               unsigned long long* binfo, cudaStream_t s);

@@ -57,12 +57,12 @@
 namespace gpz {
 
 // Fields that are all 16-byte aligned take the kernel without shifts.
-cudaError_t launch_qse_tile(const QseArgs& a, cudaStream_t s) {
+cudaError_t launch_qse_tile(const QseArgs& a, bool early, cudaStream_t s) {
     if (a.nblocks == 0) return cudaSuccess;
-    if (a.interleaved) return launch_qse_tile_aos(a, s);  // gpz_aos.cu
+    if (a.interleaved) return launch_qse_tile_aos(a, early, s);  // gpz_aos.cu
     for (int f = 0; f < a.F; ++f)
-        if (reinterpret_cast<uintptr_t>(a.fields[f]) & 15u) return launch_qse_tile_unaligned(a, s);
-    return launch_qse_tile_layout<kTileAligned>(a, s);
+        if (reinterpret_cast<uintptr_t>(a.fields[f]) & 15u) return launch_qse_tile_unaligned(a, early, s);
+    return launch_qse_tile_layout<kTileAligned>(a, early, s);
 }
 
 }  // namespace gpz

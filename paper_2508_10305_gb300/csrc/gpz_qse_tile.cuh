@@ -380,7 +380,9 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         if (k >= s && k < end && ((t & 4) || k < 4u * lo)) tile[f * ROW + k] = __ldcs(a.fields[f] + first + (k - s));
     }
     if (!tile_overlays_hist(F, LAY)) clear_hist_row(reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY)));
-    if (PRE) wait_for_previous_kernel();  // the range pass's results; the tile above is the caller's data
+    // the range pass's results; the tile above is complete before the range
+    // pass starts, or the launch is an ordinary one (launch_qse_tile's `early`)
+    if (PRE) wait_for_previous_kernel();
     // ---- 2. the field constants from the block's extremes: those of the
     // range pass (loaded with the step constants while the tile is in
     // flight), or found in the tile, a warp per field
@@ -424,7 +426,7 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         uint2 e = make_uint2(0u, 0u);
         FieldParams p = {};
         if (lane < F) {
-            e = PRE ? __ldg(a.bext + (size_t)b * F + lane) : S.ext[lane];
+            e = PRE ? load_after_wait(a.bext + (size_t)b * F + lane) : S.ext[lane];
             p = a.d_params ? a.d_params[lane] : a.params[lane];
         }
         tile_constants<F>(e, p, a.G, lane < F ? (uint32_t)lane * ROW + shift(lane) : 0u, S);

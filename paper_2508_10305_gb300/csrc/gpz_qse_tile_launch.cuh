@@ -32,13 +32,13 @@ __global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_qse_tile_
 }
 
 template <int F, bool PRE, int LAY>
-cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
+cudaError_t launch_qse_tile_fp(const QseArgs& a, bool early, cudaStream_t s) {
     const size_t smem = tile_smem_bytes(F, LAY);
     auto kern = gpz_qse_tile_kernel<F, PRE, LAY>;
     static_assert(tile_smem_bytes(F, LAY) + sizeof(TileShared) <= 48u * 1024u, "within the default limit of a CTA");
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;
-    if (PRE) {
+    if (PRE && early) {
         e = launch_dependent(kern, a.nblocks, kTileThreads, smem, s, a);
     } else {
         kern<<<a.nblocks, kTileThreads, smem, s>>>(a);
@@ -51,11 +51,11 @@ cudaError_t launch_qse_tile_fp(const QseArgs& a, cudaStream_t s) {
 // One layout's launches (a translation unit each, so that they compile in
 // parallel: gpz_qse_tile.cu, gpz_qse_tile_unaligned.cu, gpz_aos.cu).
 template <int LAY>
-cudaError_t launch_qse_tile_layout(const QseArgs& a, cudaStream_t s) {
+cudaError_t launch_qse_tile_layout(const QseArgs& a, bool early, cudaStream_t s) {
     const bool pre = a.bext != nullptr;
     switch (a.F) {
 #define GPZ_CASE(FF) \
-    case FF: return pre ? launch_qse_tile_fp<FF, true, LAY>(a, s) : launch_qse_tile_fp<FF, false, LAY>(a, s);
+    case FF: return pre ? launch_qse_tile_fp<FF, true, LAY>(a, early, s) : launch_qse_tile_fp<FF, false, LAY>(a, early, s);
         GPZ_CASE(1)
         GPZ_CASE(2)
         GPZ_CASE(3)

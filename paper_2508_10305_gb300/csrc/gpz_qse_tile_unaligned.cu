@@ -7,8 +7,8 @@
 
 namespace gpz {
 
-cudaError_t launch_qse_tile_unaligned(const QseArgs& a, cudaStream_t s) {
-    return launch_qse_tile_layout<kTileUnaligned>(a, s);
+cudaError_t launch_qse_tile_unaligned(const QseArgs& a, bool early, cudaStream_t s) {
+    return launch_qse_tile_layout<kTileUnaligned>(a, early, s);
 }
 
 }  // namespace gpz

@@ -208,6 +208,15 @@ struct BitAppender {
     }
 };
 
+// The order and the size of a block stored raw.
+template <int F, int TH>
+__device__ __forceinline__ void raw_done(const QseArgs& a, uint32_t b, int n_b, int t) {
+    const uint64_t first = (uint64_t)b * kBlock;
+    if (a.perm)
+        for (int i = t; i < n_b; i += TH) a.perm[first + i] = (uint32_t)(first + i);
+    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, 1u + (uint32_t)F * (uint32_t)n_b);
+}
+
 template <int F, int TH = kThreads>
 __device__ __forceinline__ void write_raw(const QseArgs& a, uint32_t b, int n_b, int t) {
     const uint64_t first = (uint64_t)b * kBlock;
@@ -231,9 +240,7 @@ __device__ __forceinline__ void write_raw(const QseArgs& a, uint32_t b, int n_b,
                 if (t + k * TH < n_b) out[1 + f * n_b + t + k * TH] = __float_as_uint(v[k]);
         }
     }
-    if (a.perm)
-        for (int i = t; i < n_b; i += TH) a.perm[first + i] = (uint32_t)(first + i);
-    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, 1u + (uint32_t)F * (uint32_t)n_b);
+    raw_done<F, TH>(a, b, n_b, t);
 }
 
 // The general per-block path: any block, including codes >= 2^23, values

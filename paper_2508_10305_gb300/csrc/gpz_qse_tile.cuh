@@ -123,6 +123,24 @@ __device__ __forceinline__ void tile_constants(const uint2 e, const FieldParams&
     if (lane == 0) S.blk = make_uint4(flags, W, keybits, 0u);
 }
 
+// The block stored raw, from its tile: a second read of the input through L2
+// (write_raw) by 128 threads made a 2^24 x 6 snapshot with a NaN in every block
+// 0.378 -> 0.413 ms; 0.345 this way.
+template <int F, int LAY>
+__device__ __forceinline__ void tile_write_raw(const QseArgs& a, const float* tile, const TileShared& S, uint32_t b,
+                                               int n_b) {
+    const int t = threadIdx.x;
+    uint32_t* out = a.temp + (size_t)b * a.slot_words;
+    if (t == 0) out[0] = 1u;
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+        const float* row = tile + (LAY == kTileUnaligned ? (int)S.fc[f].row : f * kBlock);
+        for (int i = t; i < n_b; i += kTileThreads)
+            out[1 + f * n_b + i] = __float_as_uint(LAY == kTileRecords ? tile[i * F + f] : row[i]);
+    }
+    raw_done<F, kTileThreads>(a, b, n_b, t);
+}
+
 // Steps 3 to 5 for a block whose records are at most 32 NR bits wide (NR = 2
 // or 4): the common case keeps two registers per record instead of four.
 template <int F, bool FULL, int LAY, int NR, class Idx>
@@ -436,7 +454,7 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
     const uint4 blk = S.blk;
     const uint32_t flags = blk.x, W = blk.y;
     if (flags & kTfNonFinite) {
-        write_raw<F, kTileThreads>(a, b, n_b, t);
+        tile_write_raw<F, LAY>(a, tile, S, b, n_b);
         return;
     }
     if ((flags & kTfBig) || W > kFastRecordBits) {

@@ -22,6 +22,10 @@ def test_raw_blocks(gpz, oracle, F, n, offset, mode):  # noqa: F811
     bits = x.view(np.uint32)
     assert np.array_equal(o.view(np.uint32), bits)
     st = torch.from_numpy(s.copy()).cuda()
+    rec = torch.zeros(n * F + 1, device="cuda")
+    for at in (0, 1):  # compressed from records, one word past a 16-byte boundary too
+        rec[at:at + n * F] = torch.from_numpy(x.T.copy()).cuda().view(-1)
+        assert torch.equal(gpz.compress_aos(rec[at:at + n * F], F, 1e-2, mode, 3)[0], st)
     assert np.array_equal(gpz.decompress_aos(st, F, n).cpu().numpy().view(np.uint32), bits.T)
     assert np.array_equal(gpz.decompress_f64(st, F, n).cpu().numpy().view(np.uint64), x.astype(np.float64).view(np.uint64))
     out = torch.zeros(n * F + 1, device="cuda")  # records one word past a 16-byte boundary

@@ -197,26 +197,6 @@ struct WideAppender {
 };
 
 template <int F>
-__device__ __forceinline__ void wide_write_raw(const WideQseArgs& a, uint32_t b, int n_b, int t) {
-    const uint64_t first = (uint64_t)b * kBlock;
-    uint32_t* out = a.temp + (size_t)b * a.slot_words;
-    if (t == 0) out[0] = 1u;
-#pragma unroll
-    for (int f = 0; f < F; ++f) {
-        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(a.fields[f] + first);
-        for (int i = t; i < n_b; i += kWideThreads) {
-            const unsigned long long u = __ldg(src + i);
-            const uint32_t k = 1u + 2u * ((uint32_t)f * (uint32_t)n_b + (uint32_t)i);
-            out[k] = (uint32_t)u;
-            out[k + 1] = (uint32_t)(u >> 32);
-        }
-    }
-    if (a.perm)
-        for (int i = t; i < n_b; i += kWideThreads) a.perm[first + i] = (uint32_t)(first + i);
-    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, 1u + 2u * (uint32_t)F * (uint32_t)n_b);
-}
-
-template <int F>
 __device__ __forceinline__ void wide_block_general(const WideQseArgs& a, uint8_t* dsm, WideShared& S, uint32_t b) {
     constexpr int P = F < 3 ? F : 3;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -279,7 +259,7 @@ __device__ __forceinline__ void wide_block_general(const WideQseArgs& a, uint8_t
     if (__any_sync(0xffffffffu, nonfinite) && lane == 0) atomicOr(&S.flags, 1u);
     __syncthreads();
     if (S.flags & 1u) {
-        wide_write_raw<F>(a, b, n_b, t);
+        wide_write_raw<F, kWideThreads>(a, b, n_b, t);
         return;
     }
     // fields whose first candidates pass for certain (flag bit 2 + f)
@@ -332,7 +312,7 @@ __device__ __forceinline__ void wide_block_general(const WideQseArgs& a, uint8_t
     if (__any_sync(0xffffffffu, fail) && lane == 0) atomicOr(&S.flags, 2u);
     __syncthreads();
     if (S.flags & 2u) {
-        wide_write_raw<F>(a, b, n_b, t);
+        wide_write_raw<F, kWideThreads>(a, b, n_b, t);
         return;
     }
 
@@ -457,7 +437,7 @@ __device__ __forceinline__ void wide_block_general(const WideQseArgs& a, uint8_t
     const uint32_t rwords = ceil_words((uint32_t)n_b * W);
     const uint32_t enc = hdr + dwords + cwords + rwords;
     if (enc >= 1u + 2u * (uint32_t)F * (uint32_t)n_b) {
-        wide_write_raw<F>(a, b, n_b, t);
+        wide_write_raw<F, kWideThreads>(a, b, n_b, t);
         return;
     }
 

@@ -102,6 +102,33 @@ __device__ __forceinline__ bool first_candidate_exact(double bmin, double bmax, 
            fmax(fabs(bmin), fabs(bmax)) <= p.eb * 0x1p45;
 }
 
+// A block stored raw: its values as they are, field after field; a thread has
+// all of its values of a field in flight.
+template <int F, int TH>
+__device__ __forceinline__ void wide_write_raw(const WideQseArgs& a, uint32_t b, int n_b, int t) {
+    constexpr int N = kBlock / TH;
+    const uint64_t first = (uint64_t)b * kBlock;
+    uint32_t* out = a.temp + (size_t)b * a.slot_words;
+    if (t == 0) out[0] = 1u;
+#pragma unroll 1
+    for (int f = 0; f < F; ++f) {
+        const unsigned long long* src = reinterpret_cast<const unsigned long long*>(a.fields[f] + first);
+        unsigned long long v[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) v[k] = t + k * TH < n_b ? __ldg(src + t + k * TH) : 0ull;
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            if (t + k * TH >= n_b) continue;
+            uint32_t* at = out + 1 + 2 * (f * n_b + t + k * TH);
+            at[0] = (uint32_t)v[k];
+            at[1] = (uint32_t)(v[k] >> 32);
+        }
+    }
+    if (a.perm)
+        for (int i = t; i < n_b; i += TH) a.perm[first + i] = (uint32_t)(first + i);
+    if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, 1u + 2u * (uint32_t)F * (uint32_t)n_b);
+}
+
 // Stages 1-3 of the blocks the common path takes, the others into the
 // general list (gpz_wide_fast.cu).
 cudaError_t launch_wide_fast(const WideQseArgs& a, cudaStream_t s);

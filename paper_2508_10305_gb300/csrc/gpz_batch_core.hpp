@@ -73,9 +73,11 @@ void core_pack(const BatchCore& c, uint8_t* host);
 BatchDevice core_device_view(const BatchCore& c, uint8_t* device);
 
 // Enqueue one run on s: clear the workspace's control words, then the kernels.
-// timed: record per-kernel events when stage timing is on.
+// timed: record per-kernel events when stage timing is on.  `blocks` enqueues
+// the kernel over a group's blocks (tests pass another).
 gpz_status core_enqueue(const BatchCore& c, const BatchDevice& dev, uint8_t* ws, uint64_t* d_out_sizes,
-                        cudaStream_t s, bool timed);
+                        cudaStream_t s, bool timed,
+                        cudaError_t (*blocks)(const BatchCompressArgs&, int, cudaStream_t) = launch_batch_compress);
 
 }  // namespace host
 }  // namespace gpz

@@ -12,7 +12,7 @@ namespace gpz {
 // One CTA per block of the group: the tile kernel's code, with the chunk's
 // arguments in shared memory, in the layout that every chunk of the group
 // allows.
-template <int F, bool PRE, int LAY>
+template <int F, bool PRE, int LAY, class Idx = SlotBlock>
 __global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_batch_tile_kernel(BatchCompressArgs g) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ TileShared S;
@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_batch_til
     const uint32_t gb = g.block_first + blockIdx.x;
     load_chunk_args(g, __ldg(g.block_map + gb), gb, A, slot);
     __syncthreads();
-    const SlotBlock idx{slot};
+    const Idx idx{slot};
     if ((uint64_t)(idx.b() + 1) * kBlock <= A.n)
         qse_block_tile<F, true, PRE, LAY>(A, dsm, S, idx);
     else

@@ -12,6 +12,7 @@
 
 #include "gpz.h"
 #include "gpz_internal.cuh"
+#include "gpz_wide.cuh"
 
 namespace gpz {
 namespace host {
@@ -137,13 +138,13 @@ RangeTargets compress_range_targets(uint64_t n, int F);
 constexpr int kRangeCtasMax = 152 * 8;  // partials held for this many CTAs
 
 // gpz_compress, optionally with the range pass already done (gpz_api.cu).
-// With `interleaved` (16-byte aligned F-field records, d_fields[f] =
+// `tile` enqueues the tile kernel (tests pass another).  With `interleaved` (16-byte aligned F-field records, d_fields[f] =
 // interleaved + f) the tile kernel reads the records themselves; a relative
 // bound then needs the range pass done.
 gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_params* p, void* d_out,
                          uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size, uint32_t* d_perm,
                          void* d_ws, uint64_t ws_size, void* stream, bool range_done,
-                         const float* interleaved = nullptr);
+                         const float* interleaved = nullptr, cudaError_t (*tile)(const QseArgs&, bool, cudaStream_t) = launch_qse_tile);
 
 // gpz_decompress; with `interleaved` the values go to F-field records there
 // (d_fields[f] = interleaved + f, 4-byte aligned) (gpz_api.cu).
@@ -159,11 +160,13 @@ cudaError_t launch_decompress64(const DecArgs& a, cudaStream_t s);
 namespace host {
 
 // The 64-bit form (gpz_wide.cu): its workspace, and compression with
-// absolute bounds eb[f] (the header records `mode`).
+// absolute bounds eb[f] (the header records `mode`); `fast` enqueues its fast
+// kernel (tests pass another).
 uint64_t wide_workspace_size(uint64_t n, int F);
 gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G, int mode, const double* eb,
                          void* d_out, uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size,
-                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre = false);
+                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre = false,
+                         cudaError_t (*fast)(const WideQseArgs&, cudaStream_t) = launch_wide_fast);
 
 }  // namespace host
 }  // namespace gpz

@@ -46,12 +46,14 @@ struct QseShared {
 // Where the fast path gets its block's index: the grid (one CTA per block),
 // or a shared-memory slot (the batched kernel's block within its chunk)
 // re-read at each use, so that the index holds no register through the
-// block code.
+// block code.  kUnstable (tests only): every block's sort fails its check.
 struct GridBlock {
+    static constexpr bool kUnstable = false;
     __device__ __forceinline__ uint32_t b() const { return blockIdx.x; }   // block within its array
     __device__ __forceinline__ uint32_t id() const { return blockIdx.x; }  // entry for the general list
 };
 struct SlotBlock {
+    static constexpr bool kUnstable = false;
     const volatile uint32_t* slot;  // [0]: block within its array, [1]: entry for the general list
     __device__ __forceinline__ uint32_t b() const { return slot[0]; }
     __device__ __forceinline__ uint32_t id() const { return slot[1]; }

@@ -320,7 +320,7 @@ __device__ __forceinline__ void tile_encode(const QseArgs& a, uint8_t* dsm, Tile
     fence_proxy_async_shared();  // the staging words are read by a bulk copy (async proxy)
     __syncthreads();
     if (t == 0) bulk_s2g_start(a.temp + (size_t)b * a.slot_words, stage, ((enc + 3u) & ~3u) * 4u);
-    if (!sorted_order(key, order, valid, i0, n_b, a.perm != nullptr, S)) {
+    if (!sorted_order(key, order, valid, i0, n_b, a.perm != nullptr, S) || Idx::kUnstable) {
         if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = idx.id();  // not stable: the general kernel redoes it
     } else {
         if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, enc);

@@ -11,30 +11,32 @@ namespace gpz {
 // no SM yet) and would otherwise end the kernel alone; 1.7*10^7 x 3 records
 // with 43 in the last block: 102 -> 93 us.
 struct LastFirst {
+    static constexpr bool kUnstable = false;
     __device__ __forceinline__ uint32_t b() const { return blockIdx.x ? blockIdx.x - 1u : gridDim.x - 1u; }  // block within its array
     __device__ __forceinline__ uint32_t id() const { return b(); }  // entry for the general list
 };
 
 struct LastBlock {
+    static constexpr bool kUnstable = false;
     __device__ __forceinline__ uint32_t b() const { return gridDim.x - 1u; }
     __device__ __forceinline__ uint32_t id() const { return b(); }
 };
 
-template <int F, bool PRE, int LAY>
+template <int F, bool PRE, int LAY, class First = LastFirst, class Last = LastBlock>
 __global__ void __launch_bounds__(kTileThreads, tile_ctas(F, LAY)) gpz_qse_tile_kernel(const __grid_constant__ QseArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ TileShared S;
     // the grid's last block may be ragged
     if (blockIdx.x != 0u || (uint64_t)gridDim.x * kBlock == a.n)
-        qse_block_tile<F, true, PRE, LAY>(a, dsm, S, LastFirst{});
+        qse_block_tile<F, true, PRE, LAY>(a, dsm, S, First{});
     else
-        qse_block_tile<F, false, PRE, LAY>(a, dsm, S, LastBlock{});
+        qse_block_tile<F, false, PRE, LAY>(a, dsm, S, Last{});
 }
 
-template <int F, bool PRE, int LAY>
+template <int F, bool PRE, int LAY, class First = LastFirst, class Last = LastBlock>
 cudaError_t launch_qse_tile_fp(const QseArgs& a, bool early, cudaStream_t s) {
     const size_t smem = tile_smem_bytes(F, LAY);
-    auto kern = gpz_qse_tile_kernel<F, PRE, LAY>;
+    auto kern = gpz_qse_tile_kernel<F, PRE, LAY, First, Last>;
     static_assert(tile_smem_bytes(F, LAY) + sizeof(TileShared) <= 48u * 1024u, "within the default limit of a CTA");
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (e != cudaSuccess) return e;

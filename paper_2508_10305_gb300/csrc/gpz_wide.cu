@@ -1052,7 +1052,8 @@ uint64_t wide_workspace_size(uint64_t n, int F) {
 // cleared before it.
 gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G, int mode, const double* eb,
                          void* d_out, uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size,
-                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre) {
+                         uint32_t* d_perm, void* d_ws, uint64_t ws_size, cudaStream_t s, bool pre,
+                         cudaError_t (*fast)(const WideQseArgs&, cudaStream_t)) {
     const uint64_t nb = nblocks_of(n);
     if (nb + 2ull * (uint64_t)F * n >= (1ull << 32)) return GPZ_ERR_UNSUPPORTED;
     if (out_capacity < gpz_bound_size_wide(n, F)) return GPZ_ERR_CAPACITY;
@@ -1084,7 +1085,7 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     qa.general_list = stream_words + table_start;  // the offset table's place, written by the scan later
     qa.general_count = status + 2;
     if (nb > 0) {
-        if (launch_wide_fast(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;
+        if (fast(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;
         rec.mark("wide_qse");
         if (launch_wide_general(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;
         rec.mark("wide_general");

@@ -133,5 +133,7 @@ __device__ __forceinline__ void wide_write_raw(const WideQseArgs& a, uint32_t b,
 // general list (gpz_wide_fast.cu).
 cudaError_t launch_wide_fast(const WideQseArgs& a, cudaStream_t s);
 cudaError_t prepare_wide_fast(int F);  // its attributes on the current device
+// Tests: three fields, every block's sort failing its check.
+cudaError_t launch_wide_fast_unstable(const WideQseArgs& a, cudaStream_t s);
 
 }  // namespace gpz

@@ -108,7 +108,8 @@ __device__ __forceinline__ bool out_of_reach(unsigned long long nmin, unsigned l
 
 }  // namespace
 
-template <int F>
+// UNSTABLE (tests only): every block's sort fails its check.
+template <int F, bool UNSTABLE = false>
 __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel(const __grid_constant__ WideQseArgs a) {
     extern __shared__ __align__(128) uint8_t dsm[];
     __shared__ WfShared S;
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
     fence_proxy_async_shared();  // the staging words are read by a bulk copy (async proxy)
     __syncthreads();
     if (t == 0) bulk_s2g_start(out, stage, ((enc + 3u) & ~3u) * 4u);
-    if (!sorted_order(key, order, valid, i0, n_b, a.perm != nullptr, S)) {
+    if (!sorted_order(key, order, valid, i0, n_b, a.perm != nullptr, S) || UNSTABLE) {
         if (t == 0) a.general_list[atomicAdd(a.general_count, 1u)] = b;  // not stable: the general kernel redoes it
     } else {
         if (t == 0) store_size(a.sizes, a.sums, a.sum_shift, b, enc);
@@ -313,9 +314,9 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
 
 namespace {
 
-template <int F>
+template <int F, bool UNSTABLE = false>
 cudaError_t prepare_wide_fast_f() {
-    auto kern = gpz_wide_fast_kernel<F>;
+    auto kern = gpz_wide_fast_kernel<F, UNSTABLE>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wf_smem_bytes(F));
     return e != cudaSuccess ? e : cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
 }
@@ -340,6 +341,14 @@ cudaError_t launch_wide_fast(const WideQseArgs& a, cudaStream_t s) {
         case 8: return launch_wide_fast_f<8>(a, s);
     }
     return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_wide_fast_unstable(const WideQseArgs& a, cudaStream_t s) {
+    if (a.F != 3) return cudaErrorInvalidValue;
+    const cudaError_t e = prepare_wide_fast_f<3, true>();
+    if (e != cudaSuccess) return e;
+    gpz_wide_fast_kernel<3, true><<<a.nblocks, kTileThreads, wf_smem_bytes(3), s>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t prepare_wide_fast(int F) {

@@ -141,6 +141,11 @@ def _load():
     L.gpz_test_scan_timeout.restype = C.c_int
     L.gpz_test_block_lookback_timeout.argtypes = [C.c_uint32, C.c_uint32, vp, u64, P(C.c_int), vp]
     L.gpz_test_block_lookback_timeout.restype = C.c_int
+    L.gpz_test_unstable_sort_workspace_size.argtypes = [u64]
+    L.gpz_test_unstable_sort_workspace_size.restype = u64
+    L.gpz_test_unstable_sort.argtypes = [C.c_int, P(vp), u64, P(gpz_params), vp, u64, P(u64), vp, vp, u64,
+                                         P(C.c_uint32), vp]
+    L.gpz_test_unstable_sort.restype = C.c_int
     # batched entry points (include/gpz_batch.h)
     L.gpz_batch_create_compress.argtypes = [P(gpz_compress_chunk), C.c_uint32, P(vp)]
     L.gpz_batch_create_compress.restype = C.c_int

@@ -95,3 +95,31 @@ def test_a_block_is_listed_once_and_only_when_left(gpz, oracle, kind, offset, mo
     if mode == 0:  # the bound, and so every block's route, is the one worked out
         assert listed == (0 if kind == "coded" else nb)
         assert nb <= warps <= 4 * nb
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["coded", "general", "raw"])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_routes_in_records_and_batches(gpz, oracle, kind, offset):  # noqa: F811
+    """The same blocks as records, and as a chunk of a batch beside one that
+    takes the ordinary way, from every word of a 16-byte unit."""
+    x = blocks(kind, 5, 3 + offset)[:, :5 * BLOCK - 100]
+    n = x.shape[1]
+    ref, perm = oracle.compress(x, EB, 0, 3)
+    rec = torch.zeros(3 * n + 4, device="cuda")
+    rec[offset:offset + 3 * n] = torch.from_numpy(x.T.copy()).cuda().view(-1)
+    got, p = gpz.compress_aos(rec[offset:offset + 3 * n], 3, EB, 0, 3, want_perm=True)
+    assert np.array_equal(got.cpu().numpy(), ref)
+    assert np.array_equal(p.cpu().numpy().astype(np.uint32), perm)
+    y = (np.random.default_rng(7).random((3, 3000)) * 50.0).astype(np.float32)
+    chunks, refs = [], []
+    for v, at in ((y, 0), (x, offset)):
+        buf = torch.zeros(3, v.shape[1] + 8, device="cuda")
+        buf[:, at:at + v.shape[1]] = torch.from_numpy(v)
+        chunks.append(([buf[f, at:at + v.shape[1]] for f in range(3)], gpz.make_params(3, EB, 0, 3)))
+        refs.append(oracle.compress(v, EB, 0, 3)[0])
+    c = gpz.BatchCompressor(chunks)
+    c()
+    assert c.status()[0] == gpz.OK
+    for s, r in zip(c.streams(), refs):
+        assert np.array_equal(s.cpu().numpy(), r)

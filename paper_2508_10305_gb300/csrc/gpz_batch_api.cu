@@ -217,8 +217,7 @@ gpz_status gpz_batch_tune(gpz_batch* p, void* d_ws, uint64_t ws_size, uint64_t* 
     cudaStream_t s = (cudaStream_t)stream;
     const BatchCore& c = p->core;
     // one parameter at a time, the others at their best so far: the Q.S.E.
-    // body (when a group can take the tile body), the range slice (relative
-    // bounds only), then the compaction grid
+    // body, the range slice (relative bounds only), then the compaction grid
     std::vector<std::vector<gpz_batch_config>> stages;
     if (c.kind == 0) stages.push_back({{0, 0, 0, 1}, {0, 0, 0, 2}});
     if (c.kind == 0 && c.any_rel) {

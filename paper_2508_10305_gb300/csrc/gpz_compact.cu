@@ -229,9 +229,9 @@ __global__ void __launch_bounds__(32 * kCompactWarps) gpz_place_kernel(const __g
         copy_block(a.temp + (size_t)(b0 + k) * a.slot_words, payload + s_off[k], s_off[k + 1] - s_off[k], lane);
 }
 
-// Blocks per CTA: one per warp, two when the grid would otherwise pass two
-// waves of six CTAs per SM (one / two / four per warp on 2^25 x 3 uniform
-// positions: 56.5 / 55.0 / 59.2 us).
+// Blocks per CTA: one per warp, two when the grid would otherwise pass twelve
+// CTAs per SM, of which five are resident (46 registers; one / two / four per
+// warp on 2^25 x 3 uniform positions: 56.5 / 55.0 / 59.2 us).
 cudaError_t launch_place(const CompactArgs& a, const PlaceArgs& args, cudaStream_t s) {
     PlaceArgs p = args;
     p.log_blocks = 3;

@@ -203,7 +203,7 @@ __device__ __forceinline__ void decode_wide(const DecArgs& a, const uint32_t* bl
 struct DecCore {  // everything a block's decoding keeps in shared memory but its staged words
     uint16_t uniq[kMaxBins];
     uint32_t mask[32];
-    uint32_t warp_uc[kDecWarps];  // per warp: id sum | count sum << 15
+    uint32_t warp_uc[kDecWarps];  // per warp: id sum | count sum << 14
     uint32_t bad;
     // the block's constants, checked by warp 0 and read by every warp
     uint32_t ok, raw, U, wd, wc, W, keybits, G;

@@ -1,7 +1,7 @@
 // gpz_qse_tile.cuh -- the per-block body of the shared-memory tile
 // compression kernel (Sections 4.1-4.3), used by the single-array kernel
 // (gpz_qse_tile.cu, which describes the design), the interleaved-record
-// kernel (gpz_aos.cu) and the batched kernel (gpz_batch_compress.cu).  Idx
+// kernel (gpz_aos.cu) and the batched kernel (gpz_batch_tile.cuh).  Idx
 // gives the block within its array (b()) and its entry for the general list
 // (id()).
 #pragma once
@@ -45,8 +45,10 @@ __host__ __device__ constexpr uint32_t tile_smem_bytes(int F, int layout) {
 
 // Resident CTAs per SM the kernels are compiled for: what shared memory
 // allows (227 KB, 1 KB reserved per CTA, about 0.6 KB of static memory), at
-// most nine (56 registers per thread; more CTAs spill, see gpz_qse_tile.cu),
-// eight from five fields on (64 registers).
+// most nine (56 registers per thread), eight from five fields on (64
+// registers): the counts that measured best, although from three fields on
+// 140 to 600 bytes of a thread's values then live in local memory (see
+// gpz_qse_tile.cu for fewer and more CTAs).
 constexpr int kTileMaxCtas = 9;
 __host__ __device__ constexpr int tile_ctas(int F, int layout) {
     const int by_smem = (int)((227u * 1024u) / (tile_smem_bytes(F, layout) + 1024u + 640u));

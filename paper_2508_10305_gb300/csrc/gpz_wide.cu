@@ -1082,7 +1082,7 @@ gpz_status wide_compress(const double* const* d_fields, uint64_t n, int F, int G
     qa.nblocks = (uint32_t)nb;
     const uint32_t table_start = (uint32_t)(kHeaderWords + 4 * F);
     uint32_t* stream_words = static_cast<uint32_t*>(d_out);
-    qa.general_list = stream_words + table_start;  // the offset table's place, written by the scan later
+    qa.general_list = stream_words + table_start;  // the offset table's place, which the copy kernel writes after the general kernel
     qa.general_count = status + 2;
     if (nb > 0) {
         if (fast(qa, s) != cudaSuccess) return GPZ_ERR_CUDA;

@@ -370,7 +370,7 @@ gpz_status gpz_compress_aos(const float* d_aos, uint64_t n, const gpz_params* p,
         for (int f = 0; f < F; ++f) fields[f] = direct ? d_aos + f : soa + (uint64_t)f * ld;
         // the compression workspace sits at the start, so gpz_sync_status(d_ws) reads its status
         rc = compress_impl(fields, n, p, d_out, out_capacity, d_out_size, h_out_size, d_perm, ws, cws, stream,
-                           range_done, direct && n > 0 ? d_aos : nullptr);
+                           range_done, direct && n > 0 ? d_aos : nullptr, /*fields_ready=*/direct);
     }
     if (own) {  // as gpz_compress without a workspace: synchronise and return the device-side status
         if (rc == GPZ_OK) {

@@ -244,7 +244,7 @@ RangeTargets compress_range_targets(uint64_t n, int F) {
 gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_params* p, void* d_out,
                          uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size, uint32_t* d_perm,
                          void* d_ws, uint64_t ws_size, void* stream, bool range_done,
-                         const float* interleaved, cudaError_t (*tile)(const QseArgs&, bool, cudaStream_t)) {
+                         const float* interleaved, bool fields_ready, cudaError_t (*tile)(const QseArgs&, bool, cudaStream_t)) {
     if (!p || !d_out || !aligned(d_out, 4)) return GPZ_ERR_INVALID_ARG;
     const int F = p->n_fields;
     if (F < 1 || F > kMaxFields || p->seg_bits < 0 || p->seg_bits > kMaxSegBits ||
@@ -366,10 +366,7 @@ gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_par
             qa.deferred_count = status + 8;
         }
         if (nb > 0) {
-            // with range_done the fields may have been written by a kernel of this
-            // call (a transpose, the rounding of doubles)
-            const bool early = rel && !range_done;
-            const cudaError_t e = fused ? launch_qse_direct(qa, s) : tile(qa, early, s);
+            const cudaError_t e = fused ? launch_qse_direct(qa, s) : tile(qa, fields_ready, s);
             if ((rc = cuda_status(e)) != GPZ_OK) break;
             rec.mark("qse");
             ++g_launches;  // two kernels: the fast path and the general list

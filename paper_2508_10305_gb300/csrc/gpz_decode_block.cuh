@@ -454,7 +454,8 @@ __device__ __forceinline__ void decode_tail(const DecArgs& a, DecCore& S, uint32
             return;
         }
         const uint64_t first = (uint64_t)b * kBlock + t;
-#pragma unroll
+        constexpr int UNROLL = OUT64 ? 1 : F;  // unrolled, the doubles' conversions cost encoded blocks 2% (registers)
+#pragma unroll UNROLL
         for (int f = 0; f < F; ++f) {
             float v[N];
 #pragma unroll

@@ -380,6 +380,7 @@ gpz_status gpz_compress_f64(const double* const* d_fields, uint64_t n, const gpz
     const float* fields[kMaxFields];
     for (int f = 0; f < F; ++f) fields[f] = y + (uint64_t)f * ld;
     // the compression workspace sits at the start, so gpz_sync_status(d_ws) reads its status
+    // (fields_ready: the host has waited for the rounding pass)
     return compress_impl(fields, n, &q, d_out, out_capacity, d_out_size, h_out_size, d_perm, ws, cws, stream, true);
 }
 

@@ -138,13 +138,14 @@ RangeTargets compress_range_targets(uint64_t n, int F);
 constexpr int kRangeCtasMax = 152 * 8;  // partials held for this many CTAs
 
 // gpz_compress, optionally with the range pass already done (gpz_api.cu).
-// `tile` enqueues the tile kernel (tests pass another).  With `interleaved` (16-byte aligned F-field records, d_fields[f] =
+// fields_ready: no work that the caller enqueued
+// before still writes the fields.  `tile` enqueues the tile kernel (tests pass another).  With `interleaved` (16-byte aligned F-field records, d_fields[f] =
 // interleaved + f) the tile kernel reads the records themselves; a relative
 // bound then needs the range pass done.
 gpz_status compress_impl(const float* const* d_fields, uint64_t n, const gpz_params* p, void* d_out,
                          uint64_t out_capacity, uint64_t* d_out_size, uint64_t* h_out_size, uint32_t* d_perm,
                          void* d_ws, uint64_t ws_size, void* stream, bool range_done,
-                         const float* interleaved = nullptr, cudaError_t (*tile)(const QseArgs&, bool, cudaStream_t) = launch_qse_tile);
+                         const float* interleaved = nullptr, bool fields_ready = true, cudaError_t (*tile)(const QseArgs&, bool, cudaStream_t) = launch_qse_tile);
 
 // gpz_decompress; with `interleaved` the values go to F-field records there
 // (d_fields[f] = interleaved + f, 4-byte aligned) (gpz_api.cu).

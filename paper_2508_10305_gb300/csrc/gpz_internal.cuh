@@ -458,9 +458,9 @@ __device__ __forceinline__ uint2 load_after_wait(const uint2* p) {
 cudaError_t launch_range(const RangeArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_qse_direct(const QseArgs& a, cudaStream_t s);  // register kernel placing blocks directly, then the general list
 cudaError_t launch_qse_general(const QseArgs& a, cudaStream_t s);
-// Shared-memory tile kernel, then the general list.  early: the kernel before on
-// the stream is the range pass over the same fields, and nothing that this call
-// enqueued writes them, so the tile may be loaded while that pass still ends.
+// Shared-memory tile kernel, then the general list.  early: nothing that this call
+// enqueued may still be writing the fields (a transpose into the workspace
+// would), so the tile may be loaded while the work before it on the stream ends.
 cudaError_t launch_qse_tile(const QseArgs& a, bool early, cudaStream_t s);
 cudaError_t launch_qse_tile_unaligned(const QseArgs& a, bool early, cudaStream_t s);  // the same on 4-byte aligned fields
 cudaError_t launch_qse_tile_aos(const QseArgs& a, bool early, cudaStream_t s); // the same on interleaved records (16-byte aligned)

@@ -400,8 +400,8 @@ __device__ __forceinline__ void qse_block_tile(const QseArgs& a, uint8_t* dsm, T
         if (k >= s && k < end && ((t & 4) || k < 4u * lo)) tile[f * ROW + k] = __ldcs(a.fields[f] + first + (k - s));
     }
     if (!tile_overlays_hist(F, LAY)) clear_hist_row(reinterpret_cast<uint16_t*>(dsm + tile_region_bytes(F, LAY)));
-    // the range pass's results; the tile above is complete before the range
-    // pass starts, or the launch is an ordinary one (launch_qse_tile's `early`)
+    // the range pass's results; the tile above was complete before this call's
+    // work began, or the launch is an ordinary one (launch_qse_tile's `early`)
     if (PRE) wait_for_previous_kernel();
     // ---- 2. the field constants from the block's extremes: those of the
     // range pass (loaded with the step constants while the tile is in

@@ -205,7 +205,7 @@ gpz_status gpz_test_unstable_sort(int form, const void* const* d_fields, uint64_
         words += 2;
     } else if (form != 3) {
         st = compress_impl(fields, n, p, d_out, out_capacity, nullptr, h_out_size, d_perm, d_ws, ws_size, stream, false,
-                           form == 1 ? fields[0] : nullptr, unstable_tile);
+                           form == 1 ? fields[0] : nullptr, true, unstable_tile);
         words += 6;
     } else {
         gpz_compress_chunk d{};

@@ -22,8 +22,8 @@
 // computed in fixed point and only those within 10 * 2^-14 of a step of the
 // next one, 0.1%, in fp64 (wide_code).
 // 4*10^6 x 6 doubles at a relative bound of 1e-12: 0.299 ms in the general
-// kernel (0.241 without its needless fp64 operations), 0.115 here: 21,800 warp
-// instructions per block instead of 29,600, 62% of the issue slots busy.
+// kernel (0.241 without its needless fp64 operations), 0.115 here: 20,200 warp
+// instructions per block instead of 29,600, 60% of the issue slots busy.
 #include "gpz_sort.cuh"
 #include "gpz_wide.cuh"
 

@@ -29,24 +29,41 @@
 
 namespace gpz {
 
+// Where the arguments lie is a matter of measurement: read from the parameter
+// bank for aligned fields and doubles (2^26 x 6: 0.319 -> 0.314 ms, 2^23 x 6
+// doubles 0.084 -> 0.079), from a copy for fields of any alignment, whose stores index
+// the field pointers more often (3*10^7 x 3: 0.128 from the bank, 0.113 from a copy).
 template <int F, int OUT>
-__global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_decompress_kernel(DecArgs a) {
+__global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_decompress_kernel(const __grid_constant__ DecArgs a) {
     __shared__ DecShared<F> S;
     decode_block<F, OUT, false>(a, S, DecGridBlock{});
+}
+template <int F>
+__global__ void __launch_bounds__(kDecThreads, dec_ctas(F)) gpz_decompress_any_kernel(DecArgs a) {
+    __shared__ DecShared<F> S;
+    decode_block<F, kOutAny, false>(a, S, DecGridBlock{});
+}
+
+template <int F, int OUT>
+void launch_decompress_f(const DecArgs& a, cudaStream_t s) {
+    if constexpr (OUT == kOutAny)
+        gpz_decompress_any_kernel<F><<<a.nblocks, kDecThreads, 0, s>>>(a);
+    else
+        gpz_decompress_kernel<F, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a);
 }
 
 template <int OUT>
 cudaError_t launch_decompress_out(const DecArgs& a, cudaStream_t s) {
     if (a.nblocks == 0) return cudaSuccess;
     switch (a.F) {
-        case 1: gpz_decompress_kernel<1, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 2: gpz_decompress_kernel<2, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 3: gpz_decompress_kernel<3, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 4: gpz_decompress_kernel<4, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 5: gpz_decompress_kernel<5, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 6: gpz_decompress_kernel<6, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 7: gpz_decompress_kernel<7, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
-        case 8: gpz_decompress_kernel<8, OUT><<<a.nblocks, kDecThreads, 0, s>>>(a); break;
+        case 1: launch_decompress_f<1, OUT>(a, s); break;
+        case 2: launch_decompress_f<2, OUT>(a, s); break;
+        case 3: launch_decompress_f<3, OUT>(a, s); break;
+        case 4: launch_decompress_f<4, OUT>(a, s); break;
+        case 5: launch_decompress_f<5, OUT>(a, s); break;
+        case 6: launch_decompress_f<6, OUT>(a, s); break;
+        case 7: launch_decompress_f<7, OUT>(a, s); break;
+        case 8: launch_decompress_f<8, OUT>(a, s); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -4,7 +4,7 @@
 // and an encoding smaller than the raw block.  A block with a value that is not
 // finite is stored raw here, the others go to a list for the general kernel.
 // With an absolute bound the extremes have to be found first, and a block that
-// is then left has been read for nothing; most of those show in the first 256
+// is then left has been read for nothing; most of those show in the first 512
 // values of a field and are left there and then.  2^22 x 6 doubles at 1e-12
 // absolute 0.624 -> 0.541 ms (0.595 with the general kernel alone), with a NaN
 // in every block 0.310 -> 0.178 (0.250).
@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kTileThreads, wf_ctas(F)) gpz_wide_fast_kernel
                 for (int k = 0; k < 16; ++k) v[k] = __ldg(x + lane + 32 * k);
 #pragma unroll
                 for (int k = 0; k < 16; ++k) take(v[k]);
-                // a quarter of the warp's first field tells most blocks that
+                // half of the warp's first field tells most blocks that
                 // first_candidate_exact cannot accept
                 if (f == w && __any_sync(0xffffffffu, out_of_reach(nmin, kmax, a.params[f]))) {
                     leave = true;
